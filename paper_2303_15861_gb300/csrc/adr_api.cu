@@ -142,6 +142,14 @@ struct adr_ctx {
     unsigned* d_slots = nullptr;           // max-abs slots of the arrays a step produces
     int* d_err = nullptr;                  // device error word (bounded waits)
 
+    // FP64 on the tensor cores (contract_f64.cu): cut factors with their row parameters, phi tables
+    bool f64_grid = false;                 // the grid is one the kernel is the faster on
+    bool f64tc = false;                    // ... and every factor is within its range
+    adr::F64Tiles t64[3];
+    uint8_t* d_img64[kFactorKinds][3] = {{nullptr}};
+    int2* d_rows64[kFactorKinds][3] = {{nullptr}};
+    double* d_phi64[3] = {nullptr, nullptr, nullptr};   // phi_k(tau (l1 + l2 + l3)) at the nodes, k = 0, 1, 2
+
     // batched 2-D instances (p.batch > 0)
     std::unique_ptr<adr_batch_state> bs;
 
@@ -236,6 +244,28 @@ cudaError_t upload_tc(adr_ctx* c, int kind, int m, const std::vector<double>& M)
     if (e == cudaSuccess) e = cudaMemcpy(c->d_img2[kind][m], f2.img.data(), f2.img.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(c->d_fsc2[kind][m], f2.fscale.data(), f2.fscale.size() * sizeof(float), cudaMemcpyHostToDevice);
+    return e;
+}
+
+const void* dense_factor(const adr_ctx* c, int kind, int m);
+
+// Cut the uploaded factor of a kind for the FP64 tensor-core contraction. Factors outside its range
+// (an entry that is not finite or at least 2^400) take the context back to the FMA kernel.
+cudaError_t upload_f64(adr_ctx* c, int kind, int m, const std::vector<double>& M) {
+    if (!c->f64_grid || !c->f64tc) return cudaSuccess;
+    for (double v : M)
+        if (!(std::fabs(v) < std::ldexp(1.0, 400))) {
+            c->f64tc = false;
+            return cudaSuccess;
+        }
+    const adr::F64Tiles& t = c->t64[m];
+    cudaError_t e = cudaSuccess;
+    if (!c->d_img64[kind][m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_img64[kind][m]), adr::f64_image_bytes(t));
+    if (e == cudaSuccess && !c->d_rows64[kind][m])
+        e = cudaMalloc(reinterpret_cast<void**>(&c->d_rows64[kind][m]), size_t(t.nOut) * t.rows * sizeof(int2));
+    if (e == cudaSuccess)
+        e = adr::launch_f64_factor(static_cast<const double*>(dense_factor(c, kind, m)), c->n[m], t, c->d_img64[kind][m],
+                                   c->d_rows64[kind][m], nullptr);
     return e;
 }
 
@@ -341,6 +371,14 @@ enum FactorKind { FK_EXP_HALF = 0, FK_EXP_ONE = 1, FK_V = 2, FK_VINV = 3, FK_EXP
 static_assert(int(FK_EXP_HALF) == adr::BR_EXP_HALF && int(FK_EXP_ONE) == adr::BR_EXP_ONE && int(FK_V) == adr::BR_V &&
                   int(FK_VINV) == adr::BR_VINV,
               "factor kinds and batch roles share their numbering");
+
+// The dense factor of a kind along direction m (0-based).
+const void* dense_factor(const adr_ctx* c, int kind, int m) {
+    return kind >= kLevel0 ? c->d_El[kind - kLevel0][m]
+         : kind == FK_EXP_HALF ? c->d_E[0][m] : kind == FK_EXP_ONE ? c->d_E[1][m]
+         : kind == FK_EXP_ALPHA ? c->d_E[2][m]
+         : kind == FK_V ? c->d_V[m] : c->d_Vi[m];
+}
 
 bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
@@ -449,6 +487,40 @@ const unsigned* Sched::consume(const void* buf) {
     return sl;
 }
 
+// FP64 context on the tensor cores: one mu-mode pass (contract_f64.cu).
+void push_mode_f64(Sched& S, int mu, int kind, const double* x, double* y, int epi, const double* base, double alpha, int phik) {
+    const adr_ctx* c = S.c;
+    const adr::F64Tiles& t = c->t64[mu - 1];
+    adr::F64Args a;
+    a.X = x;
+    a.Y = y;
+    a.factor = static_cast<const double*>(dense_factor(c, kind, mu - 1));
+    a.fimg = c->d_img64[kind][mu - 1];
+    a.rows = c->d_rows64[kind][mu - 1];
+    a.n = c->n[mu - 1];
+    for (int nu = 1; nu < mu; ++nu) a.Q *= c->n[nu - 1];
+    a.npos = static_cast<long long>(c->N) / a.n;
+    a.nK = t.nK;
+    a.nOut = t.nOut;
+    a.ntiles = int(t.ntiles);
+    a.vec2 = a.n % 2 == 0 && aligned16(x);
+    a.epi = epi;
+    a.base = base;
+    a.alpha = alpha;
+    if (epi == adr::EPI_PHI) {
+        a.phi = c->d_phi64[phik];
+        a.phik = phik;
+        a.ctau = c->p.tau;
+        for (int m = 0; m < c->dim; ++m) a.lam[m] = c->d_lam[m];
+        a.n1 = c->n[0];
+        a.n2 = c->n[1];
+    }
+    a.err = c->d_err;
+    const bool mode1 = mu == 1;
+    const int cols = t.cols;
+    S.ops.push_back({[a, mode1, cols](cudaStream_t s) { return adr::launch_contract_f64(a, mode1, cols, s); }, OP_CONTRACT_TC});
+}
+
 // One mu-mode pass y = x x_mu M_kind with epilogue (epi, base, alpha, phik).
 template <typename T>
 void push_mode(Sched& S, int mu, int kind, const T* x, T* y, int epi = adr::EPI_STORE,
@@ -459,12 +531,14 @@ void push_mode(Sched& S, int mu, int kind, const T* x, T* y, int epi = adr::EPI_
         push_mode_batch<T>(S, mu, kind, x, y, epi, base, alpha, phik);
         return;
     }
+    if constexpr (sizeof(T) == 8) {
+        if (c->f64tc) {
+            push_mode_f64(S, mu, kind, x, y, epi, base, alpha, phik);
+            return;
+        }
+    }
     if (!c->tc) {
-        const void* M = kind >= kLevel0 ? c->d_El[kind - kLevel0][mu - 1]
-                      : kind == FK_EXP_HALF ? c->d_E[0][mu - 1] : kind == FK_EXP_ONE ? c->d_E[1][mu - 1]
-                      : kind == FK_EXP_ALPHA ? c->d_E[2][mu - 1]
-                      : kind == FK_V ? c->d_V[mu - 1] : c->d_Vi[mu - 1];
-        auto a = mode_args<T>(c, mu, static_cast<const T*>(M), x, y);
+        auto a = mode_args<T>(c, mu, static_cast<const T*>(dense_factor(c, kind, mu - 1)), x, y);
         a.epi = epi; a.base = base; a.alpha = alpha; a.phik = phik; a.ctau = c->p.tau;
         for (int m = 0; m < 3; ++m) a.lam[m] = (m < c->dim) ? c->d_lam[m] : nullptr;
         S.ops.push_back({[a](cudaStream_t s) { return adr::launch_contract(a, s); }, OP_CONTRACT_SIMT});
@@ -1685,6 +1759,7 @@ adr_status setup_doubling(adr_ctx* c) {
         for (int i = 0; i < sh && e == cudaSuccess; ++i) {
             e = upload(c, &c->d_El[i][m], (*levels)[size_t(i)]);
             if (e == cudaSuccess && c->tc) e = upload_tc(c, kLevel0 + i, m, (*levels)[size_t(i)]);
+            if (e == cudaSuccess) e = upload_f64(c, kLevel0 + i, m, (*levels)[size_t(i)]);
         }
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "upload doubling factors");
@@ -1793,6 +1868,18 @@ adr_status create_periodic(const adr_params* p, void* cuda_stream, adr_ctx** out
 
 }  // namespace
 
+namespace {
+// Whether an FP64 grid runs its contractions on the tensor cores: from about 4 million FMAs for the
+// longest direction's pass. Lawson2a, us per step on the FMA pipes / tensor cores: 128^2 (2.1 M) 99 / 95,
+// 40 x 36 x 33 (1.9 M) 114 / 147, 48^3 (5.3 M) 141 / 149, 200 x 150 (6 M) 147 / 110, 60^3 (13 M) 266 / 160,
+// 500 x 400 (100 M) 1162 / 230.
+bool use_f64_tc(const adr_ctx* c) {
+    int longest = 0;
+    for (int m = 0; m < c->dim; ++m) longest = std::max(longest, c->n[m]);
+    return longest <= adr::kF64MaxN && double(c->N) * longest >= 4e6;
+}
+}  // namespace
+
 // ===================================================================== C ABI
 extern "C" {
 
@@ -1840,7 +1927,13 @@ adr_status adr_create(const adr_params* p, void* cuda_stream, adr_ctx** out) {
     {
         cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&c->d_err), sizeof(int));
         if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, sizeof(int));
-        if (e == cudaSuccess && c->tc) e = cudaMalloc(reinterpret_cast<void**>(&c->d_slots), kSlots * sizeof(unsigned));
+        if (c->fp64 && use_f64_tc(c.get())) {
+            c->f64_grid = true;
+            for (int m = 0; m < c->dim; ++m)
+                c->t64[m] = adr::f64_tiles(c->n[m], static_cast<long long>(N) / c->n[m], m == 0);
+        }
+        if (e == cudaSuccess && c->tc)
+            e = cudaMalloc(reinterpret_cast<void**>(&c->d_slots), kSlots * sizeof(unsigned));
         if (e != cudaSuccess) {
             adr_destroy(c.release());
             return fail(nullptr, ADR_ERR_ALLOC, std::string("context: ") + cudaGetErrorString(e));
@@ -1900,6 +1993,7 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
     cudaError_t e = upload(c, &c->d_a, amb);
     if (e != cudaSuccess) return cuda_fail(c, e, "upload a");
 
+    c->f64tc = c->f64_grid;
     c->eig_real = true;
     struct CachedE { int n; double beta, c; std::vector<double> E; };
     std::vector<CachedE> cache;
@@ -1925,6 +2019,7 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
                 E = &cache.back().E;
             }
             e = upload(c, &c->d_E[ci][m], *E);
+            if (e == cudaSuccess) e = upload_f64(c, ci == 2 ? FK_EXP_ALPHA : ci, m, *E);
             if (e != cudaSuccess) return cuda_fail(c, e, "upload E");
             if (c->tc) {
                 e = upload_tc(c, ci == 2 ? FK_EXP_ALPHA : ci, m, *E);
@@ -1939,6 +2034,8 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
         if (e == cudaSuccess) e = upload(c, &c->d_Vi[m], eg.Vinv);
         if (e == cudaSuccess && !c->d_lam[m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_lam[m]), c->n[m] * sizeof(double));
         if (e == cudaSuccess) e = cudaMemcpy(c->d_lam[m], eg.lam.data(), c->n[m] * sizeof(double), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = upload_f64(c, FK_V, m, eg.V);
+        if (e == cudaSuccess) e = upload_f64(c, FK_VINV, m, eg.Vinv);
         if (e == cudaSuccess && c->tc) e = upload_tc(c, FK_V, m, eg.V);
         if (e == cudaSuccess && c->tc) e = upload_tc(c, FK_VINV, m, eg.Vinv);
         if (e == cudaSuccess && c->tc) {
@@ -1970,7 +2067,19 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
             c->phi_route = ADR_PHI_DOUBLING;
         } else {
             c->phi_route = ADR_PHI_EIGEN;
+            // the phi factors at the nodes: evaluated in the contraction's epilogue they would take
+            // longer than the contraction
+            for (int k = 1; k <= 2 && c->f64tc; ++k) {
+                if (!c->d_phi64[k]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_phi64[k]), c->N * sizeof(double));
+                if (e == cudaSuccess)
+                    e = adr::launch_f64_phi(c->d_phi64[k], k, c->p.tau, c->d_lam, c->n[0], c->n[1], c->N, nullptr);
+                if (e != cudaSuccess) return cuda_fail(c, e, "phi tables");
+            }
         }
+    }
+    if (c->f64tc) {                        // the kernels above ran on the legacy stream
+        e = cudaStreamSynchronize(nullptr);
+        if (e != cudaSuccess) return cuda_fail(c, e, "cut factors");
     }
     c->coeffs_set = true;
     return ADR_OK;
@@ -2356,6 +2465,9 @@ void adr_destroy(adr_ctx* c) {
     for (auto& row : c->d_fsc) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
     for (auto& row : c->d_img2) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
     for (auto& row : c->d_fsc2) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
+    for (auto& row : c->d_img64) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
+    for (auto& row : c->d_rows64) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
+    for (auto& p : c->d_phi64) { void* q = p; free_dev(q); p = nullptr; }
     for (auto& p : c->d_zt) { void* q = p; free_dev(q); p = nullptr; }
     { void* q = c->d_slots; free_dev(q); c->d_slots = nullptr; }
     { void* q = c->d_err; free_dev(q); c->d_err = nullptr; }

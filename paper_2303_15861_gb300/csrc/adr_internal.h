@@ -176,6 +176,45 @@ struct TmaArgs : TcArgs {
 bool tma_supported(int n, long long Q, const void* x, const void* xlo);
 cudaError_t launch_contract_tma(TmaArgs a, long long P, cudaStream_t s);
 
+// K2 in FP64 on the tensor cores (contract_f64.cu): the state seen as [P][n][Q] (mode 1: Q = 1),
+// contracted along n with a factor cut into seven slices.
+constexpr int kF64Slices = 7;
+constexpr int kF64Chunk = 32;        // K per factor tile
+constexpr int kF64MaxN = 1024;       // longest line (the cut factor takes 14 n^2 bytes)
+
+struct F64Tiles {
+    int cols = 64;                   // tile columns: outputs (modes >= 2) or fibres (mode 1)
+    int rows = 64;                   // factor rows per tile
+    int nOut = 0, nK = 0;            // factor tiles, K chunks
+    long long ntiles = 0;
+};
+F64Tiles f64_tiles(int n, long long npos, bool mode1);
+size_t f64_image_bytes(const F64Tiles& t);
+
+struct F64Args {
+    const double* X = nullptr;
+    double* Y = nullptr;
+    const double* factor = nullptr;  // dense, row-major (for lines contracted with plain FMAs)
+    const uint8_t* fimg = nullptr;   // its slices
+    const int2* rows = nullptr;      // per factor row: exponent of the result's unit less that of the state, shift
+    int n = 0;
+    long long Q = 1, npos = 0;       // npos: positions P Q (modes >= 2) or fibres P (mode 1)
+    int nK = 0, nOut = 0, ntiles = 0;
+    bool vec2 = false;               // mode 1: rows of X 16-byte aligned
+    int epi = EPI_STORE;
+    const double* base = nullptr;    // EPI_AXPY (may be Y)
+    double alpha = 0;
+    const double* phi = nullptr;     // EPI_PHI: table over the nodes, or NULL with the fields below
+    int phik = 1;
+    double ctau = 0;
+    const double* lam[3] = {nullptr, nullptr, nullptr};
+    int n1 = 1, n2 = 1;
+    int* err = nullptr;
+};
+cudaError_t launch_contract_f64(const F64Args& a, bool mode1, int cols, cudaStream_t s);
+cudaError_t launch_f64_factor(const double* M, int n, const F64Tiles& t, uint8_t* img, int2* rows, cudaStream_t s);
+cudaError_t launch_f64_phi(double* tab, int k, double ctau, const double* const lam[3], int n1, int n2, size_t N, cudaStream_t s);
+
 // Host: slice an FP64 factor into the tensor-core image, with output tiles of `rows` rows
 // and K chunks of `chunk` (64: 128-byte swizzle, contract_tc.cu; 32: 64-byte swizzle,
 // contract_tma.cu); slices F0, F1, 2^-8 F1, 2^-8 F2 (chunk 64, standard) or F0..F3 (chunk 32,
