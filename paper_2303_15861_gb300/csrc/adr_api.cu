@@ -145,9 +145,8 @@ struct adr_ctx {
     // FP64 on the tensor cores (contract_f64.cu): cut factors with their row parameters, phi tables
     bool f64_grid = false;                 // the grid is one the kernel is the faster on
     bool f64tc = false;                    // ... and every factor is within its range
-    adr::F64Tiles t64[3];
     uint8_t* d_img64[kFactorKinds][3] = {{nullptr}};
-    int2* d_rows64[kFactorKinds][3] = {{nullptr}};
+    int* d_rows64[kFactorKinds][3] = {{nullptr}};
     double* d_phi64[3] = {nullptr, nullptr, nullptr};   // phi_k(tau (l1 + l2 + l3)) at the nodes, k = 0, 1, 2
 
     // batched 2-D instances (p.batch > 0)
@@ -258,13 +257,13 @@ cudaError_t upload_f64(adr_ctx* c, int kind, int m, const std::vector<double>& M
             c->f64tc = false;
             return cudaSuccess;
         }
-    const adr::F64Tiles& t = c->t64[m];
+    const int n = c->n[m];
     cudaError_t e = cudaSuccess;
-    if (!c->d_img64[kind][m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_img64[kind][m]), adr::f64_image_bytes(t));
+    if (!c->d_img64[kind][m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_img64[kind][m]), adr::f64_image_bytes(n));
     if (e == cudaSuccess && !c->d_rows64[kind][m])
-        e = cudaMalloc(reinterpret_cast<void**>(&c->d_rows64[kind][m]), size_t(t.nOut) * t.rows * sizeof(int2));
+        e = cudaMalloc(reinterpret_cast<void**>(&c->d_rows64[kind][m]), adr::f64_rows(n) * sizeof(int));
     if (e == cudaSuccess)
-        e = adr::launch_f64_factor(static_cast<const double*>(dense_factor(c, kind, m)), c->n[m], t, c->d_img64[kind][m],
+        e = adr::launch_f64_factor(static_cast<const double*>(dense_factor(c, kind, m)), n, c->d_img64[kind][m],
                                    c->d_rows64[kind][m], nullptr);
     return e;
 }
@@ -490,7 +489,6 @@ const unsigned* Sched::consume(const void* buf) {
 // FP64 context on the tensor cores: one mu-mode pass (contract_f64.cu).
 void push_mode_f64(Sched& S, int mu, int kind, const double* x, double* y, int epi, const double* base, double alpha, int phik) {
     const adr_ctx* c = S.c;
-    const adr::F64Tiles& t = c->t64[mu - 1];
     adr::F64Args a;
     a.X = x;
     a.Y = y;
@@ -500,10 +498,6 @@ void push_mode_f64(Sched& S, int mu, int kind, const double* x, double* y, int e
     a.n = c->n[mu - 1];
     for (int nu = 1; nu < mu; ++nu) a.Q *= c->n[nu - 1];
     a.npos = static_cast<long long>(c->N) / a.n;
-    a.nK = t.nK;
-    a.nOut = t.nOut;
-    a.ntiles = int(t.ntiles);
-    a.vec2 = a.n % 2 == 0 && aligned16(x);
     a.epi = epi;
     a.base = base;
     a.alpha = alpha;
@@ -516,9 +510,7 @@ void push_mode_f64(Sched& S, int mu, int kind, const double* x, double* y, int e
         a.n2 = c->n[1];
     }
     a.err = c->d_err;
-    const bool mode1 = mu == 1;
-    const int cols = t.cols;
-    S.ops.push_back({[a, mode1, cols](cudaStream_t s) { return adr::launch_contract_f64(a, mode1, cols, s); }, OP_CONTRACT_TC});
+    S.ops.push_back({[a](cudaStream_t s) { return adr::launch_contract_f64(a, s); }, OP_CONTRACT_TC});
 }
 
 // One mu-mode pass y = x x_mu M_kind with epilogue (epi, base, alpha, phik).
@@ -1869,14 +1861,14 @@ adr_status create_periodic(const adr_params* p, void* cuda_stream, adr_ctx** out
 }  // namespace
 
 namespace {
-// Whether an FP64 grid runs its contractions on the tensor cores: from about 4 million FMAs for the
-// longest direction's pass. Lawson2a, us per step on the FMA pipes / tensor cores: 128^2 (2.1 M) 99 / 95,
-// 40 x 36 x 33 (1.9 M) 114 / 147, 48^3 (5.3 M) 141 / 149, 200 x 150 (6 M) 147 / 110, 60^3 (13 M) 266 / 160,
-// 500 x 400 (100 M) 1162 / 230.
+// Whether an FP64 grid runs its contractions on the tensor cores: from about 1.5 million FMAs for the
+// longest direction's pass. ETD2RK, us per step on the FMA pipes / tensor cores: 64^2 (0.3 M) 80 / 77, 32^3
+// (1.0 M) 116 / 129, 40 x 36 x 33 (1.9 M) 156 / 145, 128^2 (2.1 M) 133 / 97, 48^3 (5.3 M) 196 / 146,
+// 200 x 150 (6 M) 198 / 115, 500 x 400 (100 M) 1522 / 269.
 bool use_f64_tc(const adr_ctx* c) {
     int longest = 0;
     for (int m = 0; m < c->dim; ++m) longest = std::max(longest, c->n[m]);
-    return longest <= adr::kF64MaxN && double(c->N) * longest >= 4e6;
+    return longest <= adr::kF64MaxN && double(c->N) * longest >= 1.5e6;
 }
 }  // namespace
 
@@ -1927,13 +1919,8 @@ adr_status adr_create(const adr_params* p, void* cuda_stream, adr_ctx** out) {
     {
         cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&c->d_err), sizeof(int));
         if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, sizeof(int));
-        if (c->fp64 && use_f64_tc(c.get())) {
-            c->f64_grid = true;
-            for (int m = 0; m < c->dim; ++m)
-                c->t64[m] = adr::f64_tiles(c->n[m], static_cast<long long>(N) / c->n[m], m == 0);
-        }
-        if (e == cudaSuccess && c->tc)
-            e = cudaMalloc(reinterpret_cast<void**>(&c->d_slots), kSlots * sizeof(unsigned));
+        c->f64_grid = c->fp64 && use_f64_tc(c.get());
+        if (e == cudaSuccess && c->tc) e = cudaMalloc(reinterpret_cast<void**>(&c->d_slots), kSlots * sizeof(unsigned));
         if (e != cudaSuccess) {
             adr_destroy(c.release());
             return fail(nullptr, ADR_ERR_ALLOC, std::string("context: ") + cudaGetErrorString(e));

@@ -182,25 +182,14 @@ constexpr int kF64Slices = 7;
 constexpr int kF64Chunk = 32;        // K per factor tile
 constexpr int kF64MaxN = 1024;       // longest line (the cut factor takes 14 n^2 bytes)
 
-struct F64Tiles {
-    int cols = 64;                   // tile columns: outputs (modes >= 2) or fibres (mode 1)
-    int rows = 64;                   // factor rows per tile
-    int nOut = 0, nK = 0;            // factor tiles, K chunks
-    long long ntiles = 0;
-};
-F64Tiles f64_tiles(int n, long long npos, bool mode1);
-size_t f64_image_bytes(const F64Tiles& t);
-
 struct F64Args {
     const double* X = nullptr;
     double* Y = nullptr;
     const double* factor = nullptr;  // dense, row-major (for lines contracted with plain FMAs)
     const uint8_t* fimg = nullptr;   // its slices
-    const int2* rows = nullptr;      // per factor row: exponent of the result's unit less that of the state, shift
+    const int* rows = nullptr;       // per factor row: exponent of the result's unit less that of the line
     int n = 0;
-    long long Q = 1, npos = 0;       // npos: positions P Q (modes >= 2) or fibres P (mode 1)
-    int nK = 0, nOut = 0, ntiles = 0;
-    bool vec2 = false;               // mode 1: rows of X 16-byte aligned
+    long long Q = 1, npos = 0;       // npos: positions P Q (modes >= 2) or fibres P (mode 1, Q = 1)
     int epi = EPI_STORE;
     const double* base = nullptr;    // EPI_AXPY (may be Y)
     double alpha = 0;
@@ -210,9 +199,15 @@ struct F64Args {
     const double* lam[3] = {nullptr, nullptr, nullptr};
     int n1 = 1, n2 = 1;
     int* err = nullptr;
+    // set by the launcher
+    int nK = 0, nOut = 0, ntiles = 0;
+    bool vec2 = false;               // mode 1: rows of X 16-byte aligned
+    bool vec4 = false;               // modes >= 2: four columns are 32 aligned bytes
 };
-cudaError_t launch_contract_f64(const F64Args& a, bool mode1, int cols, cudaStream_t s);
-cudaError_t launch_f64_factor(const double* M, int n, const F64Tiles& t, uint8_t* img, int2* rows, cudaStream_t s);
+cudaError_t launch_contract_f64(F64Args a, cudaStream_t s);
+size_t f64_image_bytes(int n);
+int f64_rows(int n);                 // rows of the image (n rounded up to whole tiles)
+cudaError_t launch_f64_factor(const double* M, int n, uint8_t* img, int* rows, cudaStream_t s);
 cudaError_t launch_f64_phi(double* tab, int k, double ctau, const double* const lam[3], int n1, int n2, size_t N, cudaStream_t s);
 
 // Host: slice an FP64 factor into the tensor-core image, with output tiles of `rows` rows

@@ -18,8 +18,9 @@
 // the slice products left out (i + j > 6), and one rounding of the result to FP64. A chain of K FMAs rounds
 // K times. Against exact sums, e^{c tau A}, V and V^-1 for n = 24..300, b = 1..50, smooth and random
 // states: relative l2 4e-17 to 1.6e-16, where the FMA kernel has 9e-17 to 6.3e-16, and the smaller of the two in every case.
-// Time of a pass, FMA kernel -> this one: 256^3 6.9 ms -> 0.33 (mode 1) and 0.47 ms, 128^3 526 -> 42 to 62 us,
-// 60^3 33 -> 15 to 18 us.
+// Time of a pass, FMA kernel -> this one: 256^3 6.9 ms -> 0.24 ms, 128^3 526 -> 31 us (39 with the phi table), 60^3
+// 33 -> 12 us. At the BF16 rate the products of a 256^3 pass take 0.13 ms; the rest is the assembly of a tile,
+// which cannot overlap its MMAs (the accumulators fill TMEM), and the producers just behind them.
 //
 // es belongs to one line (the n values that are contracted together): the producers read a tile's lines
 // once for their largest exponents and a second time, from L2, to cut them. One es for the whole array would
@@ -29,14 +30,17 @@
 // 2^-500..2^500, are contracted with plain FMAs by the epilogue, so that such values propagate as
 // in any FP64 sum.
 //
-// Work split. 128 rows (TMEM lanes) lie along the contiguous direction: for modes >= 2 they are 128
-// positions (q fastest, p and q flattened, so a short q leaves no empty rows) and the columns are outputs; for mode 1
-// they are outputs and the columns are fibres. N = 64 columns (448 of the 512 TMEM columns), or 32 where 64 would leave
-// SMs without a tile. Per CTA and SM: 8 producer warps load FP64 from global memory (the next chunk in
+// Work split. The factor is the A operand, 128 outputs (TMEM lanes) a tile; the lines are the B operand,
+// N = 64 of them (448 of the 512 TMEM columns), or 32 where 64 would leave SMs without a tile. For modes >= 2
+// the lines of a tile are consecutive positions, p and q flattened, so a short q leaves no empty
+// columns. Per CTA and SM: 8 producer warps load FP64 from global memory (the next chunk in
 // registers while this one is cut, no alignment rules, so every shape takes this kernel) and
 // store the slices; one thread issues the MMAs; one copies the pre-cut factor; 8 warps put the results together.
-// Cutting and assembling use integer instructions throughout (about 40 each): one FP64 instruction
-// occupies its pipe as long as 64 of the others.
+// With the lines as the A operand, 128 a tile, and 64 outputs, each line of a 256^3 grid is cut four
+// times instead of twice, which took 460 us a pass.
+// Cutting and assembling use integer instructions, one FP64-pipe instruction per result: one of
+// those occupies its pipe as long as 64 of the others. Tried, us a pass at 128^3 / 256^3 (29 / 241 as it is): the conversion
+// in integers too 33 / 265; the line maxima of the next tile read while a tile is cut 31 / 243 (mode 1) and 268.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -59,17 +63,18 @@ constexpr int kMmaWarp = kProducerWarps + kEpiWarps;
 constexpr int kLoadWarp = kMmaWarp + 1;
 constexpr int kThreads = (kLoadWarp + 1) * 32;
 
-template <bool SA, int N>
+template <int N>
 struct Cfg {
-    static constexpr int ATILE = kM * kKc * 2, BTILE = N * kKc * 2;   // one slice tile of either operand
-    static constexpr int STILE = SA ? ATILE : BTILE, FTILE = SA ? BTILE : ATILE;
+    static constexpr int FTILE = kM * kKc * 2, STILE = N * kKc * 2;   // one slice tile of either operand
     static constexpr int SBYTES = kSl * STILE, FBYTES = kSl * FTILE;  // one stage
-    static constexpr int NS = SA ? 2 : 3, NF = SA ? 3 : 2;            // ring depths: 196 KB at N = 64
+    static constexpr int NS = 3, NF = 2;                              // ring depths: 196 KB at N = 64
     static constexpr int SMEM = NS * SBYTES + NF * FBYTES + 1024;
     static constexpr uint32_t TMEM = N == 64 ? 512 : 256;             // 7 N columns, a power of two
     static constexpr int COLS = N / (kEpiWarps / 4);                  // columns per epilogue warp
     static constexpr int WIDE = 256 / N;                              // slices per MMA (N <= 256)
-    static_assert(SMEM <= 227 * 1024, "shared memory budget");
+    static constexpr int KV = N * kKc / (kProducerWarps * 32);        // K values a producer thread cuts per chunk
+    static constexpr int KG = kKc / KV;                               // threads per line
+    static_assert(SMEM <= 222 * 1024, "shared memory budget");
 };
 
 __device__ __forceinline__ uint32_t idesc_of(int ncols) {   // FP32 accumulator, BF16 operands, M = 128
@@ -96,22 +101,34 @@ __device__ __forceinline__ void cut(double x, int etop, float (&s)[kSl]) {
     s[6] = __uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7440)) - 8388736.f;
 }
 
-// Cut 8 values along K and store them as 16-byte chunk j of row r of the seven slice tiles.
-template <int TILE>
-__device__ __forceinline__ void cut_store8(const double (&v)[8], int etop, uint32_t tile0, int r, int j) {
-    uint32_t w[kSl][4];
+// Cut KV (4 or 8) values along K and store them at K position k of row r of the seven slice tiles.
+template <int TILE, int KV>
+__device__ __forceinline__ void cut_store(const double (&v)[KV], int etop, uint32_t tile0, int r, int k) {
+    uint32_t w[kSl][KV / 2];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
+    for (int e = 0; e < KV / 2; ++e) {
         float a[kSl], b[kSl];
         cut(v[2 * e], etop, a);
         cut(v[2 * e + 1], etop, b);
 #pragma unroll
         for (int q = 0; q < kSl; ++q) w[q][e] = __byte_perm(__float_as_uint(a[q]), __float_as_uint(b[q]), 0x7632);
     }
-    const uint32_t off = swz64(r, j);
+    const uint32_t dst = tile0 + swz64(r, k >> 3) + (k & 7) * 2;
 #pragma unroll
-    for (int q = 0; q < kSl; ++q)
-        st_shared_v4(tile0 + q * TILE + off, make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]));
+    for (int q = 0; q < kSl; ++q) {
+        if constexpr (KV == 8)
+            st_shared_v4(dst + q * TILE, make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]));
+        else
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dst + q * TILE), "r"(w[q][0]), "r"(w[q][1]) : "memory");
+    }
+}
+
+// 32-byte (256-bit) accesses: four consecutive doubles.
+__device__ __forceinline__ void ld4(const double* p, double (&v)[4]) {
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void st4(double* p, const double (&v)[4]) {
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]) : "memory");
 }
 
 // Four columns of the seven accumulators, `stride` TMEM columns apart.
@@ -139,21 +156,21 @@ __device__ __forceinline__ void tmem_ld4x7(uint32_t t0, uint32_t stride, float (
         for (int j = 0; j < 4; ++j) d[k][j] = __uint_as_float(r[4 * k + j]);
 }
 
-// The result from its seven sums: T = t 2^sh + r with |t| < 2^51 and 0 <= r < 2^sh, in units of 2^e.
-// t goes into the mantissa of 1.5 2^52 2^(e + sh) and r into that of 2^52 2^e; the difference of
-// the first to 1.5 2^52 2^(e + sh) + 2^52 2^e is exact, adding the second rounds once: two FP64
-// instructions.
-__device__ __forceinline__ double assemble(const float (&d)[kSl][4], int c, int sh, int e) {
+// The result from its seven sums, in units of 2^e: T = 2^24 h + l, shifted right (rounding) by the ex >= 0 places that
+// leave it 62 bits; the conversion to FP64 rounds to nearest, and the unit goes into the exponent.
+__device__ __forceinline__ double assemble(const float (&d)[kSl][4], int c, int e) {
     int v[kSl];
 #pragma unroll
     for (int k = 0; k < kSl; ++k) v[k] = __float2int_rn(d[k][c]);
     const long long h = static_cast<long long>(v[0]) * (1 << 24) + static_cast<long long>(v[1]) * (1 << 16) +
                         static_cast<long long>(v[2]) * (1 << 8) + v[3];
     const long long l = static_cast<long long>(v[4]) * (1 << 16) + static_cast<long long>(v[5]) * (1 << 8) + v[6];
-    const long long t = (h << (24 - sh)) + (l >> sh);
-    const long long top = static_cast<long long>(((1075 + e + sh) << 20) | 0x80000) << 32;
-    const double hi = __longlong_as_double(top + t) - __longlong_as_double(top + (1LL << (52 - sh)));
-    return hi + __hiloint2double((1075 + e) << 20, int(l) & ((1 << sh) - 1));
+    const int top = int(h >> 32);                            // |T| < 2^(88 - clz)
+    const int ex = max(26 - __clz(top ^ (top >> 31)), 0);
+    const long long t = (h << (24 - ex)) + ((l + ((1 << ex) >> 1)) >> ex);
+    const double r = static_cast<double>(t);
+    const int up = t ? (e + ex) << 20 : 0;
+    return __hiloint2double(__double2hiint(r) + up, __double2loint(r));
 }
 
 // One output by plain FMAs, k ascending (lines whose values do not fit the slices).
@@ -169,9 +186,8 @@ __device__ __forceinline__ unsigned f64_amax_bits(double v) {
     return (unsigned(__double2hiint(v)) & 0x7FFFFFFFu) | (__double2loint(v) != 0 ? 1u : 0u);
 }
 
-// The phi factor of node o: from the table, or evaluated where the context keeps none.
-__device__ __forceinline__ double f64_phi(const F64Args& p, long long o) {
-    if (p.phi) return __ldg(p.phi + o);
+// The phi factor of node o, where the context keeps no table.
+__device__ __noinline__ double f64_phi_eval(const F64Args& p, long long o) {
     double ls = p.lam[0][o % p.n1] + p.lam[1][(o / p.n1) % p.n2];
     if (p.lam[2]) ls += p.lam[2][o / p.n1 / p.n2];
     return phi_eval(p.phik, p.ctau * ls);
@@ -179,17 +195,19 @@ __device__ __forceinline__ double f64_phi(const F64Args& p, long long o) {
 
 constexpr int kNoCut = 1 << 20;          // es of a line that fma_dot contracts
 
-template <bool SA, int N, int EPI>
+template <bool MODE1, int N, int EPI>
 __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_constant__ F64Args p) {
-    using C = Cfg<SA, N>;
+    using C = Cfg<N>;
     extern __shared__ uint8_t smem_raw[];
     constexpr uint32_t kSF = 0, kSE = kSF + 8 * C::NS, kFF = kSE + 8 * C::NS, kFE = kFF + 8 * C::NF, kAF = kFE + 8 * C::NF,
                        kAE = kAF + 8, kDR = kAE + 8;
     __shared__ __align__(8) uint64_t bars[kDR / 8 + 1];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
-    __shared__ int es_s[4][kM];                              // per line of the last four tiles
-    __shared__ unsigned half_s[2][2][kM];                    // SA: the two halves of a line's max|x|
+    // per line of the last four tiles: its exponent es, and its offset in the state (k = 0)
+    __shared__ int es_s[4][N];
+    __shared__ long long off_s[4][N];
+    __shared__ unsigned part_s[2][C::KG][N];                 // modes >= 2: the parts of a line's max|x|
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;     // state-slice ring
@@ -228,112 +246,119 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
     const uint32_t tmem = tmem_base_s;
 
     const int n = p.n;
-    const long long Q = p.Q;
+    const long long Q = MODE1 ? 1 : p.Q;
     const int items = (p.ntiles - int(blockIdx.x) + int(gridDim.x) - 1) / int(gridDim.x) * p.nK;   // (tile, K chunk) in order
 
     if (warp == kLoadWarp) {
         // ------------------------------------------------------------ factor loader (bulk copies)
         if (lane == 0) {
-            int s = 0;
+            int s = 0, issued = 0;
             uint32_t ph = 1;
             for (int tile = blockIdx.x; tile < p.ntiles && !abort_s; tile += gridDim.x) {
                 const uint8_t* src = p.fimg + size_t(tile % p.nOut) * p.nK * C::FBYTES;
-                for (int c = 0; c < p.nK; ++c, src += C::FBYTES) {
+                for (int c = 0; c < p.nK; ++c, src += C::FBYTES, ++issued) {
                     if (!mbar_wait(fempty(s), ph, p.err, 64, &abort_s, 32)) break;
                     mbar_arrive_expect_tx(ffull(s), C::FBYTES);
                     bulk_g2s(fbase + s * C::FBYTES, src, C::FBYTES, ffull(s));
                     if (++s == C::NF) { s = 0; ph ^= 1; }
                 }
             }
+            // no copy may land after the CTA has gone (they have, unless a wait gave up)
+            const long long t0 = clock64();
+            for (int k = max(issued - C::NF, 0); k < issued; ++k)
+                while (!mbar_try_wait(ffull(k % C::NF), uint32_t(k / C::NF) & 1u) && clock64() - t0 < kWaitCycles) {}
         }
     } else if (warp < kProducerWarps) {
         // ------------------------------------------------------------ producers (global -> slices)
-        // SA: a thread cuts 16 K values of one position (two chunks of 8); mode 1: 8 of one fibre
-        // (N = 32: the upper half of the warps has no rows).
-        constexpr int NV = SA ? 2 : 1;
+        // KG threads a line, each KV consecutive K values of a chunk: neighbouring lanes along K for mode 1,
+        // along the positions otherwise, so that a warp reads whole sectors.
+        constexpr int KV = C::KV, KG = C::KG;
         const int t = threadIdx.x;
-        const int row = SA ? (t & (kM - 1)) : (t >> 2);
-        const int kofs = SA ? 16 * (t >> 7) : 8 * (t & 3);
-        const bool busy = SA || row < N;
-        double v[NV][8];
-        // the (tile, chunk) whose values are being loaded, and this thread's row of that tile
-        int ltile = blockIdx.x, lc = 0;
+        const int row = MODE1 ? t / KG : t % N, kg = MODE1 ? t % KG : t / N;
+        const int kofs = KV * kg;
+        double v[KV];
+        // the (tile, chunk) whose values are being loaded, and this thread's line of that tile
+        int ltile = blockIdx.x, lc = 0, etop = 0;
         const double* xrow = nullptr;
         bool lrow = false, live = true;
+        long long xoff = 0;
         auto set_row = [&]() {
-            const unsigned pos = unsigned(ltile / p.nOut) * (SA ? kM : N) + row;
-            lrow = ltile < p.ntiles && busy && pos < unsigned(p.npos);
-            const unsigned q = SA ? pos % unsigned(Q) : 0u;
-            xrow = SA ? p.X + (long long)(pos / unsigned(Q)) * n * Q + q : p.X + (long long)pos * n;
+            const unsigned pos = unsigned(ltile / p.nOut) * N + row;
+            lrow = ltile < p.ntiles && pos < unsigned(p.npos);
+            xoff = MODE1 ? (long long)pos * n : (long long)(pos / unsigned(Q)) * n * Q + pos % unsigned(Q);
+            xrow = p.X + xoff + kofs * Q;
         };
-        auto load8 = [&](int h) {
-            const int k0 = lc * kKc + kofs + 8 * h;
-            const double* x = xrow + (SA ? (long long)k0 * Q : (long long)k0);
-            if (SA) {
+        auto load = [&](int k0, double (&w)[KV]) {           // K values k0 + kofs.. (0 past the line's end)
+            const double* x = xrow + k0 * Q;
+            if (MODE1 && p.vec2) {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) v[h][e] = (lrow && k0 + e < n) ? __ldg(x + e * Q) : 0.0;
-            } else if (p.vec2) {
-#pragma unroll
-                for (int e = 0; e < 8; e += 2) {
-                    const double2 w = (lrow && k0 + e < n) ? __ldg(reinterpret_cast<const double2*>(x + e)) : make_double2(0.0, 0.0);
-                    v[h][e] = w.x;
-                    v[h][e + 1] = w.y;
+                for (int e = 0; e < KV; e += 2) {
+                    const double2 u = (lrow && k0 + kofs + e < n) ? __ldg(reinterpret_cast<const double2*>(x + e)) : make_double2(0.0, 0.0);
+                    w[e] = u.x;
+                    w[e + 1] = u.y;
                 }
             } else {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) v[h][e] = (lrow && k0 + e < n) ? __ldg(x + e) : 0.0;
+                for (int e = 0; e < KV; ++e) w[e] = (lrow && k0 + kofs + e < n) ? __ldg(x + e * Q) : 0.0;
             }
         };
-        // es of this thread's line: the chunk in v and the line's other chunks
-        int etop = 0;
+        auto amax = [&](const double (&w)[KV], unsigned m) {
+#pragma unroll
+            for (int e = 0; e < KV; ++e) m = max(m, f64_amax_bits(w[e]));
+            return m;
+        };
+        // es of this thread's line, of which v holds the first chunk
         auto line_scale = [&](int tl) {
-            unsigned m = 0;
-#pragma unroll
-            for (int h = 0; h < NV; ++h)
-#pragma unroll
-                for (int e = 0; e < 8; ++e) m = max(m, f64_amax_bits(v[h][e]));
-            for (int k0 = kKc + kofs; k0 < n; k0 += kKc) {
-                const double* x = xrow + (SA ? (long long)k0 * Q : (long long)k0);
-#pragma unroll
-                for (int e = 0; e < 8 * NV; ++e)
-                    if (lrow && k0 + e < n) m = max(m, f64_amax_bits(__ldg(x + (SA ? e * Q : (long long)e))));
+            unsigned m = amax(v, 0u);
+            int c = 1;
+            for (; c + 1 < p.nK; c += 2) {                   // two chunks of loads in flight
+                double w[KV], u[KV];
+                load(c * kKc, w);
+                load((c + 1) * kKc, u);
+                m = amax(u, amax(w, m));
             }
-            if (SA) {                                        // two threads a line, in different warps
-                half_s[tl & 1][t >> 7][row] = m;
+            if (c < p.nK) {
+                double w[KV];
+                load(c * kKc, w);
+                m = amax(w, m);
+            }
+            if (MODE1) {
+#pragma unroll
+                for (int o = 1; o < KG; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+            } else {
+                part_s[tl & 1][kg][row] = m;
                 asm volatile("bar.sync 1, %0;" ::"n"(kProducerWarps * 32) : "memory");
-                m = max(m, half_s[tl & 1][1 - (t >> 7)][row]);
-            } else {                                         // four neighbouring lanes a line
-                m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
-                m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+#pragma unroll
+                for (int o = 0; o < KG; ++o) m = max(m, part_s[tl & 1][o][row]);
             }
             const int eb = int(m >> 20);
-            const bool cut_it = m == 0u || (eb >= 1023 - 500 && eb <= 1023 + 500);
+            live = m == 0u || (eb >= 1023 - 500 && eb <= 1023 + 500);
             etop = m ? eb : 1022;                            // es + 1022
-            if (busy && kofs == 0) es_s[tl & 3][row] = cut_it ? etop - 1022 : kNoCut;
-            live = cut_it;
+            if (kg == 0) {
+                es_s[tl & 3][row] = live ? etop - 1022 : kNoCut;
+                off_s[tl & 3][row] = xoff;
+            }
         };
         set_row();
-#pragma unroll
-        for (int h = 0; h < NV; ++h) load8(h);
+        load(0, v);
         line_scale(0);
         for (int it = 0, ss = 0, sph = 1, tl = 0; it < items; ++it) {
-            // waits decide warp-uniformly: the per-warp arrivals below need every lane
-            if (!__all_sync(0xffffffffu, mbar_wait(sempty(ss), sph, p.err, 1, &abort_s, 32))) break;
+            // after an abort the wait returns at once and the loop runs out, so that every producer warp
+            // still meets the others at line_scale's barrier
+            mbar_wait(sempty(ss), sph, p.err, 1, &abort_s, 32);
+            __syncwarp();
             const bool next_tile = ++lc == p.nK;
             if (next_tile) {
                 lc = 0;
                 ltile += gridDim.x;
                 set_row();
             }
+            if (!live) {
 #pragma unroll
-            for (int h = 0; h < NV; ++h) {
-                if (!live) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) v[h][e] = 0.0;
-                }
-                if (busy) cut_store8<C::STILE>(v[h], etop, sbase + ss * C::SBYTES, row, kofs / 8 + h);
-                load8(h);                                    // in flight until the next chunk is cut
+                for (int e = 0; e < KV; ++e) v[e] = 0.0;
             }
+            cut_store<C::STILE, KV>(v, etop, sbase + ss * C::SBYTES, row, kofs);
+            load(lc * kKc, v);                               // in flight until the next chunk is cut
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(sfull(ss));
@@ -344,65 +369,60 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
         // ------------------------------------------------------------ epilogue
         const int ew = (warp - kProducerWarps) & 3;          // TMEM lane quarter (warp % 4)
         const int part = (warp - kProducerWarps) >> 2;       // column part
-        const int row = ew * 32 + lane;
+        const int jlo = part * C::COLS, jhi = jlo + C::COLS;
         const uint32_t tbase = tmem + (uint32_t(ew * 32) << 16);
         uint32_t seg = 0;
         int tl = 0;
         bool ok = true;
         for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x, ++tl) {
             const int pt = tile / p.nOut, ot = tile % p.nOut;
-            bool rvalid;
-            long long off0, cstep;
-            int ncol, rsh = 16, rexp = 0;
-            const double* xline = nullptr;                   // SA: this position's line; mode 1: the first fibre's
-            if (SA) {
-                const unsigned pos = unsigned(pt) * kM + row;
-                rvalid = pos < unsigned(p.npos);
-                off0 = ((long long)(pos / unsigned(Q)) * n + (long long)ot * N) * Q + pos % unsigned(Q);
-                xline = p.X + (long long)(pos / unsigned(Q)) * n * Q + pos % unsigned(Q);
-                cstep = Q;
-                ncol = min(N, n - ot * N);
-            } else {
-                const int irow = ot * kM + row;
-                rvalid = irow < n;
-                const int2 rp = __ldg(p.rows + irow);        // padded to whole tiles
-                rsh = rp.y;
-                rexp = rp.x;
-                xline = p.X + (long long)pt * N * n;
-                off0 = (long long)pt * N * n + irow;
-                cstep = n;
-                ncol = min(N, int(p.npos) - pt * N);
-            }
+            const int irow = ot * kM + ew * 32 + lane;       // this lane's output
+            const bool rvalid = irow < n;
+            const bool warp_on = ot * kM + ew * 32 < n;
+            const int ncol = min(N, int(p.npos - (long long)pt * N));
+            const int rexp = __ldg(p.rows + irow);           // padded to whole tiles
+            const long long ioff = irow * Q;
+            const long long* off_t = off_s[tl & 3];
+            const int* es_t = es_s[tl & 3];
             for (int c0 = 0; c0 < p.nK; c0 += kSegChunks, ++seg) {
                 const bool first = c0 == 0;
-                const int jlo = part * C::COLS, jhi = jlo + C::COLS;
-                // the axpy's base, the phi table's values or the earlier segments' sum, one group ahead
-                double bcur[4], bnxt[4];
-                double ycur[4], ynxt[4];
-                auto load_side = [&](int j0, double (&b)[4], double (&y)[4]) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool in = rvalid && j0 + j < ncol;
-                        const long long o = off0 + (long long)(j0 + j) * cstep;
-                        b[j] = y[j] = 0.0;
-                        if (EPI == EPI_AXPY && in && first) b[j] = p.base[o];
-                        if (EPI == EPI_PHI && in) b[j] = f64_phi(p, o);
-                        if (in && !first) y[j] = p.Y[o];
-                    }
-                };
-                load_side(jlo, bcur, ycur);
                 const bool waited = mbar_wait(accf, seg & 1u, p.err, 2, &abort_s, 32);
                 if (!__all_sync(0xffffffffu, waited)) { ok = false; break; }
                 tc_fence_after();
-                const int* es_t = es_s[tl & 3];
-                const int esrow = SA ? es_t[row] : 0;
+                if (!warp_on) {
+                    if (lane == 0) mbar_arrive(acce);
+                    continue;
+                }
+                // the axpy's base or the phi table's values of four columns, and the earlier segments' sum,
+                // one group ahead
+                double bcur[4], bnxt[4];
+                auto load_base = [&](int j0, double (&b)[4]) {
+                    if (EPI == EPI_STORE || (EPI == EPI_AXPY && !first)) return;
+                    if (EPI == EPI_PHI && !p.phi) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) b[j] = rvalid && j0 + j < ncol ? f64_phi_eval(p, off_t[j0 + j] + ioff) : 0.0;
+                        return;
+                    }
+                    const double* src = EPI == EPI_PHI ? p.phi : p.base;
+                    if (p.vec4 && rvalid && j0 + 3 < ncol) {
+                        ld4(src + off_t[j0] + ioff, b);
+                        return;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) b[j] = rvalid && j0 + j < ncol ? src[off_t[j0 + j] + ioff] : 0.0;
+                };
+                load_base(jlo, bcur);
 #pragma unroll 1
                 for (int j0 = jlo; j0 < jhi; j0 += 4) {
                     float d[kSl][4];
-                    if (j0 + 4 < jhi) load_side(j0 + 4, bnxt, ynxt);
-                    int es4[4];
+                    if (j0 + 4 < jhi) load_base(j0 + 4, bnxt);
+                    int es[4];
+                    long long off[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) es4[j] = SA ? esrow : es_t[j0 + j];
+                    for (int j = 0; j < 4; ++j) {
+                        es[j] = es_t[j0 + j];
+                        off[j] = off_t[j0 + j] + ioff;
+                    }
                     __syncwarp();
                     tmem_ld4x7(tbase + j0, uint32_t(N), d);
                     if (j0 + 4 >= jhi) {                     // the last columns are in registers: TMEM is free
@@ -410,35 +430,46 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
                         __syncwarp();
                         if (lane == 0) mbar_arrive(acce);
                     }
+                    double v[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        int sh = rsh, e = rexp;
-                        if (SA) {
-                            const int2 cp = __ldg(p.rows + ot * N + j0 + j);
-                            sh = cp.y;
-                            e = cp.x;
-                        }
-                        double v = 0.0;
-                        if (es4[j] != kNoCut) v = assemble(d, j, sh, e + es4[j]);
-                        else if (first && rvalid && j0 + j < ncol)
-                            v = SA ? fma_dot(p.factor + (long long)(ot * N + j0 + j) * n, xline, n, Q)
-                                   : fma_dot(p.factor + (long long)(ot * kM + row) * n, xline + (long long)(j0 + j) * n, n, 1);
-                        if (EPI == EPI_PHI) v *= bcur[j];
-                        if (EPI == EPI_AXPY) v = first ? fma(p.alpha, v, bcur[j]) : fma(p.alpha, v, ycur[j]);
-                        else if (!first) v += ycur[j];
-                        if (rvalid && j0 + j < ncol) p.Y[off0 + (long long)(j0 + j) * cstep] = v;
+                    for (int j = 0; j < 4; ++j) v[j] = assemble(d, j, rexp + es[j]);
+                    if (max(max(es[0], es[1]), max(es[2], es[3])) == kNoCut) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (es[j] == kNoCut)
+                                v[j] = first && rvalid && j0 + j < ncol
+                                           ? fma_dot(p.factor + (long long)irow * n, p.X + off[j] - ioff, n, Q) : 0.0;
+                    }
+                    if (EPI == EPI_PHI) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) v[j] *= bcur[j];
+                    }
+                    if (EPI == EPI_AXPY && first) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) v[j] = fma(p.alpha, v[j], bcur[j]);
+                    }
+                    if (!first) {                            // lines past one segment: add to the earlier ones' sum
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (rvalid && j0 + j < ncol) v[j] = fma(EPI == EPI_AXPY ? p.alpha : 1.0, v[j], p.Y[off[j]]);
+                    }
+                    if (p.vec4 && rvalid && j0 + 3 < ncol) {
+                        st4(p.Y + off[0], v);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (rvalid && j0 + j < ncol) p.Y[off[j]] = v[j];
                     }
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) { bcur[j] = bnxt[j]; ycur[j] = ynxt[j]; }
+                    for (int j = 0; j < 4; ++j) bcur[j] = bnxt[j];
                 }
             }
         }
     } else if (warp == kMmaWarp && lane == 0) {
         // ------------------------------------------------------------ MMA issuer
-        // With X the slices of the A operand and Y those of B (X = S, Y = F for SA, else the other way),
-        // X_i.Y_j adds to D_(i+j). The Y tiles lie one after another, as do the accumulators, so X_i
-        // takes up to 256 / N consecutive Y_j in one MMA of up to 256 columns: 10 MMAs per
-        // K step instead of 28 at N = 64, and X_i is read from shared memory once for them.
+        // F_i.S_j adds to D_(i+j). The S tiles lie one after another, as do the accumulators, so F_i
+        // takes up to 256 / N consecutive S_j in one MMA of up to 256 columns: 10 MMAs per
+        // K step instead of 28 at N = 64, and F_i is read from shared memory once for them.
         uint32_t seg = 0, sph = 0, fph = 0;
         int s = 0, fs = 0;
         bool ok = true;
@@ -453,7 +484,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
                 if (!mbar_wait(sfull(s), sph, p.err, 8, &abort_s)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t sS = sbase + s * C::SBYTES, sF = fbase + fs * C::FBYTES;
-                const uint64_t a0 = sdesc64(SA ? sS : sF), b0 = sdesc64(SA ? sF : sS);
+                const uint64_t a0 = sdesc64(sF), b0 = sdesc64(sS);
 #pragma unroll
                 for (int kk = 0; kk < kKc / 16; ++kk) {
                     const uint64_t adv = uint64_t(kk * 32) >> 4;
@@ -462,8 +493,8 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
 #pragma unroll
                         for (int j = 0; j < kSl - i; j += C::WIDE) {
                             const int w = (kSl - i - j) < C::WIDE ? (kSl - i - j) : C::WIDE;
-                            tc_mma(tmem + (i + j) * N, a0 + adv + uint64_t(i * C::ATILE >> 4),
-                                   b0 + adv + uint64_t(j * C::BTILE >> 4), idesc_of(w * N),
+                            tc_mma(tmem + (i + j) * N, a0 + adv + uint64_t(i * C::FTILE >> 4),
+                                   b0 + adv + uint64_t(j * C::STILE >> 4), idesc_of(w * N),
                                    (first && kk == 0 && i == 0) ? 0u : 1u);
                         }
                 }
@@ -491,44 +522,32 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
     }
 }
 
-// Cut the dense factor (n x n, row-major) into its image: per (tile of `rows` rows, K chunk of 32)
-// seven 64-byte-swizzled K-major tiles, and per row {ef, sh}. One block per padded row.
-__global__ void f64_factor_kernel(const double* M, int n, int rows, int nK, uint8_t* img, int2* rp) {
+// Cut the dense factor (n x n, row-major) into its image: per (tile of 128 rows, K chunk of 32)
+// seven 64-byte-swizzled K-major tiles; and per row the exponent of the result's unit, less es. One block per
+// padded row.
+__global__ void f64_factor_kernel(const double* M, int n, int nK, uint8_t* img, int* rows) {
     const int i = blockIdx.x;
     __shared__ unsigned smax;
-    __shared__ double ssum;
-    if (threadIdx.x == 0) { smax = 0; ssum = 0.0; }
+    if (threadIdx.x == 0) smax = 0;
     __syncthreads();
     unsigned m = 0;
     if (i < n)
         for (int k = threadIdx.x; k < n; k += blockDim.x) m = max(m, f64_amax_bits(M[(size_t)i * n + k]));
     atomicMax(&smax, m);
     __syncthreads();
-    const int e = int(smax >> 20);
     // max|f| < 2^ef; rows below 2^-500 keep that scale (their digits are then smaller)
-    const int ef = smax ? max(e - 1022, -500) : 0;
-    double sum = 0.0;
-    if (i < n)
-        for (int k = threadIdx.x; k < n; k += blockDim.x) sum += fabs(M[(size_t)i * n + k]);
-    atomicAdd(&ssum, sum);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // |T| <= 2^64 sum|f| 2^-ef: sh so that T / 2^sh stays below 2^51 (n <= 1024: sh <= 24)
-        int q = 0;
-        const double s = ldexp(ssum, -ef) * (1.0 + 1e-6);
-        if (s > 0.0) frexp(s, &q);
-        rp[i] = make_int2(ef - 64, min(max(13 + q, 1), 24));
-    }
-    uint8_t* tile = img + (size_t)(i / rows) * nK * kSl * rows * 64;
+    const int ef = smax ? max(int(smax >> 20) - 1022, -500) : 0;
+    if (threadIdx.x == 0) rows[i] = ef - 64;
+    uint8_t* tile = img + (size_t)(i / kM) * nK * kSl * kM * 64;
     for (int k = threadIdx.x; k < nK * kKc; k += blockDim.x) {
         const double f = (i < n && k < n) ? M[(size_t)i * n + k] : 0.0;
         float s[kSl];
         cut(f, ef + 1022, s);
         const int kc = k % kKc;
-        uint8_t* dst = tile + (size_t)(k / kKc) * kSl * rows * 64 + swz64(i % rows, kc / 8) + (kc % 8) * 2;
+        uint8_t* dst = tile + (size_t)(k / kKc) * kSl * kM * 64 + swz64(i % kM, kc / 8) + (kc % 8) * 2;
 #pragma unroll
         for (int q = 0; q < kSl; ++q)
-            *reinterpret_cast<uint16_t*>(dst + (size_t)q * rows * 64) = uint16_t(__float_as_uint(s[q]) >> 16);
+            *reinterpret_cast<uint16_t*>(dst + (size_t)q * kM * 64) = uint16_t(__float_as_uint(s[q]) >> 16);
     }
 }
 
@@ -551,43 +570,30 @@ int sm_count() {
     return sms;
 }
 
-template <bool SA, int N, int EPI>
+template <bool MODE1, int N, int EPI>
 cudaError_t launch_variant(const F64Args& a, cudaStream_t s) {
-    static const cudaError_t attr = cudaFuncSetAttribute(f64_contract_kernel<SA, N, EPI>,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<SA, N>::SMEM);
+    static const cudaError_t attr = cudaFuncSetAttribute(f64_contract_kernel<MODE1, N, EPI>,
+                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<N>::SMEM);
     if (attr != cudaSuccess) return attr;
-    const long long grid = a.ntiles < sm_count() ? a.ntiles : sm_count();
-    f64_contract_kernel<SA, N, EPI><<<unsigned(grid), kThreads, Cfg<SA, N>::SMEM, s>>>(a);
+    const int grid = a.ntiles < sm_count() ? a.ntiles : sm_count();
+    f64_contract_kernel<MODE1, N, EPI><<<unsigned(grid), kThreads, Cfg<N>::SMEM, s>>>(a);
     return cudaGetLastError();
 }
 
-template <bool SA, int N>
+template <bool MODE1, int N>
 cudaError_t launch_epi(const F64Args& a, cudaStream_t s) {
-    if (a.epi == EPI_PHI) return launch_variant<SA, N, EPI_PHI>(a, s);
-    if (a.epi == EPI_AXPY) return launch_variant<SA, N, EPI_AXPY>(a, s);
-    return launch_variant<SA, N, EPI_STORE>(a, s);
+    if (a.epi == EPI_PHI) return launch_variant<MODE1, N, EPI_PHI>(a, s);
+    if (a.epi == EPI_AXPY) return launch_variant<MODE1, N, EPI_AXPY>(a, s);
+    return launch_variant<MODE1, N, EPI_STORE>(a, s);
 }
 
 }  // namespace
 
-F64Tiles f64_tiles(int n, long long npos, bool mode1) {
-    F64Tiles t;
-    t.nK = (n + kKc - 1) / kKc;
-    // 64 columns, or 32 where 64 would give fewer tiles than SMs
-    for (int cols : {64, 32}) {
-        t.cols = cols;
-        t.rows = mode1 ? kM : cols;                          // factor rows per tile
-        t.nOut = (n + t.rows - 1) / t.rows;
-        t.ntiles = (mode1 ? (npos + cols - 1) / cols : (npos + kM - 1) / kM) * t.nOut;
-        if (t.ntiles >= sm_count()) break;
-    }
-    return t;
-}
+size_t f64_image_bytes(int n) { return size_t((n + kM - 1) / kM) * kM * ((n + kKc - 1) / kKc) * kKc * 2 * kSl; }
+int f64_rows(int n) { return (n + kM - 1) / kM * kM; }
 
-size_t f64_image_bytes(const F64Tiles& t) { return size_t(t.nOut) * t.rows * t.nK * kKc * 2 * kSl; }
-
-cudaError_t launch_f64_factor(const double* M, int n, const F64Tiles& t, uint8_t* img, int2* rows, cudaStream_t s) {
-    f64_factor_kernel<<<t.nOut * t.rows, 128, 0, s>>>(M, n, t.rows, t.nK, img, rows);
+cudaError_t launch_f64_factor(const double* M, int n, uint8_t* img, int* rows, cudaStream_t s) {
+    f64_factor_kernel<<<f64_rows(n), 128, 0, s>>>(M, n, (n + kKc - 1) / kKc, img, rows);
     return cudaGetLastError();
 }
 
@@ -597,10 +603,19 @@ cudaError_t launch_f64_phi(double* tab, int k, double ctau, const double* const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_contract_f64(const F64Args& a, bool mode1, int cols, cudaStream_t s) {
-    if (a.ntiles <= 0) return cudaSuccess;
-    if (mode1) return cols == 64 ? launch_epi<false, 64>(a, s) : launch_epi<false, 32>(a, s);
-    return cols == 64 ? launch_epi<true, 64>(a, s) : launch_epi<true, 32>(a, s);
+cudaError_t launch_contract_f64(F64Args a, cudaStream_t s) {
+    if (a.npos <= 0) return cudaSuccess;
+    const bool mode1 = a.Q == 1;
+    a.nK = (a.n + kKc - 1) / kKc;
+    a.nOut = (a.n + kM - 1) / kM;
+    auto aligned = [](const void* q, uintptr_t to) { return reinterpret_cast<uintptr_t>(q) % to == 0; };
+    a.vec2 = a.n % 2 == 0 && aligned(a.X, 16);
+    // groups of four columns are four consecutive nodes: modes >= 2, q a multiple of 4
+    a.vec4 = !mode1 && a.Q % 4 == 0 && aligned(a.Y, 32) && aligned(a.base, 32) && aligned(a.phi, 32);
+    const bool wide = (a.npos + 63) / 64 * a.nOut >= sm_count();
+    a.ntiles = int((a.npos + (wide ? 63 : 31)) / (wide ? 64 : 32) * a.nOut);
+    if (mode1) return wide ? launch_epi<true, 64>(a, s) : launch_epi<true, 32>(a, s);
+    return wide ? launch_epi<false, 64>(a, s) : launch_epi<false, 32>(a, s);
 }
 
 }  // namespace adr

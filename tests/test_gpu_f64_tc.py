@@ -14,7 +14,7 @@ from test_gpu_parity import adr, check_guards, guarded, make_case, torch
 
 pytestmark = pytest.mark.gpu
 
-# every one above the work from which FP64 contexts use the tensor cores (4e6 FMAs a pass)
+# every one above the work from which FP64 contexts use the tensor cores (1.5e6 FMAs a pass)
 DIMS = [(65, 400), (257, 127), (520, 60), (300, 130), (64, 64, 64), (127, 33, 65), (31, 129, 96), (130, 65, 67)]
 
 
