@@ -63,6 +63,10 @@ constexpr int kMmaWarp = kProducerWarps + kEpiWarps;
 constexpr int kLoadWarp = kMmaWarp + 1;
 constexpr int kThreads = (kLoadWarp + 1) * 32;
 
+// Tiles whose line scales are kept: the producers run ahead of the epilogue by the tile whose MMAs wait for it and, at one
+// chunk a tile, by one tile more per stage of their ring.
+constexpr int kTileBufs = 8;
+
 template <int N>
 struct Cfg {
     static constexpr int FTILE = kM * kKc * 2, STILE = N * kKc * 2;   // one slice tile of either operand
@@ -74,7 +78,8 @@ struct Cfg {
     static constexpr int WIDE = 256 / N;                              // slices per MMA (N <= 256)
     static constexpr int KV = N * kKc / (kProducerWarps * 32);        // K values a producer thread cuts per chunk
     static constexpr int KG = kKc / KV;                               // threads per line
-    static_assert(SMEM <= 222 * 1024, "shared memory budget");
+    static_assert(NS + 3 <= kTileBufs, "line scales of every tile in flight");
+    static_assert(SMEM <= 215 * 1024, "shared memory budget");
 };
 
 __device__ __forceinline__ uint32_t idesc_of(int ncols) {   // FP32 accumulator, BF16 operands, M = 128
@@ -204,9 +209,9 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
     __shared__ __align__(8) uint64_t bars[kDR / 8 + 1];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
-    // per line of the last four tiles: its exponent es, and its offset in the state (k = 0)
-    __shared__ int es_s[4][N];
-    __shared__ long long off_s[4][N];
+    // per line of the last tiles: its exponent es, and its offset in the state (k = 0)
+    __shared__ int es_s[kTileBufs][N];
+    __shared__ long long off_s[kTileBufs][N];
     __shared__ unsigned part_s[2][C::KG][N];                 // modes >= 2: the parts of a line's max|x|
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -335,8 +340,8 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
             live = m == 0u || (eb >= 1023 - 500 && eb <= 1023 + 500);
             etop = m ? eb : 1022;                            // es + 1022
             if (kg == 0) {
-                es_s[tl & 3][row] = live ? etop - 1022 : kNoCut;
-                off_s[tl & 3][row] = xoff;
+                es_s[tl & (kTileBufs - 1)][row] = live ? etop - 1022 : kNoCut;
+                off_s[tl & (kTileBufs - 1)][row] = xoff;
             }
         };
         set_row();
@@ -382,8 +387,8 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
             const int ncol = min(N, int(p.npos - (long long)pt * N));
             const int rexp = __ldg(p.rows + irow);           // padded to whole tiles
             const long long ioff = irow * Q;
-            const long long* off_t = off_s[tl & 3];
-            const int* es_t = es_s[tl & 3];
+            const long long* off_t = off_s[tl & (kTileBufs - 1)];
+            const int* es_t = es_s[tl & (kTileBufs - 1)];
             for (int c0 = 0; c0 < p.nK; c0 += kSegChunks, ++seg) {
                 const bool first = c0 == 0;
                 const bool waited = mbar_wait(accf, seg & 1u, p.err, 2, &abort_s, 32);
