@@ -125,6 +125,7 @@ struct adr_ctx {
 
     // device memory (library-owned)
     void* d_a = nullptr;                   // nodal (a - abar)
+    void* d_face[3] = {nullptr, nullptr, nullptr};   // FP64 flux form: its face weights instead
     void* d_E[3][3] = {{nullptr}};         // e^{c tau A_mu}, c = 0.5 (0), 1 (1), alpha (2)
     void* d_V[3] = {nullptr};
     void* d_Vi[3] = {nullptr};
@@ -722,7 +723,8 @@ void push_stencil(Sched& S, StencilArgs<T> s, bool record_input = false);
 template <typename T>
 StencilArgs<T> linear_base(const adr_ctx* c, const T* u) {
     StencilArgs<T> s = stencil_base<T>(c, u);
-    s.a = static_cast<const T*>(c->d_a0);
+    s.a = static_cast<const T*>(c->d_a0);   // FP64: no array at all
+    for (int m = 0; m < 3; ++m) s.face[m] = nullptr;
     for (int m = 0; m < 3; ++m) s.bmb[m] = 0.0;
     for (int i = 0; i < 4; ++i) s.r[i] = 0.0;
     return s;
@@ -827,6 +829,7 @@ StencilArgs<T> stencil_base(const adr_ctx* c, const T* u) {
     s.u = u;
     s.err = c->d_err;
     s.a = static_cast<const T*>(c->d_a);
+    for (int m = 0; m < 3; ++m) s.face[m] = static_cast<const T*>(c->d_face[m]);
     s.apitch = c->apitch;
     s.dim = c->dim;
     s.n1 = c->n[0];
@@ -1756,7 +1759,7 @@ adr_status setup_doubling(adr_ctx* c) {
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "upload doubling factors");
     const size_t abytes = size_t(c->apitch) * (c->n[1] + 2) * (c->dim == 3 ? c->n[2] + 2 : 1) * c->esize;
-    if (!c->d_a0) {
+    if (!c->d_a0 && !c->fp64) {            // the FP64 stencil takes no array for zero
         e = cudaMalloc(&c->d_a0, abytes);
         if (e == cudaSuccess) e = cudaMemset(c->d_a0, 0, abytes);
     }
@@ -1979,6 +1982,19 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
     if (c->d_a) { void* q = c->d_a; free_dev(q); c->d_a = nullptr; }
     cudaError_t e = upload(c, &c->d_a, amb);
     if (e != cudaSuccess) return cuda_fail(c, e, "upload a");
+    if (c->fp64 && c->p.form == ADR_FORM_FLUX) {   // face weights in place of the nodal array
+        const long long next[3] = {1, c->apitch, (long long)c->apitch * N2};
+        for (int m = 0; m < c->dim && e == cudaSuccess; ++m) {
+            const double h = neumann ? 1.0 / c->n[m] : 1.0 / (c->n[m] + 1);
+            if (!c->d_face[m]) e = cudaMalloc(&c->d_face[m], amb.size() * sizeof(double));
+            if (e == cudaSuccess)
+                e = adr::launch_f64_faces(static_cast<const double*>(c->d_a), static_cast<double*>(c->d_face[m]), 1.0 / (h * h),
+                                          next[m], (long long)amb.size(), nullptr);
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+        if (e != cudaSuccess) return cuda_fail(c, e, "face weights");
+        free_dev(c->d_a);
+    }
 
     c->f64tc = c->f64_grid;
     c->eig_real = true;
@@ -2432,6 +2448,7 @@ void adr_destroy(adr_ctx* c) {
         { void* q = b.d_bslots; free_dev(q); b.d_bslots = nullptr; }
     }
     free_dev(c->d_a);
+    for (auto& q : c->d_face) free_dev(q);
     for (auto& row : c->d_E) for (auto& p : row) free_dev(p);
     for (auto& p : c->d_V) free_dev(p);
     for (auto& p : c->d_Vi) free_dev(p);

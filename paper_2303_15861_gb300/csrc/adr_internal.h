@@ -87,6 +87,8 @@ struct StencilArgs {
                                      // node (j1, j2, j3) in 0..n+1 at
                                      // (j3 * (n2 + 2) + j2) * apitch + j1 + 3
     int apitch = 0;                  // row pitch of a: multiple of 4, >= n1 + 5
+    const T* face[3] = {nullptr, nullptr, nullptr};   // FP64 flux form: (1/2h^2) times the sums of a across the
+                                     // faces, at the lower node, laid out as a (NULL: a = 0)
     int dim = 3, n1 = 1, n2 = 1, n3 = 1;
     bool neumann = false;            // homogeneous Neumann faces at x_mu = 1: mirror ghosts
     bool adelta = false;             // (a - abar) Lap u instead of div((a - abar) grad u)
@@ -226,6 +228,8 @@ cudaError_t launch_contract_tc(const TcArgs& a, cudaStream_t s);
 cudaError_t launch_amax(const float* x, size_t n, unsigned* slot, cudaStream_t s);
 
 cudaError_t launch_stencil(const StencilArgs<double>& a, cudaStream_t s);
+// Face weights of one direction from the nodal array (next: elements to the next node along it).
+cudaError_t launch_f64_faces(const double* a, double* w, double inv_h2, long long next, long long total, cudaStream_t s);
 cudaError_t launch_stencil(const StencilArgs<float>& a, cudaStream_t s);
 cudaError_t launch_contract(const ContractArgs<double>& a, cudaStream_t s);
 cudaError_t launch_contract(const ContractArgs<float>& a, cudaStream_t s);

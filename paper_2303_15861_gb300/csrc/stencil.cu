@@ -9,11 +9,10 @@
 // Dirichlet ghosts u = 0. F = g + A u.
 //
 // Layout: u is n3*n2*n1 (x1 fastest), the nodal (a - abar) is (n3+2)(n2+2)(n1+2).
-// A CTA covers 32 x 8 nodes of (x1, x2) and ZCHUNK planes of x3.
+// These are the FP32 forms (FP64: stencil_f64.cu). A CTA covers 32 x 8 nodes of (x1, x2) and ZCHUNK planes of x3.
 #include <cuda_runtime.h>
 
 #include <cstdint>
-#include <type_traits>
 
 #include "adr_internal.h"
 #include "stencil_core.cuh"
@@ -443,54 +442,51 @@ cudaError_t launch_march(const StencilArgs<float>& p, const Coefs<float>& c, boo
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_impl(const StencilArgs<T>& p, cudaStream_t s) {
-    Coefs<T> c;
+cudaError_t launch_f32(const StencilArgs<float>& p, cudaStream_t s) {
+    Coefs<float> c;
     for (int m = 0; m < 3; ++m) {
-        c.ih2[m] = T(p.inv_h2[m]);
-        c.i2h[m] = T(p.inv_2h[m]);
-        c.bmb[m] = T(p.bmb[m]);
-        c.beta[m] = T(p.beta[m]);
+        c.ih2[m] = float(p.inv_h2[m]);
+        c.i2h[m] = float(p.inv_2h[m]);
+        c.bmb[m] = float(p.bmb[m]);
+        c.beta[m] = float(p.beta[m]);
     }
-    c.abar = T(p.abar);
-    c.r0 = T(p.r[0]); c.r1 = T(p.r[1]); c.r2 = T(p.r[2]); c.r3 = T(p.r[3]);
+    c.abar = float(p.abar);
+    c.r0 = float(p.r[0]); c.r1 = float(p.r[1]); c.r2 = float(p.r[2]); c.r3 = float(p.r[3]);
     bool needF = false;
     for (int j = 0; j < kMaxOut; ++j) {
-        c.cg[j] = T(p.cg[j]); c.cF[j] = T(p.cF[j]);
-        state_coefs<T>(p.cu[j], p.cx[j], c.cu[j], c.cx[j]);
+        c.cg[j] = float(p.cg[j]); c.cF[j] = float(p.cF[j]);
+        state_coefs<float>(p.cu[j], p.cx[j], c.cu[j], c.cx[j]);
         if (j < p.nout && p.cF[j] != 0.0) needF = true;
     }
     dim3 block(TX * TY);
-    if constexpr (std::is_same<T, float>::value) {
-        bool aligned = (p.n1 % 4 == 0) && (p.apitch % 4 == 0) && (reinterpret_cast<uintptr_t>(p.u) % 16 == 0) &&
-                       (reinterpret_cast<uintptr_t>(p.a) % 16 == 0);
-        for (int j = 0; j < p.nout; ++j) aligned = aligned && (reinterpret_cast<uintptr_t>(p.out[j]) % 16 == 0);
-        for (int e = 0; e < p.nx; ++e) aligned = aligned && (reinterpret_cast<uintptr_t>(p.X[e]) % 16 == 0);
-        // the vectorised 2-D kernel has Dirichlet ghosts and the flux form only
-        if (p.dim == 2 && (p.neumann || p.adelta)) aligned = false;
-        if (p.u_lo) aligned = aligned && (reinterpret_cast<uintptr_t>(p.u_lo) % 16 == 0);
-        if (aligned) {
-            dim3 g4((p.n1 / 4 + 31) / 32, (p.n2 + 7) / 8, p.dim == 3 ? (p.n3 + ZV - 1) / ZV : 1);
-            if (p.dim == 3) {
-                if (stencil_tma_usable(p)) return launch_stencil_tma(p, c, needF, s);
-                const int zb = kMarchPlanes;
-                dim3 gm((p.n1 / 4 + 31) / 32, (p.n2 + 7) / 8, (p.n3 + zb - 1) / zb);
-                return launch_march(p, c, needF, zb, gm, s);
-            } else {
-                if (p.u_lo) stencil_vec4_kernel<2, true><<<g4, 256, 0, s>>>(p, c, needF);
-                else        stencil_vec4_kernel<2, false><<<g4, 256, 0, s>>>(p, c, needF);
-            }
-            return cudaGetLastError();
+    bool aligned = (p.n1 % 4 == 0) && (p.apitch % 4 == 0) && (reinterpret_cast<uintptr_t>(p.u) % 16 == 0) &&
+                   (reinterpret_cast<uintptr_t>(p.a) % 16 == 0);
+    for (int j = 0; j < p.nout; ++j) aligned = aligned && (reinterpret_cast<uintptr_t>(p.out[j]) % 16 == 0);
+    for (int e = 0; e < p.nx; ++e) aligned = aligned && (reinterpret_cast<uintptr_t>(p.X[e]) % 16 == 0);
+    // the vectorised 2-D kernel has Dirichlet ghosts and the flux form only
+    if (p.dim == 2 && (p.neumann || p.adelta)) aligned = false;
+    if (p.u_lo) aligned = aligned && (reinterpret_cast<uintptr_t>(p.u_lo) % 16 == 0);
+    if (aligned) {
+        dim3 g4((p.n1 / 4 + 31) / 32, (p.n2 + 7) / 8, p.dim == 3 ? (p.n3 + ZV - 1) / ZV : 1);
+        if (p.dim == 3) {
+            if (stencil_tma_usable(p)) return launch_stencil_tma(p, c, needF, s);
+            const int zb = kMarchPlanes;
+            dim3 gm((p.n1 / 4 + 31) / 32, (p.n2 + 7) / 8, (p.n3 + zb - 1) / zb);
+            return launch_march(p, c, needF, zb, gm, s);
+        } else {
+            if (p.u_lo) stencil_vec4_kernel<2, true><<<g4, 256, 0, s>>>(p, c, needF);
+            else        stencil_vec4_kernel<2, false><<<g4, 256, 0, s>>>(p, c, needF);
         }
+        return cudaGetLastError();
     }
     dim3 grid((p.n1 + TX - 1) / TX, (p.n2 + TY - 1) / TY, p.dim == 3 ? (p.n3 + ZCHUNK - 1) / ZCHUNK : 1);
-    const bool lo = std::is_same<T, float>::value && p.u_lo != nullptr;
+    const bool lo = p.u_lo != nullptr;
     if (p.dim == 3) {
-        if (lo) stencil_kernel<T, 3, ZCHUNK, true><<<grid, block, 0, s>>>(p, c, needF);
-        else    stencil_kernel<T, 3, ZCHUNK, false><<<grid, block, 0, s>>>(p, c, needF);
+        if (lo) stencil_kernel<float, 3, ZCHUNK, true><<<grid, block, 0, s>>>(p, c, needF);
+        else    stencil_kernel<float, 3, ZCHUNK, false><<<grid, block, 0, s>>>(p, c, needF);
     } else {
-        if (lo) stencil_kernel<T, 2, 1, true><<<grid, block, 0, s>>>(p, c, needF);
-        else    stencil_kernel<T, 2, 1, false><<<grid, block, 0, s>>>(p, c, needF);
+        if (lo) stencil_kernel<float, 2, 1, true><<<grid, block, 0, s>>>(p, c, needF);
+        else    stencil_kernel<float, 2, 1, false><<<grid, block, 0, s>>>(p, c, needF);
     }
     return cudaGetLastError();
 }
@@ -509,8 +505,7 @@ __global__ void convert_kernel(const double* in, float* out, size_t n) {
 
 }  // namespace
 
-cudaError_t launch_stencil(const StencilArgs<double>& a, cudaStream_t s) { return launch_impl(a, s); }
-cudaError_t launch_stencil(const StencilArgs<float>& a, cudaStream_t s) { return launch_impl(a, s); }
+cudaError_t launch_stencil(const StencilArgs<float>& a, cudaStream_t s) { return launch_f32(a, s); }
 
 cudaError_t launch_amax(const float* x, size_t n, unsigned* slot, cudaStream_t s) {
     const int blocks = int(std::min<size_t>((n + 255) / 256, 152 * 8));

@@ -1,0 +1,293 @@
+// K1 in FP64 (Eq. (nonlin), Section 3; see stencil.cu for the discretisation): every grid form, 2-D and
+// 3-D, Dirichlet or Neumann faces, flux or a Lap u form.
+//
+// What bounds it. The FP64 pipe: 2 instructions' lanes per clock and SM, so one FP64 instruction per
+// node costs as much time as 12 bytes of HBM traffic. The kernel therefore trades memory for
+// instructions: the face weights w_mu = (1/2h^2) ((a - abar)_i + (a - abar)_{i+e}) are stored (three arrays
+// beside u instead of one: 24 bytes more a node, 6 additions and 9 multiplications less), differences
+// are formed once per face and shared (pairs along x1 in a thread, planes along x3 in
+// registers), and terms whose coefficient is zero are left out by branches that every thread takes alike.
+// Per node and direction: d+ (shared), two FMAs with the face weights; M = u+ - u- and one FMA
+// where b - beta is not zero; for F, L = d+ - d- and one FMA with abar / h^2, and one FMA of M with beta / (2h).
+// u + tau/2 g in 3-D: 16 FP64 instructions a node instead of about 75; F and g: 27 instead of 85.
+// Time of a launch, per-node kernel -> this one (us): 256^3, one output 2139 -> 788, two outputs and one or two
+// stage inputs 2460 -> 975; 128^3, F and g 379 -> 197, g - G0 283 -> 104; 60^3 Neumann, a Lap u form 39 -> 22; 32^2 12.6 -> 7.0.
+#include <cuda_runtime.h>
+
+#include "adr_internal.h"
+#include "stencil_core.cuh"
+
+namespace adr {
+namespace {
+
+constexpr int kTX = 32, kTY = 8;         // threads of a block along x1 (V nodes each), the most along x2
+
+// Folded per-direction weights.
+struct Weights {
+    double w2[3];                        // (b - beta) / (2h)
+    double wa[3], wb[3];                 // abar / h^2, beta / (2h)
+    double ih2[3];
+    const double* face[3];               // face weights, laid out as StencilArgs::a (NULL: a = abar everywhere)
+    // which terms there are: tested as integers, since a comparison of doubles costs an FP64 instruction
+    unsigned adv, advF;                  // bit mu: w2, wb not zero
+    int start[kMaxOut];                  // a term of coefficient one: 1 u, 2 + e X_e; 0 none
+    unsigned terms[kMaxOut];             // the other terms that are not zero: bits kTu, kTg, kTF, kTx + e
+};
+constexpr unsigned kTu = 0, kTg = 1, kTF = 2, kTx = 3;
+
+template <int V>
+__device__ __forceinline__ void ldv(const double* p, double (&v)[V]) {
+    if constexpr (V == 2) {
+        const double2 t = __ldg(reinterpret_cast<const double2*>(p));
+        v[0] = t.x;
+        v[1] = t.y;
+    } else {
+        v[0] = __ldg(p);
+    }
+}
+template <int V>
+__device__ __forceinline__ void stv(double* p, const double (&v)[V]) {
+    if constexpr (V == 2) *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+    else *p = v[0];
+}
+
+// A thread owns V consecutive x1 nodes of one row and walks zb planes of x3; u of the planes z - 1 and z
+// and the face weights below plane z stay in registers, the neighbours along x1 and x2 come from L1.
+template <int DIM, int V, bool ADELTA, bool NEEDF>
+__global__ void __launch_bounds__(kTX * kTY) stencil_f64_kernel(StencilArgs<double> p, Coefs<double> c, Weights w, int zb) {
+    const int n1 = p.n1, n2 = p.n2, n3 = DIM == 3 ? p.n3 : 1;
+    const int i1 = (int(blockIdx.x) * kTX + int(threadIdx.x % kTX)) * V;
+    const int i2 = int(blockIdx.y) * int(blockDim.x / kTX) + int(threadIdx.x / kTX);
+    if (i1 >= n1 || i2 >= n2) return;                        // V = 2: n1 is even
+    const long long plane_u = (long long)n1 * n2, plane_a = (long long)p.apitch * (n2 + 2);
+    const int z0 = DIM == 3 ? int(blockIdx.z) * zb : 0, z1 = DIM == 3 ? min(z0 + zb, n3) : 1;
+    const double* u = p.u + (long long)i2 * n1 + i1 + z0 * plane_u;
+    const long long ao = (long long)(i2 + 1) * p.apitch + (i1 + 4) + (DIM == 3 ? (z0 + 1) * plane_a : 0);
+    const double* aC = ADELTA && p.a ? p.a + ao : nullptr;
+    const bool faces = !ADELTA && w.face[0];
+    const double* f1 = faces ? w.face[0] + ao : nullptr;
+    const double* f2 = faces ? w.face[1] + ao : nullptr;
+    const double* f3 = faces && DIM == 3 ? w.face[2] + ao : nullptr;
+
+    double uM[V], uC[V], dM[V], fM[V];
+    ldv<V>(u, uC);
+#pragma unroll
+    for (int k = 0; k < V; ++k) uM[k] = fM[k] = 0.0;
+    if (DIM == 3) {
+        if (z0 > 0) ldv<V>(u - plane_u, uM);
+        if (faces) ldv<V>(f3 - plane_a, fM);
+#pragma unroll
+        for (int k = 0; k < V; ++k) dM[k] = uC[k] - uM[k];
+    }
+    long long idx = (long long)i2 * n1 + i1 + z0 * plane_u;
+    for (int z = z0; z < z1; ++z) {
+        double uP[V], uS[V], uN[V], fS[V], fN[V], fE[V], fP[V], a0[V], x[kMaxExtra][V];
+        double uW = 0.0, uE = 0.0, fW = 0.0;
+#pragma unroll
+        for (int k = 0; k < V; ++k) uP[k] = uS[k] = uN[k] = 0.0;
+        if (DIM == 3) {
+            if (z + 1 < n3) ldv<V>(u + plane_u, uP);
+            else if (p.neumann) {                            // Neumann face: the ghost mirrors plane n3 - 2
+#pragma unroll
+                for (int k = 0; k < V; ++k) uP[k] = uM[k];
+            }
+        }
+        if (i2 > 0) ldv<V>(u - n1, uS);
+        if (i2 + 1 < n2) ldv<V>(u + n1, uN);
+        else if (p.neumann) {
+#pragma unroll
+            for (int k = 0; k < V; ++k) uN[k] = uS[k];
+        }
+        if (i1 > 0) uW = __ldg(u - 1);
+        if (i1 + V < n1) uE = __ldg(u + V);
+        else if (p.neumann) uE = V == 2 ? uC[0] : uW;
+        if (faces) {
+            fW = __ldg(f1 - 1);
+            ldv<V>(f1, fE);
+            ldv<V>(f2 - p.apitch, fS);
+            ldv<V>(f2, fN);
+            if (DIM == 3) ldv<V>(f3, fP);
+        }
+        if (ADELTA && aC) ldv<V>(aC, a0);
+#pragma unroll
+        for (int e = 0; e < kMaxExtra; ++e)
+            if (e < p.nx) ldv<V>(p.X[e] + idx, x[e]);
+
+        double dW = uC[0] - uW;
+        double res[kMaxOut][V];
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            const double uk = uC[k], ue = k + 1 < V ? uC[V - 1] : uE, uw = k ? uC[0] : uW;
+            const double dE = ue - uk, dN = uN[k] - uk, dS = uk - uS[k];
+            const double dP = DIM == 3 ? uP[k] - uk : 0.0;
+            double g = fma(uk, fma(uk, fma(uk, c.r3, c.r2), c.r1), c.r0);
+            double l1 = 0.0, l2 = 0.0, l3 = 0.0;             // second differences
+            if (ADELTA || NEEDF) {
+                l1 = dE - dW;
+                l2 = dN - dS;
+                if (DIM == 3) l3 = dP - dM[k];
+            }
+            if (ADELTA) {
+                if (aC) {
+                    double s = w.ih2[0] * l1;
+                    s = fma(w.ih2[1], l2, s);
+                    if (DIM == 3) s = fma(w.ih2[2], l3, s);
+                    g = fma(a0[k], s, g);
+                }
+            } else if (faces) {
+                g = fma(fE[k], dE, g);
+                g = fma(-(k ? fE[0] : fW), dW, g);
+                g = fma(fN[k], dN, g);
+                g = fma(-fS[k], dS, g);
+                if (DIM == 3) {
+                    g = fma(fP[k], dP, g);
+                    g = fma(-fM[k], dM[k], g);
+                }
+            }
+            double F = 0.0;
+            const bool a1 = w.adv & 1u, a2 = w.adv & 2u, a3 = DIM == 3 && (w.adv & 4u);
+            const bool b1 = NEEDF && (w.advF & 1u), b2 = NEEDF && (w.advF & 2u), b3 = NEEDF && DIM == 3 && (w.advF & 4u);
+            double m1 = 0.0, m2 = 0.0, m3 = 0.0;             // centred differences, where a term takes them
+            if (a1 || b1) m1 = ue - uw;
+            if (a2 || b2) m2 = uN[k] - uS[k];
+            if (a3 || b3) m3 = uP[k] - uM[k];
+            if (a1) g = fma(w.w2[0], m1, g);
+            if (a2) g = fma(w.w2[1], m2, g);
+            if (a3) g = fma(w.w2[2], m3, g);
+            if (NEEDF) {
+                F = fma(w.wa[0], l1, g);
+                F = fma(w.wa[1], l2, F);
+                if (DIM == 3) F = fma(w.wa[2], l3, F);
+                if (b1) F = fma(w.wb[0], m1, F);
+                if (b2) F = fma(w.wb[1], m2, F);
+                if (b3) F = fma(w.wb[2], m3, F);
+            }
+#pragma unroll
+            for (int j = 0; j < kMaxOut; ++j) {
+                if (j >= p.nout) continue;
+                const unsigned tm = w.terms[j];
+                double v = w.start[j] == 1 ? uk : 0.0;
+#pragma unroll
+                for (int e = 0; e < kMaxExtra; ++e)
+                    if (w.start[j] == 2 + e) v = x[e][k];
+                if (tm & (1u << kTu)) v = fma(c.cu[j], uk, v);
+                if (tm & (1u << kTg)) v = fma(c.cg[j], g, v);
+                if (NEEDF && (tm & (1u << kTF))) v = fma(c.cF[j], F, v);
+#pragma unroll
+                for (int e = 0; e < kMaxExtra; ++e)
+                    if (tm & (1u << (kTx + e))) v = fma(c.cx[j][e], x[e][k], v);
+                res[j][k] = v;
+            }
+            if (DIM == 3) dM[k] = dP;
+            dW = dE;
+        }
+#pragma unroll
+        for (int j = 0; j < kMaxOut; ++j)
+            if (j < p.nout) stv<V>(p.out[j] + idx, res[j]);
+        if (DIM == 3) {
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+                uM[k] = uC[k];
+                uC[k] = uP[k];
+                fM[k] = fP[k];
+            }
+            u += plane_u;
+            idx += plane_u;
+            if (faces) { f1 += plane_a; f2 += plane_a; f3 += plane_a; }
+            if (ADELTA && aC) aC += plane_a;
+        }
+    }
+}
+
+// w_mu at every node that has a next one along mu, from the nodal (a - abar).
+__global__ void f64_faces_kernel(const double* a, double* w, double half_ih2, long long next, long long total) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i + next < total; i += (long long)gridDim.x * blockDim.x)
+        w[i] = half_ih2 * (a[i] + a[i + next]);
+}
+
+int sm_count() {
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        return v > 0 ? v : 1;
+    }();
+    return sms;
+}
+
+template <int DIM, int V>
+cudaError_t launch_v(const StencilArgs<double>& p, const Coefs<double>& c, const Weights& w, bool needF, cudaStream_t s) {
+    const int gx = (p.n1 + kTX * V - 1) / (kTX * V), sms = sm_count();
+    int ty = kTY, zb = 1;
+    if (DIM == 3) {
+        // planes a block walks: about eight blocks per SM in all, and no fewer than 2 planes
+        // (each block loads the plane below its first one)
+        const int want = (8 * sms + gx * ((p.n2 + ty - 1) / ty) - 1) / (gx * ((p.n2 + ty - 1) / ty));
+        zb = p.n3 / (want < 1 ? 1 : want);
+        zb = zb < 2 ? 2 : zb > 32 ? 32 : zb;
+    }
+    const int gz = DIM == 3 ? (p.n3 + zb - 1) / zb : 1;
+    // small grids: a block on every SM (32^2 in four blocks of 8 rows: 14.8 us instead of 7.0)
+    while (ty > 1 && gx * ((p.n2 + ty - 1) / ty) * gz < 2 * sms) ty /= 2;
+    const dim3 grid(gx, (p.n2 + ty - 1) / ty, gz);
+    const int threads = kTX * ty;
+    if (p.adelta) {
+        if (needF) stencil_f64_kernel<DIM, V, true, true><<<grid, threads, 0, s>>>(p, c, w, zb);
+        else       stencil_f64_kernel<DIM, V, true, false><<<grid, threads, 0, s>>>(p, c, w, zb);
+    } else {
+        if (needF) stencil_f64_kernel<DIM, V, false, true><<<grid, threads, 0, s>>>(p, c, w, zb);
+        else       stencil_f64_kernel<DIM, V, false, false><<<grid, threads, 0, s>>>(p, c, w, zb);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_f64_faces(const double* a, double* w, double inv_h2, long long next, long long total, cudaStream_t s) {
+    const long long blocks = (total + 255) / 256;
+    f64_faces_kernel<<<unsigned(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(a, w, 0.5 * inv_h2, next, total);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_stencil(const StencilArgs<double>& p, cudaStream_t s) {
+    if (p.nout < 1 || p.nout > kMaxOut || p.nx < 0 || p.nx > kMaxExtra) return cudaErrorInvalidValue;
+    Coefs<double> c{};
+    Weights w{};
+    for (int m = 0; m < p.dim; ++m) {
+        w.w2[m] = p.bmb[m] * p.inv_2h[m];
+        w.wa[m] = p.abar * p.inv_h2[m];
+        w.wb[m] = p.beta[m] * p.inv_2h[m];
+        w.ih2[m] = p.inv_h2[m];
+        w.face[m] = p.face[m];
+    }
+    c.r0 = p.r[0]; c.r1 = p.r[1]; c.r2 = p.r[2]; c.r3 = p.r[3];
+    bool needF = false;
+    for (int j = 0; j < kMaxOut; ++j) {
+        c.cg[j] = p.cg[j];
+        c.cF[j] = p.cF[j];
+        state_coefs<double>(p.cu[j], p.cx[j], c.cu[j], c.cx[j]);
+        if (j >= p.nout) continue;
+        if (p.cF[j] != 0.0) needF = true;
+        w.start[j] = c.cu[j] == 1.0 ? 1 : 0;
+        for (int e = 0; e < p.nx; ++e)
+            if (!w.start[j] && c.cx[j][e] == 1.0) w.start[j] = 2 + e;
+        if (c.cu[j] != 0.0 && w.start[j] != 1) w.terms[j] |= 1u << kTu;
+        if (c.cg[j] != 0.0) w.terms[j] |= 1u << kTg;
+        if (c.cF[j] != 0.0) w.terms[j] |= 1u << kTF;
+        for (int e = 0; e < p.nx; ++e)
+            if (c.cx[j][e] != 0.0 && w.start[j] != 2 + e) w.terms[j] |= 1u << (kTx + e);
+    }
+    for (int m = 0; m < p.dim; ++m) {
+        if (w.w2[m] != 0.0) w.adv |= 1u << m;
+        if (w.wb[m] != 0.0) w.advF |= 1u << m;
+    }
+    // two nodes a thread where every row starts on 16 bytes and fills a warp
+    auto al = [](const void* q) { return reinterpret_cast<uintptr_t>(q) % 16 == 0; };
+    bool pairs = p.n1 % 2 == 0 && p.n1 >= 2 * kTX && al(p.u);
+    for (int e = 0; e < p.nx; ++e) pairs = pairs && al(p.X[e]);
+    for (int j = 0; j < p.nout; ++j) pairs = pairs && al(p.out[j]);
+    if (p.dim == 3) return pairs ? launch_v<3, 2>(p, c, w, needF, s) : launch_v<3, 1>(p, c, w, needF, s);
+    return pairs ? launch_v<2, 2>(p, c, w, needF, s) : launch_v<2, 1>(p, c, w, needF, s);
+}
+
+}  // namespace adr
