@@ -163,7 +163,7 @@ struct adr_ctx {
     void* d_psym = nullptr;                        // symbol of A
     void* d_pm[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // E(1/2), E(1), E(alpha), phi_1, phi_2
     void* d_pdif = nullptr;                        // a Lap u form: sum_mu a_mumu D_mu D_mu u
-    void* d_pcn = nullptr;                         // fused 2-D stages: the pointwise part of F, transformed
+    void* d_pcx = nullptr;                         // transform of the stage input along x1
     void* d_pz = nullptr;                          // fused 2-D stages: a Fourier-space array kept between stages
 
     // phi_k route; for the doubling route: X = tau A / 2^s, Taylor terms, level factors
@@ -615,7 +615,7 @@ adr::PeriodicArgs<T> periodic_args(const adr_ctx* c) {
     for (int i = 0; i < 4; ++i) P.r[i] = c->r[i];
     P.adelta = c->p.form == ADR_FORM_ADELTA;
     P.dif = static_cast<T*>(c->d_pdif);
-    P.CN = static_cast<adr::Cplx<T>*>(c->d_pcn);
+    P.Cx = static_cast<adr::Cplx<T>*>(c->d_pcx);
     return P;
 }
 
@@ -1798,6 +1798,9 @@ std::vector<double> wavenumbers(int n, double L) {
     return k;
 }
 
+// Points of a Fourier-space array: k_1 = 0..n_1/2, the other directions whole.
+size_t half_points(const adr_ctx* c) { return c->N / size_t(c->n[0]) * size_t(c->n[0] / 2 + 1); }
+
 adr_status create_periodic(const adr_params* p, void* cuda_stream, adr_ctx** out) {
     if (p->periodic != 1) return fail(nullptr, ADR_ERR_ARG, "periodic must be 0 or 1");
     if (p->batch != 0) return fail(nullptr, ADR_ERR_UNSUPPORTED, "periodic contexts are single grids");
@@ -1834,10 +1837,11 @@ adr_status create_periodic(const adr_params* p, void* cuda_stream, adr_ctx** out
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&c->d_err), sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, sizeof(int));
     for (int i = 0; i < 6 && e == cudaSuccess; ++i) e = cudaMalloc(&c->ws[i], N * c->esize);
-    for (int i = 0; i <= c->dim && e == cudaSuccess; ++i) e = cudaMalloc(&c->d_pc[i], 2 * N * c->esize);
+    const size_t half_bytes = 2 * half_points(c.get()) * c->esize;
+    for (int i = 0; i <= c->dim && e == cudaSuccess; ++i) e = cudaMalloc(&c->d_pc[i], half_bytes);
     if (e == cudaSuccess && p->form == ADR_FORM_ADELTA) e = cudaMalloc(&c->d_pdif, N * c->esize);
-    if (e == cudaSuccess && p->dim == 2) e = cudaMalloc(&c->d_pcn, 2 * N * c->esize);
-    if (e == cudaSuccess && p->dim == 2) e = cudaMalloc(&c->d_pz, 2 * N * c->esize);
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_pcx, half_bytes);
+    if (e == cudaSuccess && p->dim == 2) e = cudaMalloc(&c->d_pz, half_bytes);
     if (e == cudaSuccess) e = adr::periodic_prepare(c->fp64);
     if (e != cudaSuccess) {
         adr_destroy(c.release());
@@ -2123,15 +2127,17 @@ adr_status adr_set_coeffs_periodic(adr_ctx* c, const double* a_diag, const doubl
     // symbol s = sum_mu (-a^max_mu k_mu^2 + i beta_mu k_mu) and the multipliers of tau s
     std::vector<double> k[3];
     for (int m = 0; m < d; ++m) k[m] = wavenumbers(c->n[m], c->p.length);
-    std::vector<double> sym(2 * N), mult[5];
-    for (auto& v : mult) v.resize(2 * N);
+    const size_t NH = half_points(c);
+    std::vector<double> sym(2 * NH), mult[5];
+    for (auto& v : mult) v.resize(2 * NH);
     const double cexp[3] = {0.5, 1.0, adr::kLawsonAlpha};
-    for (size_t i = 0; i < N; ++i) {
+    for (size_t i = 0; i < NH; ++i) {
         size_t r = i;
         std::complex<double> sv = 0.0;
         for (int m = 0; m < d; ++m) {
-            const double km = k[m][r % size_t(c->n[m])];
-            r /= size_t(c->n[m]);
+            const size_t nm = m == 0 ? size_t(c->n[0] / 2 + 1) : size_t(c->n[m]);
+            const double km = k[m][r % nm];
+            r /= nm;
             sv += std::complex<double>(-amax[m] * km * km, c->beta[m] * km);
         }
         sym[2 * i] = sv.real();
@@ -2463,7 +2469,7 @@ void adr_destroy(adr_ctx* c) {
     free_dev(c->d_psym);
     for (auto& q : c->d_pm) free_dev(q);
     free_dev(c->d_pdif);
-    free_dev(c->d_pcn);
+    free_dev(c->d_pcx);
     free_dev(c->d_pz);
     for (auto& row : c->d_img) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }  // 5 kinds
     for (auto& row : c->d_fsc) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }

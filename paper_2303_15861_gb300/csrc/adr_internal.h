@@ -416,7 +416,9 @@ struct PeriodicArgs {
     int dim = 2;
     int n[3] = {1, 1, 1};
     long long N = 0;
+    // Fourier-space arrays hold k_1 = 0..n_1/2 of real fields (periodic.cu): (n_1/2 + 1) n_2 (n_3) elements
     Cplx<T>* Cu = nullptr;                 // transform of the stage input
+    Cplx<T>* Cx = nullptr;                 // its transform along x1
     Cplx<T>* C[3] = {nullptr, nullptr, nullptr};   // work: derivatives, fluxes, outputs (d of them)
     const Cplx<T>* tw[3] = {nullptr, nullptr, nullptr};   // e^{-2 pi i j / n_mu}, j < n_mu / 2
     const T* k[3] = {nullptr, nullptr, nullptr};          // wavenumbers (Nyquist 0)
@@ -426,7 +428,6 @@ struct PeriodicArgs {
     double r[4] = {0, 0, 0, 0};
     bool adelta = false;                   // a Lap u form: sum_mu a_mumu D_mu D_mu u + D_mu (b_mu u)
     T* dif = nullptr;                      // adelta: sum_mu a_mumu D_mu D_mu u at the nodes (work)
-    Cplx<T>* CN = nullptr;                 // fused stages: the pointwise part of F, transformed (work)
 };
 
 // One fused stage of a 2-D periodic context, computed in Fourier space from the transform of x
