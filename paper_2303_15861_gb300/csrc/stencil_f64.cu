@@ -9,10 +9,13 @@
 // registers), and terms whose coefficient is zero are left out by branches that every thread takes alike.
 // Per node and direction: d+ (shared), two FMAs with the face weights; M = u+ - u- and one FMA
 // where b - beta is not zero; for F, L = d+ - d- and one FMA with abar / h^2, and one FMA of M with beta / (2h).
-// u + tau/2 g in 3-D: 16 FP64 instructions a node instead of about 75; F and g: 27 instead of 85.
-// Time of a launch, per-node kernel -> this one (us): 256^3, one output 2139 -> 788, two outputs and one or two
-// stage inputs 2460 -> 975; 128^3, F and g 379 -> 197, g - G0 283 -> 104; 60^3 Neumann, a Lap u form 39 -> 22; 32^2 12.6 -> 7.0.
+// u + tau/2 g in 3-D: 15 FP64 instructions a node instead of about 75; F and g: 27 instead of 85.
+// Time of a launch, per-node kernel -> this one (us): 256^3 2139 -> 504 (one output), 2460 -> 607 and 692 (two outputs, one and two
+// stage inputs); 128^3 F and g 379 -> 142, g - G0 283 -> 66; 60^3 Neumann, a Lap u form 39 -> 17; 32^2 12.6 -> 7.3. The FP64 pipe
+// is then 85% busy.
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "adr_internal.h"
 #include "stencil_core.cuh"
@@ -29,8 +32,8 @@ struct Weights {
     double ih2[3];
     const double* face[3];               // face weights, laid out as StencilArgs::a (NULL: a = abar everywhere)
     // which terms there are: tested as integers, since a comparison of doubles costs an FP64 instruction
-    unsigned adv, advF;                  // bit mu: w2, wb not zero
-    int start[kMaxOut];                  // a term of coefficient one: 1 u, 2 + e X_e; 0 none
+    bool adv;                            // a w2, or a wb that F takes, is not zero
+    int start[kMaxOut];                  // a term of coefficient one: 1 u, 2 g, 3 F, 4 + e X_e; 0 none
     unsigned terms[kMaxOut];             // the other terms that are not zero: bits kTu, kTg, kTF, kTx + e
 };
 constexpr unsigned kTu = 0, kTg = 1, kTF = 2, kTx = 3;
@@ -53,7 +56,10 @@ __device__ __forceinline__ void stv(double* p, const double (&v)[V]) {
 
 // A thread owns V consecutive x1 nodes of one row and walks zb planes of x3; u of the planes z - 1 and z
 // and the face weights below plane z stay in registers, the neighbours along x1 and x2 come from L1.
-template <int DIM, int V, bool ADELTA, bool NEEDF>
+// ADV: any first-derivative term; NX: stage inputs; UT: whether an output takes a multiple of u. An instruction under a false predicate still takes its turn on the
+// FP64 pipe, and the compiler turns short branches into predicates, so what decides about few instructions is a
+// template argument.
+template <int DIM, int V, bool ADELTA, bool NEEDF, bool ADV, int NX, bool UT>
 __global__ void __launch_bounds__(kTX * kTY) stencil_f64_kernel(StencilArgs<double> p, Coefs<double> c, Weights w, int zb) {
     const int n1 = p.n1, n2 = p.n2, n3 = DIM == 3 ? p.n3 : 1;
     const int i1 = (int(blockIdx.x) * kTX + int(threadIdx.x % kTX)) * V;
@@ -81,7 +87,7 @@ __global__ void __launch_bounds__(kTX * kTY) stencil_f64_kernel(StencilArgs<doub
     }
     long long idx = (long long)i2 * n1 + i1 + z0 * plane_u;
     for (int z = z0; z < z1; ++z) {
-        double uP[V], uS[V], uN[V], fS[V], fN[V], fE[V], fP[V], a0[V], x[kMaxExtra][V];
+        double uP[V], uS[V], uN[V], fS[V], fN[V], fE[V], fP[V], a0[V], x[NX > 0 ? NX : 1][V];
         double uW = 0.0, uE = 0.0, fW = 0.0;
 #pragma unroll
         for (int k = 0; k < V; ++k) uP[k] = uS[k] = uN[k] = 0.0;
@@ -110,76 +116,83 @@ __global__ void __launch_bounds__(kTX * kTY) stencil_f64_kernel(StencilArgs<doub
         }
         if (ADELTA && aC) ldv<V>(aC, a0);
 #pragma unroll
-        for (int e = 0; e < kMaxExtra; ++e)
-            if (e < p.nx) ldv<V>(p.X[e] + idx, x[e]);
+        for (int e = 0; e < NX; ++e) ldv<V>(p.X[e] + idx, x[e]);
 
+        double g[V], au[V], F[V];                            // g, A u, F = g + A u
         double dW = uC[0] - uW;
-        double res[kMaxOut][V];
 #pragma unroll
         for (int k = 0; k < V; ++k) {
-            const double uk = uC[k], ue = k + 1 < V ? uC[V - 1] : uE, uw = k ? uC[0] : uW;
+            const double uk = uC[k], ue = k + 1 < V ? uC[V - 1] : uE;
             const double dE = ue - uk, dN = uN[k] - uk, dS = uk - uS[k];
             const double dP = DIM == 3 ? uP[k] - uk : 0.0;
-            double g = fma(uk, fma(uk, fma(uk, c.r3, c.r2), c.r1), c.r0);
+            double r = fma(uk, fma(uk, fma(uk, c.r3, c.r2), c.r1), c.r0);
             double l1 = 0.0, l2 = 0.0, l3 = 0.0;             // second differences
             if (ADELTA || NEEDF) {
                 l1 = dE - dW;
                 l2 = dN - dS;
                 if (DIM == 3) l3 = dP - dM[k];
             }
-            if (ADELTA) {
-                if (aC) {
-                    double s = w.ih2[0] * l1;
-                    s = fma(w.ih2[1], l2, s);
-                    if (DIM == 3) s = fma(w.ih2[2], l3, s);
-                    g = fma(a0[k], s, g);
-                }
-            } else if (faces) {
-                g = fma(fE[k], dE, g);
-                g = fma(-(k ? fE[0] : fW), dW, g);
-                g = fma(fN[k], dN, g);
-                g = fma(-fS[k], dS, g);
-                if (DIM == 3) {
-                    g = fma(fP[k], dP, g);
-                    g = fma(-fM[k], dM[k], g);
-                }
-            }
-            double F = 0.0;
-            const bool a1 = w.adv & 1u, a2 = w.adv & 2u, a3 = DIM == 3 && (w.adv & 4u);
-            const bool b1 = NEEDF && (w.advF & 1u), b2 = NEEDF && (w.advF & 2u), b3 = NEEDF && DIM == 3 && (w.advF & 4u);
-            double m1 = 0.0, m2 = 0.0, m3 = 0.0;             // centred differences, where a term takes them
-            if (a1 || b1) m1 = ue - uw;
-            if (a2 || b2) m2 = uN[k] - uS[k];
-            if (a3 || b3) m3 = uP[k] - uM[k];
-            if (a1) g = fma(w.w2[0], m1, g);
-            if (a2) g = fma(w.w2[1], m2, g);
-            if (a3) g = fma(w.w2[2], m3, g);
             if (NEEDF) {
-                F = fma(w.wa[0], l1, g);
-                F = fma(w.wa[1], l2, F);
-                if (DIM == 3) F = fma(w.wa[2], l3, F);
-                if (b1) F = fma(w.wb[0], m1, F);
-                if (b2) F = fma(w.wb[1], m2, F);
-                if (b3) F = fma(w.wb[2], m3, F);
+                au[k] = fma(w.wa[1], l2, w.wa[0] * l1);
+                if (DIM == 3) au[k] = fma(w.wa[2], l3, au[k]);
             }
+            if (!ADELTA && faces) {
+                r = fma(fE[k], dE, r);
+                r = fma(-(k ? fE[0] : fW), dW, r);
+                r = fma(fN[k], dN, r);
+                r = fma(-fS[k], dS, r);
+                if (DIM == 3) {
+                    r = fma(fP[k], dP, r);
+                    r = fma(-fM[k], dM[k], r);
+                }
+            }
+            if (ADELTA && aC) {
+                double s = w.ih2[0] * l1;
+                s = fma(w.ih2[1], l2, s);
+                if (DIM == 3) s = fma(w.ih2[2], l3, s);
+                r = fma(a0[k], s, r);
+            }
+            g[k] = r;
+            if (DIM == 3) dM[k] = dP;
+            dW = dE;
+        }
+        // centred differences, where a term takes them
 #pragma unroll
-            for (int j = 0; j < kMaxOut; ++j) {
-                if (j >= p.nout) continue;
-                const unsigned tm = w.terms[j];
-                double v = w.start[j] == 1 ? uk : 0.0;
+        for (int m = 0; m < (ADV ? DIM : 0); ++m) {
+            double md[V];
 #pragma unroll
-                for (int e = 0; e < kMaxExtra; ++e)
-                    if (w.start[j] == 2 + e) v = x[e][k];
-                if (tm & (1u << kTu)) v = fma(c.cu[j], uk, v);
-                if (tm & (1u << kTg)) v = fma(c.cg[j], g, v);
-                if (NEEDF && (tm & (1u << kTF))) v = fma(c.cF[j], F, v);
+            for (int k = 0; k < V; ++k)
+                md[k] = m == 0 ? (k + 1 < V ? uC[V - 1] : uE) - (k ? uC[0] : uW) : m == 1 ? uN[k] - uS[k] : uP[k] - uM[k];
 #pragma unroll
-                for (int e = 0; e < kMaxExtra; ++e)
+            for (int k = 0; k < V; ++k) {
+                g[k] = fma(w.w2[m], md[k], g[k]);
+                if (NEEDF) au[k] = fma(w.wb[m], md[k], au[k]);
+            }
+        }
+        if (NEEDF) {
+#pragma unroll
+            for (int k = 0; k < V; ++k) F[k] = g[k] + au[k];
+        }
+        double res[kMaxOut][V];
+#pragma unroll
+        for (int j = 0; j < kMaxOut; ++j) {
+            if (j >= p.nout) continue;
+            const unsigned tm = w.terms[j];
+            const int st = w.start[j];
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+                double v = st == 1 ? uC[k] : st == 2 ? g[k] : NEEDF && st == 3 ? F[k] : 0.0;
+#pragma unroll
+                for (int e = 0; e < NX; ++e)
+                    if (st == 4 + e) v = x[e][k];
+                if (UT && (tm & (1u << kTu))) v = fma(c.cu[j], uC[k], v);
+                if (tm & (1u << kTg)) v = fma(c.cg[j], g[k], v);
+                if (NEEDF && (tm & (1u << kTF))) v = fma(c.cF[j], F[k], v);
+#pragma unroll
+                for (int e = 0; e < NX; ++e)
                     if (tm & (1u << (kTx + e))) v = fma(c.cx[j][e], x[e][k], v);
                 res[j][k] = v;
             }
-            if (DIM == 3) dM[k] = dP;
-            dW = dE;
         }
 #pragma unroll
         for (int j = 0; j < kMaxOut; ++j)
@@ -231,13 +244,29 @@ cudaError_t launch_v(const StencilArgs<double>& p, const Coefs<double>& c, const
     while (ty > 1 && gx * ((p.n2 + ty - 1) / ty) * gz < 2 * sms) ty /= 2;
     const dim3 grid(gx, (p.n2 + ty - 1) / ty, gz);
     const int threads = kTX * ty;
-    if (p.adelta) {
-        if (needF) stencil_f64_kernel<DIM, V, true, true><<<grid, threads, 0, s>>>(p, c, w, zb);
-        else       stencil_f64_kernel<DIM, V, true, false><<<grid, threads, 0, s>>>(p, c, w, zb);
-    } else {
-        if (needF) stencil_f64_kernel<DIM, V, false, true><<<grid, threads, 0, s>>>(p, c, w, zb);
-        else       stencil_f64_kernel<DIM, V, false, false><<<grid, threads, 0, s>>>(p, c, w, zb);
-    }
+    auto go = [&](auto adelta, auto f, auto adv) {
+        constexpr bool AD = decltype(adelta)::value, NF = decltype(f)::value, AV = decltype(adv)::value;
+        // odd rows and 2-D grids take the form that has every term
+        if constexpr (DIM == 2 || V == 1) {
+            stencil_f64_kernel<DIM, V, AD, NF, AV, kMaxExtra, true><<<grid, threads, 0, s>>>(p, c, w, zb);
+        } else {
+            bool ut = false;
+            for (int j = 0; j < p.nout; ++j) ut = ut || (w.terms[j] & (1u << kTu));
+            switch (p.nx * 2 + (ut ? 1 : 0)) {
+            case 0: stencil_f64_kernel<DIM, V, AD, NF, AV, 0, false><<<grid, threads, 0, s>>>(p, c, w, zb); break;
+            case 1: stencil_f64_kernel<DIM, V, AD, NF, AV, 0, true><<<grid, threads, 0, s>>>(p, c, w, zb); break;
+            case 2: stencil_f64_kernel<DIM, V, AD, NF, AV, 1, false><<<grid, threads, 0, s>>>(p, c, w, zb); break;
+            case 3: stencil_f64_kernel<DIM, V, AD, NF, AV, 1, true><<<grid, threads, 0, s>>>(p, c, w, zb); break;
+            case 4: stencil_f64_kernel<DIM, V, AD, NF, AV, 2, false><<<grid, threads, 0, s>>>(p, c, w, zb); break;
+            default: stencil_f64_kernel<DIM, V, AD, NF, AV, kMaxExtra, true><<<grid, threads, 0, s>>>(p, c, w, zb); break;
+            }
+        }
+    };
+    using Yes = std::integral_constant<bool, true>;
+    using No = std::integral_constant<bool, false>;
+    auto with_adv = [&](auto adelta, auto f) { w.adv ? go(adelta, f, Yes{}) : go(adelta, f, No{}); };
+    if (p.adelta) needF ? with_adv(Yes{}, Yes{}) : with_adv(Yes{}, No{});
+    else          needF ? with_adv(No{}, Yes{}) : with_adv(No{}, No{});
     return cudaGetLastError();
 }
 
@@ -268,26 +297,28 @@ cudaError_t launch_stencil(const StencilArgs<double>& p, cudaStream_t s) {
         state_coefs<double>(p.cu[j], p.cx[j], c.cu[j], c.cx[j]);
         if (j >= p.nout) continue;
         if (p.cF[j] != 0.0) needF = true;
-        w.start[j] = c.cu[j] == 1.0 ? 1 : 0;
+        w.start[j] = c.cu[j] == 1.0 ? 1 : c.cg[j] == 1.0 ? 2 : c.cF[j] == 1.0 ? 3 : 0;
         for (int e = 0; e < p.nx; ++e)
-            if (!w.start[j] && c.cx[j][e] == 1.0) w.start[j] = 2 + e;
+            if (!w.start[j] && c.cx[j][e] == 1.0) w.start[j] = 4 + e;
         if (c.cu[j] != 0.0 && w.start[j] != 1) w.terms[j] |= 1u << kTu;
-        if (c.cg[j] != 0.0) w.terms[j] |= 1u << kTg;
-        if (c.cF[j] != 0.0) w.terms[j] |= 1u << kTF;
+        if (c.cg[j] != 0.0 && w.start[j] != 2) w.terms[j] |= 1u << kTg;
+        if (c.cF[j] != 0.0 && w.start[j] != 3) w.terms[j] |= 1u << kTF;
         for (int e = 0; e < p.nx; ++e)
-            if (c.cx[j][e] != 0.0 && w.start[j] != 2 + e) w.terms[j] |= 1u << (kTx + e);
+            if (c.cx[j][e] != 0.0 && w.start[j] != 4 + e) w.terms[j] |= 1u << (kTx + e);
     }
     for (int m = 0; m < p.dim; ++m) {
-        if (w.w2[m] != 0.0) w.adv |= 1u << m;
-        if (w.wb[m] != 0.0) w.advF |= 1u << m;
+        if (w.w2[m] != 0.0 || (needF && w.wb[m] != 0.0)) w.adv = true;
     }
+    // inputs that are not there (forms with more of them than p.nx) are read as u, with no term
+    StencilArgs<double> q = p;
+    for (int e = p.nx; e < kMaxExtra; ++e) q.X[e] = p.u;
     // two nodes a thread where every row starts on 16 bytes and fills a warp
     auto al = [](const void* q) { return reinterpret_cast<uintptr_t>(q) % 16 == 0; };
     bool pairs = p.n1 % 2 == 0 && p.n1 >= 2 * kTX && al(p.u);
     for (int e = 0; e < p.nx; ++e) pairs = pairs && al(p.X[e]);
     for (int j = 0; j < p.nout; ++j) pairs = pairs && al(p.out[j]);
-    if (p.dim == 3) return pairs ? launch_v<3, 2>(p, c, w, needF, s) : launch_v<3, 1>(p, c, w, needF, s);
-    return pairs ? launch_v<2, 2>(p, c, w, needF, s) : launch_v<2, 1>(p, c, w, needF, s);
+    if (p.dim == 3) return pairs ? launch_v<3, 2>(q, c, w, needF, s) : launch_v<3, 1>(q, c, w, needF, s);
+    return pairs ? launch_v<2, 2>(q, c, w, needF, s) : launch_v<2, 1>(q, c, w, needF, s);
 }
 
 }  // namespace adr
