@@ -71,7 +71,7 @@ def parse():
 # source the bench reports null until the kernel is captured again.
 _TRAFFIC_CAPTURE = {"n": 256, "bytes_per_launch": 86.1e6,
                     "source_sha256": "78dffd3a19003a8c961d823307beb2ea5ce7aebd44e43612de628f34843851e9"}
-_TRAFFIC_SOURCES = ("paper_2303_15861_gb300/csrc/contract_tma.cu", "paper_2303_15861_gb300/csrc/tc_common.cuh",
+_TRAFFIC_SOURCES = ("paper_2303_15861_gb300/csrc/contract_tc.cu", "paper_2303_15861_gb300/csrc/tc_common.cuh",
                     "paper_2303_15861_gb300/csrc/host_setup.cpp")
 
 

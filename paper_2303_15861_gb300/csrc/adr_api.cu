@@ -51,7 +51,7 @@ struct Op {
 
 thread_local std::string g_create_error;
 
-// Factor kinds: 0 E(0.5), 1 E(1), 2 V, 3 V^-1, 4 E(0.5) precise, 5 E(alpha); from kLevel0 the
+// Factor kinds: 0 E(0.5), 1 E(1), 2 V, 3 V^-1, 5 E(alpha); from kLevel0 the
 // factors e^{2^i tau A_mu / 2^s} of the phi doubling route, level i = kind - kLevel0.
 constexpr int kLevel0 = 8;
 constexpr int kMaxLevels = 40;
@@ -137,9 +137,8 @@ struct adr_ctx {
     bool tc = false;
     uint8_t* d_img[kFactorKinds][3] = {{nullptr}};    // sliced image per factor kind and direction
     float* d_fsc[kFactorKinds][3] = {{nullptr}};
-    uint8_t* d_img2[kFactorKinds][3] = {{nullptr}};   // the same for the TMA-fed kernel (K chunks of 32)
-    float* d_fsc2[kFactorKinds][3] = {{nullptr}};
     float* d_zt[3] = {nullptr};            // tau * lambda_mu[j] (FP32)
+    float* d_phi32[3] = {nullptr, nullptr, nullptr};   // phi_k(tau (l1 + l2 + l3)) at the nodes, k = 0, 1, 2
     unsigned* d_slots = nullptr;           // max-abs slots of the arrays a step produces
     int* d_err = nullptr;                  // device error word (bounded waits)
 
@@ -222,12 +221,9 @@ cudaError_t upload(adr_ctx* c, void** dst, const std::vector<double>& src) {
     return cudaMemcpy(*dst, tmp.data(), bytes, cudaMemcpyHostToDevice);
 }
 
-// Slice an FP64 factor for the tensor-core kernel and upload image + row scales. Mode 1
-// uses the factor as the A operand (128-row tiles), modes >= 2 as the B operand.
+// Slice an FP64 factor for the tensor-core kernel and upload image + row scales.
 cudaError_t upload_tc(adr_ctx* c, int kind, int m, const std::vector<double>& M) {
-    const bool precise = (kind == 4);   // FK_EXP_HALF_PRECISE
-    // register-fed kernel: every image in the four-slice layout of its precise variant
-    const adr::TcFactor f = adr::make_tc_factor(M, c->n[m], adr::tc_out_rows(m >= 1, true), true);
+    const adr::TcFactor f = adr::make_tc_factor(M, c->n[m]);
     cudaError_t e = cudaSuccess;
     if (!c->d_img[kind][m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_img[kind][m]), f.img.size());
     if (e == cudaSuccess && !c->d_fsc[kind][m])
@@ -235,15 +231,6 @@ cudaError_t upload_tc(adr_ctx* c, int kind, int m, const std::vector<double>& M)
     if (e == cudaSuccess) e = cudaMemcpy(c->d_img[kind][m], f.img.data(), f.img.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(c->d_fsc[kind][m], f.fscale.data(), f.fscale.size() * sizeof(float), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return e;
-    // TMA-fed kernel: 128-row output tiles, K chunks of 32
-    const adr::TcFactor f2 = adr::make_tc_factor(M, c->n[m], 128, precise, 32);
-    if (!c->d_img2[kind][m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_img2[kind][m]), f2.img.size());
-    if (e == cudaSuccess && !c->d_fsc2[kind][m])
-        e = cudaMalloc(reinterpret_cast<void**>(&c->d_fsc2[kind][m]), f2.fscale.size() * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemcpy(c->d_img2[kind][m], f2.img.data(), f2.img.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(c->d_fsc2[kind][m], f2.fscale.data(), f2.fscale.size() * sizeof(float), cudaMemcpyHostToDevice);
     return e;
 }
 
@@ -367,7 +354,7 @@ ContractArgs<T> mode_args(const adr_ctx* c, int mu, const T* M, const T* X, T* Y
     return a;
 }
 
-enum FactorKind { FK_EXP_HALF = 0, FK_EXP_ONE = 1, FK_V = 2, FK_VINV = 3, FK_EXP_HALF_PRECISE = 4, FK_EXP_ALPHA = 5 };
+enum FactorKind { FK_EXP_HALF = 0, FK_EXP_ONE = 1, FK_V = 2, FK_VINV = 3, FK_EXP_ALPHA = 5 };
 static_assert(int(FK_EXP_HALF) == adr::BR_EXP_HALF && int(FK_EXP_ONE) == adr::BR_EXP_ONE && int(FK_V) == adr::BR_V &&
                   int(FK_VINV) == adr::BR_VINV,
               "factor kinds and batch roles share their numbering");
@@ -538,62 +525,30 @@ void push_mode(Sched& S, int mu, int kind, const T* x, T* y, int epi = adr::EPI_
         return;
     }
     adr::TcArgs a;
-    const int n = c->n[mu - 1];
-    long long Q = 1, P = 1;
-    for (int nu = 1; nu < mu; ++nu) Q *= c->n[nu - 1];
-    for (int nu = mu + 1; nu <= c->dim; ++nu) P *= c->n[nu - 1];
+    a.n = c->n[mu - 1];
+    for (int nu = 1; nu < mu; ++nu) a.Q *= unsigned(c->n[nu - 1]);
+    a.npos = unsigned(c->N / size_t(a.n));
     a.X = reinterpret_cast<const float*>(x);
     a.Xlo = reinterpret_cast<const float*>(xlo);
     a.Y = reinterpret_cast<float*>(y);
-    a.precise = (kind == FK_EXP_HALF_PRECISE);
+    a.Ylo = reinterpret_cast<float*>(ylo);
     a.fimg = c->d_img[kind][mu - 1];
     a.fscale = c->d_fsc[kind][mu - 1];
-    a.n = n;
-    a.Q = Q;
-    a.state_is_a = (mu >= 2);
-    a.vec4 = (mu == 1) && (n % 4 == 0) && (reinterpret_cast<uintptr_t>(x) % 16 == 0);
-    a.npos = (mu >= 2) ? P * Q : P;
-    a.nK = (n + 63) / 64;
-    if (epi == adr::EPI_PHI) {
-        // the phi scaling is fused into a mode >= 2 pass: decode (q, p) into the other directions
-        a.zmu = c->d_zt[mu - 1];
-        a.zq_a = c->d_zt[0];
-        a.na = c->n[0];
-        a.zq_b = (mu == 3) ? c->d_zt[1] : nullptr;
-        a.zp = (mu == 2 && c->dim == 3) ? c->d_zt[2] : nullptr;
-    }
     a.epi = epi;
-    a.Ylo = reinterpret_cast<float*>(ylo);
     a.base = reinterpret_cast<const float*>(base);
     a.alpha = float(alpha);
-    a.phik = phik;
+    if (epi == adr::EPI_PHI) {
+        a.phi = c->d_phi32[phik];
+        a.phik = phik;
+        for (int m = 0; m < c->dim; ++m) a.zt[m] = c->d_zt[m];
+        a.n1 = c->n[0];
+        a.n2 = c->n[1];
+    }
     a.amax_in = S.consume(x);
     a.amax_out = S.produce(y);
     a.err = c->d_err;
-    const int tc_kind = a.precise ? OP_CONTRACT_TC_PRECISE : OP_CONTRACT_TC;
-    if (adr::tma_supported(n, Q, x, xlo)) {
-        // TMA-fed kernel: position tiles of 128 consecutive q of one p, 128-row output tiles
-        adr::TmaArgs t;
-        static_cast<adr::TcArgs&>(t) = a;
-        t.fimg = c->d_img2[kind][mu - 1];
-        t.fscale = c->d_fsc2[kind][mu - 1];
-        t.nK = (n + 31) / 32;
-        t.nOut = (n + 127) / 128;
-        t.nqt = (mu >= 2) ? (Q + 127) / 128 : 1;
-        t.ntiles = ((mu >= 2) ? P * t.nqt : (P + 127) / 128) * t.nOut;
-        const long long PP = P;
-        S.ops.push_back({[t, PP](cudaStream_t s) { return adr::launch_contract_tma(t, PP, s); }, tc_kind});
-        return;
-    }
-    // Register-fed kernel (shapes the TMA rules exclude): every pass in its precise variant, the
-    // ten-product split into exact accumulators (its images are built in that layout); the low
-    // part stays optional.
-    adr::TcArgs r = a;
-    r.precise = true;
-    const int orows = adr::tc_out_rows(r.state_is_a, true), prows = adr::tc_pos_rows(r.state_is_a, true);
-    r.nOut = (n + orows - 1) / orows;
-    r.ntiles = ((r.npos + prows - 1) / prows) * r.nOut;
-    S.ops.push_back({[r](cudaStream_t s) { return adr::launch_contract_tc(r, s); }, tc_kind});
+    S.ops.push_back({[a](cudaStream_t s) { return adr::launch_contract_tc(a, s); },
+                     epi == adr::EPI_STORE2 ? OP_CONTRACT_TC_PRECISE : OP_CONTRACT_TC});
 }
 
 // The device arrays of a periodic context as the Fourier kernels take them.
@@ -707,7 +662,7 @@ void push_exp_precise(Sched& S, const T* x, T* y, T* ylo) {
         const bool last = mu == c->dim;
         T* out = last ? y : hi[(mu - 1) % 2];
         T* outlo = last ? ylo : lo[(mu - 1) % 2];
-        push_mode<T>(S, mu, FK_EXP_HALF_PRECISE, in, out, adr::EPI_STORE2, nullptr, 0.0, 0, outlo, inlo);
+        push_mode<T>(S, mu, FK_EXP_HALF, in, out, adr::EPI_STORE2, nullptr, 0.0, 0, outlo, inlo);
         in = out;
         inlo = outlo;
     }
@@ -2030,7 +1985,6 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
             if (e != cudaSuccess) return cuda_fail(c, e, "upload E");
             if (c->tc) {
                 e = upload_tc(c, ci == 2 ? FK_EXP_ALPHA : ci, m, *E);
-                if (e == cudaSuccess && ci == 0) e = upload_tc(c, FK_EXP_HALF_PRECISE, m, *E);
                 if (e != cudaSuccess) return cuda_fail(c, e, "upload sliced E");
             }
         }
@@ -2082,9 +2036,14 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
                     e = adr::launch_f64_phi(c->d_phi64[k], k, c->p.tau, c->d_lam, c->n[0], c->n[1], c->N, nullptr);
                 if (e != cudaSuccess) return cuda_fail(c, e, "phi tables");
             }
+            for (int k = 1; k <= 2 && c->tc; ++k) {
+                if (!c->d_phi32[k]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_phi32[k]), c->N * sizeof(float));
+                if (e == cudaSuccess) e = adr::launch_phi_table(c->d_phi32[k], k, c->d_zt, c->n[0], c->n[1], c->N, nullptr);
+                if (e != cudaSuccess) return cuda_fail(c, e, "phi tables");
+            }
         }
     }
-    if (c->f64tc) {                        // the kernels above ran on the legacy stream
+    if (c->f64tc || c->tc) {               // the kernels above ran on the legacy stream
         e = cudaStreamSynchronize(nullptr);
         if (e != cudaSuccess) return cuda_fail(c, e, "cut factors");
     }
@@ -2394,7 +2353,7 @@ adr_status adr_tc_factor_slices(const adr_ctx* c, int* slices) {
     if (!c || !slices) return ADR_ERR_ARG;
     *slices = 0;
     if (!c->tc || c->bs || c->periodic || !c->coeffs_set) return ADR_OK;
-    *slices = 4;   // every standard image of the TMA-fed kernel (contract_tma.cu)
+    *slices = 4;   // every factor image (contract_tc.cu)
     return ADR_OK;
 }
 
@@ -2473,8 +2432,7 @@ void adr_destroy(adr_ctx* c) {
     free_dev(c->d_pz);
     for (auto& row : c->d_img) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }  // 5 kinds
     for (auto& row : c->d_fsc) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
-    for (auto& row : c->d_img2) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
-    for (auto& row : c->d_fsc2) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
+    for (auto& p : c->d_phi32) { void* q = p; free_dev(q); p = nullptr; }
     for (auto& row : c->d_img64) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
     for (auto& row : c->d_rows64) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
     for (auto& p : c->d_phi64) { void* q = p; free_dev(q); p = nullptr; }

@@ -1,7 +1,6 @@
 // Internal declarations shared by the translation units of libadr.
 #pragma once
 
-#include <cuda.h>
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <string>
@@ -133,50 +132,35 @@ struct ContractArgs {
     int n1 = 1, n2 = 1;
 };
 
-// K2 (tensor cores, mixed precision): see contract_tc.cu for the exact-slice split.
-// The factor M (n x n) is passed as a pre-sliced, pre-swizzled image: for output tile
-// o (128 rows) and K chunk c (64 columns), four 16 KB tiles F0, F1, 2^-8 F1, 2^-8 F2.
+// K2 (tensor cores, mixed precision; contract_tc.cu): the state seen as [P][n][Q] (mode 1: Q = 1), contracted
+// along n with a factor M (n x n) passed as a pre-sliced, pre-swizzled image.
 struct TcArgs {
     const float* X = nullptr;
-    const float* Xlo = nullptr;      // precise: optional low part of a double-float input
+    const float* Xlo = nullptr;      // optional low part of a double-float input (EPI_STORE2)
     float* Y = nullptr;
     float* Ylo = nullptr;            // EPI_STORE2: low part of the double-float result
-    const uint8_t* fimg = nullptr;   // factor image (tc_factor_image_bytes(n) bytes)
-    const float* fscale = nullptr;   // per output row i: 2^(e_i - 7)
+    const uint8_t* fimg = nullptr;   // factor image (make_tc_factor)
+    const float* fscale = nullptr;   // per output row i: 2^(e_i - 7), padded to whole tiles
     int n = 0;                       // extent of the contracted direction
-    long long Q = 1;                 // product of the faster extents (1 for mode 1)
-    long long npos = 0;              // positions P*Q (mode >= 2) or fibres P (mode 1)
-    int nK = 0, nOut = 0;            // K chunks of 64, output tiles of 128
-    long long ntiles = 0;
-    bool state_is_a = true;          // modes >= 2: true; mode 1: false
-    bool precise = false;            // four slices per operand, ten MMAs, double-float result
-    bool vec4 = false;               // mode 1: X rows 16-byte aligned (n % 4 == 0)
+    unsigned Q = 1, npos = 0;        // product of the faster extents; positions P Q
     int epi = EPI_STORE;
-    const float* base = nullptr;
+    const float* base = nullptr;     // EPI_AXPY (may be Y)
     float alpha = 0.f;
+    const float* phi = nullptr;      // EPI_PHI: table over the nodes, or NULL with the fields below
     int phik = 1;
-    // EPI_PHI (modes >= 2): z = zmu[i] + zq_a[q % na] + zq_b[q / na] + zp[p], with
-    // tau*lambda tables (FP32) of the contracted direction and of the others
-    const float* zmu = nullptr;
-    const float* zq_a = nullptr;
-    const float* zq_b = nullptr;
-    const float* zp = nullptr;
-    int na = 1;
+    const float* zt[3] = {nullptr, nullptr, nullptr};   // tau * eigenvalues per direction
+    int n1 = 1, n2 = 1;
     const unsigned* amax_in = nullptr;                  // max|X| (float bits)
     unsigned* amax_out = nullptr;                       // max|Y| accumulator (float bits)
     int* err = nullptr;                                 // bounded-wait timeout flags
+    // set by the launcher
+    int nK = 0, nOut = 0, ntiles = 0;
+    bool vec4 = false;               // mode 1: rows of X (and Xlo) 16-byte aligned
+    bool vec8 = false;               // modes >= 2: eight columns are 32 aligned bytes
 };
-
-// The TMA-fed form (contract_tma.cu): the same arguments plus tensor maps of the FP32 state
-// (and of its low part), encoded at launch; position tiles are (p, 128 consecutive q).
-struct TmaArgs : TcArgs {
-    alignas(64) CUtensorMap map_x;
-    alignas(64) CUtensorMap map_xlo;
-    long long nqt = 1;          // position tiles per p: ceil(Q / 128) (modes >= 2)
-    bool has_lo = false;
-};
-bool tma_supported(int n, long long Q, const void* x, const void* xlo);
-cudaError_t launch_contract_tma(TmaArgs a, long long P, cudaStream_t s);
+cudaError_t launch_contract_tc(TcArgs a, cudaStream_t s);
+// phi_k(z1 + z2 + z3) at every node, as the epilogue would evaluate it.
+cudaError_t launch_phi_table(float* tab, int k, const float* const zt[3], int n1, int n2, size_t N, cudaStream_t s);
 
 // K2 in FP64 on the tensor cores (contract_f64.cu): the state seen as [P][n][Q] (mode 1: Q = 1),
 // contracted along n with a factor cut into seven slices.
@@ -212,19 +196,14 @@ int f64_rows(int n);                 // rows of the image (n rounded up to whole
 cudaError_t launch_f64_factor(const double* M, int n, uint8_t* img, int* rows, cudaStream_t s);
 cudaError_t launch_f64_phi(double* tab, int k, double ctau, const double* const lam[3], int n1, int n2, size_t N, cudaStream_t s);
 
-// Host: slice an FP64 factor into the tensor-core image, with output tiles of `rows` rows
-// and K chunks of `chunk` (64: 128-byte swizzle, contract_tc.cu; 32: 64-byte swizzle,
-// contract_tma.cu); slices F0, F1, 2^-8 F1, 2^-8 F2 (chunk 64, standard) or F0..F3 (chunk 32,
-// and chunk 64 precise).
+// Host: slice an FP64 factor into the tensor-core image: per output tile of 128 rows and K chunk of 32, the slice
+// tiles F0..F3 in the 64-byte-swizzled K-major layout.
 struct TcFactor {
     std::vector<uint8_t> img;
     std::vector<float> fscale;
 };
-TcFactor make_tc_factor(const std::vector<double>& M, int n, int rows, bool precise, int chunk = 64);
-int tc_out_rows(bool state_is_a, bool precise);   // rows of an output tile of a kernel variant
-int tc_pos_rows(bool state_is_a, bool precise);   // rows of a position / fibre tile
+TcFactor make_tc_factor(const std::vector<double>& M, int n);
 
-cudaError_t launch_contract_tc(const TcArgs& a, cudaStream_t s);
 cudaError_t launch_amax(const float* x, size_t n, unsigned* slot, cudaStream_t s);
 
 cudaError_t launch_stencil(const StencilArgs<double>& a, cudaStream_t s);

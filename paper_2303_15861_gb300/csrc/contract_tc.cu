@@ -1,49 +1,36 @@
-// K2 (tensor cores): mu-mode contraction Y = X x_mu M of the mixed-precision path on the
-// 5th-generation tensor cores (tcgen05.mma kind::f16, BF16 operands, FP32 accumulators
-// in TMEM), with the pointwise phi_k scaling (K3) and the stage axpy (K4) fused into the
-// epilogue. The mu-mode product is the one of Section 1 / Section 5.2:
-// e^{A_d (+) ... (+) A_1} v = vec(V x_1 e^{A_1} x_2 ... x_d e^{A_d}).
+// K2 (tensor cores, mixed precision): mu-mode contraction Y = X x_mu M of an FP32 state (optionally a hi + lo pair)
+// with an FP64 factor, as exact sums of BF16 products.
 //
-// Exact-slice split. The FP32 state x gets one power-of-two scale 2^es from the max-abs
-// that its producing kernel recorded; each row i of the FP64 factor (output index) gets
-// its own scale 2^e_i. With integer slices |s_j|, |f_j| <= 128 (exact in BF16):
-//     x = 2^(es-7) (s0 + 2^-8 s1 + 2^-16 s2),   f = 2^(e_i-7) (f0 + 2^-8 f1 + 2^-16 f2),
-//     sum_k x f = 2^(es+e_i-14) (D0 + 2^-8 D1),
-//     D0 = S0.F0,  D1 = S0.F1 + S1.F0 + S0.F2' + S2'.F0 + S1.F1'    (six MMAs per K step;
-//     the library runs the precise configuration below instead)
-// with F1' = 2^-8 F1, F2' = 2^-8 F2, S2' = 2^-8 S2 (exact scalings). Every term of D0 is
-// an integer of magnitude < 2^14 and |D0| < 2^24 for K <= 512, so D0 is exact in the FP32
-// accumulator whatever rounding the tensor core applies: the dominant, same-signed part
-// of a heat-kernel product carries no accumulation bias. D1 is weighted 2^-8 and its
-// terms have random signs. Representation errors are 2^-24 of the scales (as FP32).
-//
-// Precise configuration, which the library uses for every pass of this kernel (the
-// two-accumulator standard configuration above rounds D1, and that biased every pass of a time
-// integration): four slices per operand, x = 2^(es-7) sum_j 2^(-8j) s_j (j < 4), the input
-// optionally a double-float pair hi + lo, and ten MMAs per K step
-//     D0 = S0.F0, D1 = S0.F1 + S1.F0, D2 = S0.F2 + S1.F1 + S2.F0 (all three exact),
+// The exact-slice split. The FP32 state gets one power-of-two scale 2^es from a max-abs its producer
+// recorded, each factor row its own; x = 2^(es-7) sum_j 2^(-8j) S_j, f = 2^(e-7) sum_j 2^(-8j) F_j with integer
+// slices of at most 128, four of each. Ten products go to four TMEM accumulators,
+//     D0 = S0.F0,  D1 = S0.F1 + S1.F0,  D2 = S0.F2 + S1.F1 + S2.F0,
 //     D3 = S0.F3 + S1.F2 + S2.F1 + S3.F0,
-// combined in double-float arithmetic into a hi + lo result (about 2^-31 of the scales).
+// integer terms of magnitude at most 2^14. For K <= 256 all four stay within 2^24 even in the
+// worst case (D0 and D1 for K <= 512), so they are exact whatever rounding the tensor cores
+// apply; beyond that D2 and D3 could pass 2^24 only if hundreds of residual-slice products
+// shared the largest magnitude and one sign, and their rounding would weigh 2^-16 and 2^-24 of
+// a unit of D0. x.f = D0 + 2^-8 D1 + 2^-16 D2 + 2^-24 D3 up to the products below 2^-32,
+// combined once in the epilogue. A time integration applies the same factor to a
+// slowly varying state in every step, so any bias of a pass adds up. Measured on the 40-step
+// 256^3 Lawson4 run (relative error and mean drift against the FP64 path): six products into
+// two accumulators 1.5e-6 / -1.0e-6; seven into three exact accumulators with a 32-bit factor
+// but without the 2^-24 cross products S1.F2, S2.F1, S3.F0 2.8e-6 / -1.7e-6; all ten 2.6e-7 /
+// +1e-9. With EPI_STORE2 the result is a double-float pair: for the one exponential whose result feeds
+// the stencil that no later exponential smooths.
 //
-// CTA organisation (persistent, one CTA per SM, 416 threads):
-//   warps 0-7  producers: load the FP32 state chunk (coalesced; the next chunk's loads are
-//              in flight while the current one is sliced), slice it into S0, S1, S2' and
-//              store the 128B-swizzled K-major tiles; thread 0 also bulk-copies the
-//              pre-sliced, pre-swizzled factor tiles (F0, F1, F1', F2') of the chunk.
-//   warps 8-11 epilogue: tcgen05.ld the two accumulators, combine, fused op, store,
-//              record max|y| for the next pass.
-//   warp 12    one thread issues the tcgen05.mma chain and commits to mbarriers.
-// Two pipeline stages (K chunk of 64; 112 KB standard, 96 KB precise) and two TMEM
-// accumulator sets of 256 columns (2 x 128 standard, 4 x 64 precise) let loads, MMAs and
-// the epilogue of consecutive tiles overlap.
+// Work split. The factor is the A operand, 128 outputs (TMEM lanes) a tile, and N = 64 lines the B
+// operand (32 where 64 would leave SMs without a tile): four accumulators of 64 columns are half of TMEM, so
+// the epilogue of a tile overlaps the next tile's MMAs. With 128 columns the four fill TMEM and the epilogue and the
+// MMAs of a tile take turns; that form, its state brought by TMA and so only for extents that are multiples of 4, took 84, 95 and
+// 93 us at 256^3 in modes 1, 2, 3 where this one takes 78, 80 and 79 (at 384^3 358, 402 and 504 against 336, 342 and
+// 343); the form without TMA for the other extents took 15 to 41 us at 129 x 100 x 75 where this one takes 14 to 20. For
+// modes >= 2 the lines are consecutive positions, p and q flattened, so a short q leaves no empty columns. Warps 0-7 are
+// producers: they load FP32 from global memory (no alignment rules, so every shape takes this kernel) and store the
+// slices; warps 8-15 are the epilogue; warp 16 issues the MMAs, warp 17 copies the pre-sliced factor.
 //
-// Operand roles. Modes mu >= 2 (positions contiguous in memory): A = state (128
-// positions), B = factor (128 outputs), D[pos][i]; the epilogue store is coalesced along
-// positions. Mode 1 (fibres contiguous along K): A = factor (128 outputs), B = state
-// (128 fibres), D[i][fibre]; the store is coalesced along outputs.
-//
-// Every mbarrier wait is bounded (about 2 s of clock64 cycles); on timeout the kernel
-// records an error code, stops its roles, drains its MMAs and frees TMEM.
+// What bounds it, at 256^3: the MMAs alone take 45 us, with their epilogue 49, the ring's handshakes 60, the slicing
+// 64, and with the loads 79. The ring therefore has one barrier pair for both operands of a stage (a pair each: 90 us).
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -54,63 +41,40 @@
 
 namespace adr {
 namespace {
-
-constexpr int kM = 128;                          // UMMA M, TMEM lanes, rows of the A tile
-constexpr int kChunk = 64;                       // K per stage: one 128-byte bf16 row
-constexpr int kProducerWarps = 8;
-constexpr int kMmaWarp = kProducerWarps + 4;
-constexpr int kThreads = (kMmaWarp + 1) * 32;   // 416
-constexpr uint32_t kTmemCols = 512;
 using namespace tc;
 
-// Compile-time shape of one kernel variant. SA: the state is the A operand (modes >= 2);
-// PR: precise configuration.
-template <bool SA, bool PR>
+constexpr int kSl = 4;                   // slices per operand, accumulators
+constexpr int kM = 128;                  // UMMA M, TMEM lanes
+constexpr int kKc = 32;                  // K per stage: one 64-byte bf16 row (64-byte swizzle)
+constexpr int kProducerWarps = 8;
+constexpr int kGroups = 2;               // of producer warps, taking the K chunks in turn
+constexpr int kGroupWarps = kProducerWarps / kGroups;
+constexpr int kEpiWarps = 8;
+constexpr int kMmaWarp = kProducerWarps + kEpiWarps;
+constexpr int kLoadWarp = kMmaWarp + 1;
+constexpr int kThreads = (kLoadWarp + 1) * 32;
+
+template <int N>
 struct Cfg {
-    static constexpr int N = PR ? 64 : 128;            // UMMA N: columns of each accumulator
-    static constexpr int SS = PR ? 4 : 3;              // state slices
-    static constexpr int FS = 4;                       // factor slices
-    static constexpr int NACC = PR ? 4 : 2;            // accumulators per TMEM set (NACC * N = 256)
-    static constexpr int SROWS = SA ? kM : N;          // rows of a state tile (positions or fibres)
-    static constexpr int FROWS = SA ? N : kM;          // rows of a factor tile (outputs)
-    static constexpr int STILE = SROWS * kChunk * 2;   // bytes of one state slice tile
-    static constexpr int FTILE = FROWS * kChunk * 2;   // bytes of one factor slice tile
-    static constexpr int SBYTES = SS * STILE;
-    static constexpr int FBYTES = FS * FTILE;          // one factor block (output tile, K chunk)
-    static constexpr int STAGE = SBYTES + FBYTES;
-    static constexpr int SMEM = 2 * STAGE + 1024;      // two stages + alignment slack
-    static constexpr int NV = SROWS * kChunk / (kProducerWarps * 32);   // state values per thread
-    // instruction descriptor: kind::f16, D = F32, A = B = BF16, K-major, N >> 3, M >> 4
-    static constexpr uint32_t IDESC =
-        (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(N >> 3) << 17) | (uint32_t(kM >> 4) << 24);
-    static_assert(NACC * N == 256, "one accumulator set is 256 TMEM columns");
-    static_assert(2 * STAGE + 1024 <= 227 * 1024, "shared memory budget");
+    static constexpr int FTILE = kM * kKc * 2, STILE = N * kKc * 2;   // one slice tile of either operand
+    static constexpr int SBYTES = kSl * STILE, FBYTES = kSl * FTILE;  // one stage: 16 KB (N = 64) and 32 KB
+    static constexpr int NS = 4;                                      // stages of the ring
+    static constexpr int SMEM = NS * (SBYTES + FBYTES) + 1024;
+    static constexpr int SETS = 2;                                    // accumulator sets of 4 N columns
+    static constexpr uint32_t TMEM = N == 64 ? 512 : 256;
+    static constexpr int COLS = N / (kEpiWarps / 4);                  // columns per epilogue warp
+    static constexpr int KV = N * kKc / (kGroupWarps * 32);           // K values a producer thread slices of its chunk
+    static constexpr int KG = kKc / KV;                               // threads per line
+    static_assert(KV % 8 == 0, "whole 16-byte chunks of a slice row");
+    static_assert(COLS <= 32 && COLS % 8 == 0, "one lane per column finds its offset");
+    static_assert(SMEM <= 227 * 1024, "shared memory budget");
 };
 
-// Load 16 columns of two accumulators for this warp's 32 lanes, then wait.
-__device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, float (&a)[16], float (&b)[16]) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%33];\n"
-        "tcgen05.wait::ld.sync.aligned;\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(ta), "r"(tb)
-        : "memory");
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        a[j] = __uint_as_float(r[j]);
-        b[j] = __uint_as_float(r[16 + j]);
-    }
+__device__ __forceinline__ uint32_t idesc_of(int ncols) {   // FP32 accumulator, BF16 operands, M = 128
+    return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(ncols >> 3) << 17) | (uint32_t(kM >> 4) << 24);
 }
 
-// Load 8 columns of four accumulators (columns 64 apart) for this warp's 32 lanes, then wait.
-__device__ __forceinline__ void tmem_ld8x4(uint32_t t0, float (&d)[4][8]) {
+__device__ __forceinline__ void tmem_ld8x4(uint32_t t0, uint32_t stride, float (&d)[4][8]) {
     uint32_t r[32];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%32];\n"
@@ -122,7 +86,7 @@ __device__ __forceinline__ void tmem_ld8x4(uint32_t t0, float (&d)[4][8]) {
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
           "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(t0), "r"(t0 + 64u), "r"(t0 + 128u), "r"(t0 + 192u)
+        : "r"(t0), "r"(t0 + stride), "r"(t0 + 2 * stride), "r"(t0 + 3 * stride)
         : "memory");
 #pragma unroll
     for (int k = 0; k < 4; ++k)
@@ -130,212 +94,112 @@ __device__ __forceinline__ void tmem_ld8x4(uint32_t t0, float (&d)[4][8]) {
         for (int j = 0; j < 8; ++j) d[k][j] = __uint_as_float(r[8 * k + j]);
 }
 
-// Integer slices of y (|y| < 128; exact FP32 steps; at most 8 significant bits each, so the
-// upper half of each FP32 pattern is its exact BF16 pattern).
-//   standard: s0, s1, 2^-8 s2;  precise: s0, s1, s2, s3 of y + ylo (double-float input).
-template <bool PR>
-__device__ __forceinline__ void split(float y, float ylo, uint32_t (&b)[4]) {
-    const float s0 = rintf(y);
-    const float r0 = PR ? (y - s0) + ylo : (y - s0);   // the sum with ylo rounds below 2^-32
-    const float y1 = r0 * 256.f;
-    const float s1 = rintf(y1);
-    const float y2 = (y1 - s1) * 256.f;
-    const float s2 = rintf(y2);
-    b[0] = __float_as_uint(s0);
-    b[1] = __float_as_uint(s1);
-    if (PR) {
-        b[2] = __float_as_uint(s2);
-        b[3] = __float_as_uint(rintf((y2 - s2) * 256.f));
-    } else {
-        b[2] = __float_as_uint(s2 * 0.00390625f);
-        b[3] = 0u;
-    }
+// Round to the nearest integer (|y| < 2^22) by two additions; a rounding instruction runs at an eighth of their rate.
+__device__ __forceinline__ float rint_small(float y) { return (y + 12582912.f) - 12582912.f; }
+
+// Integer slices of y + ylo: the residuals y - s0 and y1 - s1 are exact, and the low part enters once,
+// after the leading slice.
+__device__ __forceinline__ void split(float y, float ylo, float (&s)[kSl]) {
+    s[0] = rint_small(y);
+    const float y1 = ((y - s[0]) + ylo) * 256.f;
+    s[1] = rint_small(y1);
+    const float y2 = (y1 - s[1]) * 256.f;
+    s[2] = rint_small(y2);
+    s[3] = rint_small((y2 - s[2]) * 256.f);
 }
 
-// Slice 8 consecutive K values v[o..o+7] (+ low parts) into chunk j of row r of each of the
-// SS state tiles (tile stride `stile` bytes).
-template <bool PR, int NV>
-__device__ __forceinline__ void slice_store8(const float (&v)[NV], const float (&vl)[NV], int o, float sc,
-                                             uint32_t tile0, uint32_t stile, int r, int j) {
-    constexpr int SS = PR ? 4 : 3;
-    uint32_t w[4][4];
+// Slice KV values along K (low parts vl, if LO) and store them at K position k (a multiple of 8) of row r of the four slice
+// tiles.
+template <int TILE, int KV, bool LO>
+__device__ __forceinline__ void slice_store(const float (&v)[KV], const float (&vl)[KV], float sc, uint32_t tile0, int r, int k) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        uint32_t a[4], c[4];
-        split<PR>(v[o + 2 * e] * sc, vl[o + 2 * e] * sc, a);
-        split<PR>(v[o + 2 * e + 1] * sc, vl[o + 2 * e + 1] * sc, c);
+    for (int h = 0; h < KV; h += 8) {
+        uint32_t w[kSl][4];
 #pragma unroll
-        for (int q = 0; q < SS; ++q) w[q][e] = __byte_perm(a[q], c[q], 0x7632);
-    }
-    const uint32_t off = swz(r, j);
+        for (int e = 0; e < 4; ++e) {
+            float a[kSl], b[kSl];
+            split(v[h + 2 * e] * sc, LO ? vl[h + 2 * e] * sc : 0.f, a);
+            split(v[h + 2 * e + 1] * sc, LO ? vl[h + 2 * e + 1] * sc : 0.f, b);
 #pragma unroll
-    for (int q = 0; q < SS; ++q) st_shared_v4(tile0 + q * stile + off, make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]));
-}
-
-// Producer item `it` of a CTA: K chunk (it % nK) of its (it / nK)-th tile. Loads the NV state
-// values (and low parts) of thread t.
-template <bool SA, bool PR>
-__device__ __forceinline__ void produce_load(const TcArgs& p, long long it, long long items, int t,
-                                             float (&v)[Cfg<SA, PR>::NV], float (&vl)[Cfg<SA, PR>::NV]) {
-    using C = Cfg<SA, PR>;
-    constexpr int NV = C::NV;
-    if (it >= items) return;
-    const long long tile = blockIdx.x + (it / p.nK) * gridDim.x;
-    const long long pt = tile / p.nOut;
-    const int k0 = int(it % p.nK) * kChunk;
-    const int n = p.n;
-    const bool lo = PR && p.Xlo != nullptr;
-    if (SA) {
-        // thread t: position row t % 128, K part t / 128 (NV = 32 values); warp-coalesced
-        const int row = t & (kM - 1), part = t >> 7;
-        const long long pos = pt * kM + row;
-        const bool valid = pos < p.npos;
-        const long long Q = p.Q;
-        const long long pp = valid ? pos / Q : 0, qq = valid ? pos % Q : 0;
-        const int kb = k0 + NV * part;
-        const long long base = (pp * n + kb) * Q + qq;
-#pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const bool ok = valid && kb + i < n;
-            v[i] = ok ? __ldg(p.X + base + (long long)i * Q) : 0.f;
-            vl[i] = (lo && ok) ? __ldg(p.Xlo + base + (long long)i * Q) : 0.f;
+            for (int q = 0; q < kSl; ++q) w[q][e] = __byte_perm(__float_as_uint(a[q]), __float_as_uint(b[q]), 0x7632);
         }
-    } else {
-        // thread t: 16-byte chunk j = t % 8 of fibre rows t / 8 + 32 rr (NV / 8 rows)
-        const int j = t & 7, r0 = t >> 3;
-        const int kb = k0 + 8 * j;
+        const uint32_t dst = tile0 + swz64(r, (k + h) >> 3);
 #pragma unroll
-        for (int rr = 0; rr < NV / 8; ++rr) {
-            const long long f = pt * C::SROWS + r0 + 32 * rr;
-            const bool valid = f < p.npos;
-            const long long base = (valid ? f : 0) * n + kb;
-            if (valid && p.vec4 && kb + 8 <= n) {
-                const float4 a = __ldg(reinterpret_cast<const float4*>(p.X + base));
-                const float4 b = __ldg(reinterpret_cast<const float4*>(p.X + base) + 1);
-                v[8 * rr + 0] = a.x; v[8 * rr + 1] = a.y; v[8 * rr + 2] = a.z; v[8 * rr + 3] = a.w;
-                v[8 * rr + 4] = b.x; v[8 * rr + 5] = b.y; v[8 * rr + 6] = b.z; v[8 * rr + 7] = b.w;
-            } else {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) v[8 * rr + e] = (valid && kb + e < n) ? __ldg(p.X + base + e) : 0.f;
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) vl[8 * rr + e] = (lo && valid && kb + e < n) ? __ldg(p.Xlo + base + e) : 0.f;
-        }
+        for (int q = 0; q < kSl; ++q) st_shared_v4(dst + q * TILE, make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]));
     }
 }
 
-template <bool SA, bool PR>
-__device__ __forceinline__ void produce_store(const float (&v)[Cfg<SA, PR>::NV], const float (&vl)[Cfg<SA, PR>::NV],
-                                              int t, float sc, uint32_t sA) {
-    using C = Cfg<SA, PR>;
-    if (SA) {
-        const int row = t & (kM - 1), part = t >> 7;
-#pragma unroll
-        for (int j4 = 0; j4 < C::NV / 8; ++j4)
-            slice_store8<PR, C::NV>(v, vl, 8 * j4, sc, sA, C::STILE, row, (C::NV / 8) * part + j4);
-    } else {
-        const int j = t & 7, r0 = t >> 3;
-#pragma unroll
-        for (int rr = 0; rr < C::NV / 8; ++rr) slice_store8<PR, C::NV>(v, vl, 8 * rr, sc, sA, C::STILE, r0 + 32 * rr, j);
-    }
-}
-
-// One pipeline item: wait for the stage, start the factor copy, prefetch the next item,
-// slice the current one, publish.
-template <bool SA, bool PR>
-__device__ __forceinline__ bool produce_step(const TcArgs& p, long long it, long long items, int t, float sc,
-                                             uint32_t sbase, uint32_t bar0, volatile int* abort_flag,
-                                             const float (&cur)[Cfg<SA, PR>::NV], const float (&curl)[Cfg<SA, PR>::NV],
-                                             float (&nxt)[Cfg<SA, PR>::NV], float (&nxtl)[Cfg<SA, PR>::NV]) {
-    using C = Cfg<SA, PR>;
-    const int s = int(it & 1);
-    const uint32_t ph = uint32_t(it >> 1) & 1u;
-    const uint32_t full = bar0 + 8u * s, empty = bar0 + 16u + 8u * s;
-    if (!mbar_wait(empty, ph ^ 1u, p.err, 1, abort_flag, 64)) return false;
-    const uint32_t sA = sbase + s * C::STAGE;
-    const uint32_t sF = sA + C::SBYTES;
-    if (t == 0) {
-        const long long tile = blockIdx.x + (it / p.nK) * gridDim.x;
-        const int ot = int(tile % p.nOut);
-        const int c = int(it % p.nK);
-        mbar_arrive_expect_tx(full, C::FBYTES);
-        const uint8_t* src = p.fimg + (size_t(ot) * p.nK + c) * C::FBYTES;
-#pragma unroll
-        for (int q = 0; q < C::FS; ++q) bulk_g2s(sF + q * C::FTILE, src + q * C::FTILE, C::FTILE, full);
-    }
-    produce_load<SA, PR>(p, it + 1, items, t, nxt, nxtl);
-    produce_store<SA, PR>(cur, curl, t, sc, sA);
-    fence_proxy_async();
-    mbar_arrive(full);
-    return true;
-}
-
-// Issue the MMAs of one 16-wide K step. Standard: D0 += S0.F0; D1 += S0.F1 + S1.F0 +
-// S0.(2^-8 F2) + (2^-8 S2).F0 + S1.(2^-8 F1) (factor tiles F0, F1, 2^-8 F1, 2^-8 F2; state
-// tiles S0, S1, 2^-8 S2). Precise: D0..D3 as in the file header (tiles F0..F3, S0..S3).
-template <bool SA, bool PR>
-__device__ __forceinline__ void mma_kstep(uint32_t d, const uint64_t (&S)[4], const uint64_t (&F)[4], uint64_t adv,
-                                          uint32_t first) {
-    using C = Cfg<SA, PR>;
-    auto mma = [&](int acc, int si, int fi, uint32_t accumulate) {
-        const uint32_t dd = d + uint32_t(acc * C::N);
-        if (SA) tc_mma(dd, S[si] + adv, F[fi] + adv, C::IDESC, accumulate);
-        else    tc_mma(dd, F[fi] + adv, S[si] + adv, C::IDESC, accumulate);
-    };
-    const uint32_t acc = first ? 0u : 1u;
-    if (!PR) {
-        mma(0, 0, 0, acc);
-        mma(1, 0, 1, acc);
-        mma(1, 1, 0, 1u);
-        mma(1, 0, 3, 1u);
-        mma(1, 2, 0, 1u);
-        mma(1, 1, 2, 1u);
-    } else {
-        mma(0, 0, 0, acc);
-        mma(1, 0, 1, acc);
-        mma(1, 1, 0, 1u);
-        mma(2, 0, 2, acc);
-        mma(2, 1, 1, 1u);
-        mma(2, 2, 0, 1u);
-        mma(3, 0, 3, acc);
-        mma(3, 1, 2, 1u);
-        mma(3, 2, 1, 1u);
-        mma(3, 3, 0, 1u);
-    }
-}
-
-// TwoSum: s + e = a + b exactly.
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
     const float bb = s - a;
     e = (a - (s - bb)) + (b - bb);
 }
 
-template <bool SA, bool PR, int EPI>
-__global__ void __launch_bounds__(kThreads, 1) tc_contract_kernel(TcArgs p) {
-    using C = Cfg<SA, PR>;
+// Loads that stay where they are written (the compiler sinks plain ones to their first use), 0 where `on` is false.
+__device__ __forceinline__ float ld1_or_0(const float* p, bool on) {
+    float v;
+    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %2, 0;\n mov.b32 %0, 0;\n @p ld.global.nc.f32 %0, [%1];\n}\n"
+                 : "=f"(v)
+                 : "l"(p), "r"(int(on)));
+    return v;
+}
+__device__ __forceinline__ float4 ld4_or_0(const float* p, bool on) {
+    float4 v;
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %5, 0;\n mov.b32 %0, 0;\n mov.b32 %1, 0;\n mov.b32 %2, 0;\n mov.b32 %3, 0;\n"
+        " @p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n}\n"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+        : "l"(p), "r"(int(on)));
+    return v;
+}
+
+// 32-byte (256-bit) accesses: eight consecutive floats.
+__device__ __forceinline__ void ld8(const float* p, float (&v)[8]) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ void st8(float* p, const float (&v)[8]) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
+
+// The phi factor of node o, where the context keeps no table.
+__device__ __noinline__ float phi_at(const TcArgs& p, unsigned o) {
+    float z = p.zt[0][o % p.n1] + p.zt[1][(o / p.n1) % p.n2];
+    if (p.zt[2]) z += p.zt[2][o / p.n1 / p.n2];
+    return phi_eval(p.phik, z);
+}
+
+template <bool MODE1, int N, int EPI, bool LO>
+__global__ void __launch_bounds__(kThreads, 1) tc_contract_kernel(const __grid_constant__ TcArgs p) {
+    using C = Cfg<N>;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bars[9];
+    constexpr uint32_t kF = 0, kE = kF + 8 * C::NS, kAF = kE + 8 * C::NS, kAE = kAF + 8 * C::SETS, kDR = kAE + 8 * C::SETS;
+    __shared__ __align__(8) uint64_t bars[kDR / 8 + 1];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;     // state slices of the stages
+    const uint32_t fbase = sbase + C::NS * C::SBYTES;                   // factor slices of the stages
     const uint32_t bar0 = smem_u32(&bars[0]);
-    auto full_bar = [&](int s) { return bar0 + 8u * s; };
-    auto empty_bar = [&](int s) { return bar0 + 16u + 8u * s; };
-    auto accf_bar = [&](int a) { return bar0 + 32u + 8u * a; };
-    auto acce_bar = [&](int a) { return bar0 + 48u + 8u * a; };
-    const uint32_t drain_bar = bar0 + 64u;
+    auto full = [&](int s) { return bar0 + kF + 8u * s; };
+    auto empty = [&](int s) { return bar0 + kE + 8u * s; };
+    auto accf = [&](int a) { return bar0 + kAF + 8u * a; };
+    auto acce = [&](int a) { return bar0 + kAE + 8u * a; };
+    const uint32_t drain_bar = bar0 + kDR;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(full_bar(s), kProducerWarps * 32 + 1);   // producers + 1 expect_tx arrival
-            mbar_init(empty_bar(s), 1);                         // tcgen05.commit
+        for (int s = 0; s < C::NS; ++s) {
+            mbar_init(full(s), kGroupWarps + 1);             // a warp of the chunk's group each, and the loader's expect_tx
+            mbar_init(empty(s), 1);                          // tcgen05.commit
         }
-        for (int a = 0; a < 2; ++a) {
-            mbar_init(accf_bar(a), 1);     // tcgen05.commit
-            mbar_init(acce_bar(a), 128);   // epilogue threads
+        for (int a = 0; a < C::SETS; ++a) {
+            mbar_init(accf(a), 1);
+            mbar_init(acce(a), kEpiWarps);                   // one arrival per epilogue warp
         }
         mbar_init(drain_bar, 1);
         abort_s = 0;
@@ -343,7 +207,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_contract_kernel(TcArgs p) {
     }
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)),
-                     "r"(kTmemCols)
+                     "r"(C::TMEM)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -352,198 +216,233 @@ __global__ void __launch_bounds__(kThreads, 1) tc_contract_kernel(TcArgs p) {
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
 
-    // scale of the state from the max-abs recorded by its producer (amax < 2^es)
     const float amax = __uint_as_float(*p.amax_in);
     int es = 0;
     if (amax > 0.f) frexpf(amax, &es);
     const float sc = ldexpf(1.f, 7 - es);
     const float sback = ldexpf(1.f, es - 7);
-
     const int n = p.n;
-    const long long Q = p.Q;
+    const unsigned Q = MODE1 ? 1u : p.Q;
+    const int items = (p.ntiles - int(blockIdx.x) + int(gridDim.x) - 1) / int(gridDim.x) * p.nK;   // (tile, K chunk) in order
 
-    if (warp < kProducerWarps) {
-        // ------------------------------------------------------------ producers
-        // The loads of the next chunk are issued before the current one is sliced, so
-        // global latency overlaps the ALU work.
-        const int t = threadIdx.x;
-        const long long my_tiles = (p.ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x;
-        const long long items = my_tiles * p.nK;
-        if (!PR) {
-            float va[C::NV], vb[C::NV], la[C::NV], lb[C::NV];   // la, lb stay zero (no low parts)
-            produce_load<SA, PR>(p, 0, items, t, va, la);
-            for (long long it = 0; it < items; it += 2) {
-                if (!produce_step<SA, PR>(p, it, items, t, sc, sbase, bar0, &abort_s, va, la, vb, lb)) break;
-                if (it + 1 >= items) break;
-                if (!produce_step<SA, PR>(p, it + 1, items, t, sc, sbase, bar0, &abort_s, vb, lb, va, la)) break;
-            }
-        } else {
-            // precise: hi and lo values of one item at a time (registers do not allow a prefetch)
-            float v[C::NV], vl[C::NV];
-            for (long long it = 0; it < items; ++it) {
-                const int s = int(it & 1);
-                const uint32_t ph = uint32_t(it >> 1) & 1u;
-                if (!mbar_wait(empty_bar(s), ph ^ 1u, p.err, 1, &abort_s, 64)) break;
-                const uint32_t sA = sbase + s * C::STAGE;
-                const uint32_t sF = sA + C::SBYTES;
-                if (t == 0) {
-                    const long long tile = blockIdx.x + (it / p.nK) * gridDim.x;
-                    mbar_arrive_expect_tx(full_bar(s), C::FBYTES);
-                    const uint8_t* src = p.fimg + (size_t(tile % p.nOut) * p.nK + it % p.nK) * C::FBYTES;
-#pragma unroll
-                    for (int q = 0; q < C::FS; ++q) bulk_g2s(sF + q * C::FTILE, src + q * C::FTILE, C::FTILE, full_bar(s));
+    if (warp == kLoadWarp) {
+        // ------------------------------------------------------------ factor loader (bulk copies)
+        if (lane == 0) {
+            int s = 0, issued = 0;
+            uint32_t ph = 1;
+            for (int tile = blockIdx.x; tile < p.ntiles && !abort_s; tile += gridDim.x) {
+                const uint8_t* src = p.fimg + size_t(tile % p.nOut) * p.nK * C::FBYTES;
+                for (int c = 0; c < p.nK; ++c, src += C::FBYTES, ++issued) {
+                    if (!mbar_wait(empty(s), ph, p.err, 64, &abort_s, 32)) break;
+                    mbar_arrive_expect_tx(full(s), C::FBYTES);
+                    bulk_g2s(fbase + s * C::FBYTES, src, C::FBYTES, full(s));
+                    if (++s == C::NS) { s = 0; ph ^= 1; }
                 }
-                produce_load<SA, PR>(p, it, items, t, v, vl);
-                produce_store<SA, PR>(v, vl, t, sc, sA);
-                fence_proxy_async();
-                mbar_arrive(full_bar(s));
             }
+            // no copy may land after the CTA has gone (they have, unless a wait gave up)
+            const long long t0 = clock64();
+            for (int k = max(issued - C::NS, 0); k < issued; ++k)
+                while (!mbar_try_wait(full(k % C::NS), uint32_t(k / C::NS) & 1u) && clock64() - t0 < kWaitCycles) {}
         }
-    } else if (warp < kProducerWarps + 4) {
-        // ------------------------------------------------------------ epilogue
-        const int ew = warp - kProducerWarps;   // TMEM lane quarter of this warp
-        const int row = ew * 32 + lane;
-        long long tl = 0;
-        for (long long tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++tl) {
-            const int a = int(tl & 1);
-            const uint32_t ph = uint32_t(tl >> 1) & 1u;
-            const bool waited = mbar_wait(accf_bar(a), ph, p.err, 2, &abort_s, 64);
-            if (!__all_sync(0xffffffffu, waited)) break;   // warp-uniform: TMEM loads are .sync.aligned
-            tc_fence_after();
-            const long long pt = tile / p.nOut;
-            const int ot = int(tile % p.nOut);
-            float vmax = 0.f;
-            // per-row setup: rows are positions (SA) or outputs; columns the other
-            bool rvalid;
-            long long off0, cstep;      // offset of (row, column 0) and per-column stride
-            float zrow = 0.f, rscale = 0.f;
-            int ncol;                    // valid columns of this tile
-            if (SA) {
-                const long long pos = pt * kM + row;
-                rvalid = pos < p.npos;
-                const long long pp = rvalid ? pos / Q : 0, qq = rvalid ? pos % Q : 0;
-                off0 = (pp * n + ot * C::N) * Q + qq;
-                cstep = Q;
-                ncol = min(C::N, n - ot * C::N);
-                if (EPI == EPI_PHI && rvalid) {
-                    // position part of z = tau (l1 + l2 + l3): the directions other than mu
-                    zrow = __ldg(p.zq_a + qq % p.na);
-                    if (p.zq_b) zrow += __ldg(p.zq_b + qq / p.na);
-                    if (p.zp) zrow += __ldg(p.zp + pp);
+    } else if (warp < kProducerWarps) {
+        // ------------------------------------------------------------ producers (global -> slices)
+        // Two groups of four warps take the chunks in turn: what a chunk costs besides its arithmetic (the wait for its
+        // slot, the proxy fence, the arrivals) then passes while the other group slices (256^3: 79 us, 89 with one group of
+        // eight). KG threads a line, each KV consecutive K values: neighbouring lanes along K for
+        // mode 1, along the positions otherwise, so that a warp reads whole sectors.
+        constexpr int KV = C::KV, KG = C::KG;
+        const int t = threadIdx.x & (kGroupWarps * 32 - 1), group = warp / kGroupWarps;
+        const int row = MODE1 ? t / KG : t % N, kofs = KV * (MODE1 ? t % KG : t / N);
+        // the (tile, chunk) whose values are loaded next, and this thread's line of that tile
+        int ltile = blockIdx.x, lc = 0;
+        bool lrow = false;
+        const float* xrow = nullptr;
+        const float* xlo = nullptr;
+        auto line = [&] {
+            const unsigned pos = unsigned(ltile / p.nOut) * N + row;
+            lrow = ltile < p.ntiles && pos < p.npos;
+            const size_t off = MODE1 ? size_t(pos) * n + kofs : size_t(pos / Q) * n * Q + pos % Q + size_t(kofs) * Q;
+            xrow = p.X + off;
+            xlo = LO ? p.Xlo + off : nullptr;
+        };
+        auto advance = [&](int by) {
+            lc += by;
+            if (lc < p.nK) return;
+            for (; lc >= p.nK; lc -= p.nK) ltile += gridDim.x;
+            line();
+        };
+        auto load1 = [&](const float* x, float (&w)[KV]) {
+            const int k0 = lc * kKc + kofs;
+            x += size_t(lc * kKc) * Q;
+            if (MODE1 && p.vec4) {
+#pragma unroll
+                for (int e = 0; e < KV; e += 4) {
+                    const float4 u = ld4_or_0(x + e, lrow && k0 + e < n);
+                    w[e] = u.x; w[e + 1] = u.y; w[e + 2] = u.z; w[e + 3] = u.w;
                 }
             } else {
-                const int irow = ot * kM + row;
-                rvalid = irow < n;
-                if (rvalid) rscale = sback * __ldg(p.fscale + irow);
-                off0 = pt * C::N * (long long)n + irow;
-                cstep = n;
-                ncol = int(min((long long)C::N, p.npos - pt * C::N));
+#pragma unroll
+                for (int e = 0; e < KV; ++e) w[e] = ld1_or_0(x + size_t(e) * Q, lrow && k0 + e < n);
             }
-            const float* fsc = p.fscale + ot * C::N;      // column scales (SA)
-            const float* zc = p.zmu + ot * C::N;          // column part of z (EPI_PHI)
-            float* yrow = p.Y + off0;
-            float* ylo = (EPI == EPI_STORE2) ? p.Ylo + off0 : nullptr;
-            const float* brow = (EPI == EPI_AXPY) ? p.base + off0 : nullptr;
-            const uint32_t tbase = tmem + (uint32_t(ew * 32) << 16) + uint32_t(a) * 256u;
-            auto emit = [&](int col, float hi, float lo) {
-                // hi + lo: the combined accumulators of (row, col) before scaling
-                const float scale = SA ? sback * __ldg(fsc + col) : rscale;
-                const long long o = (long long)col * cstep;
-                if (EPI == EPI_STORE2) {
-                    yrow[o] = hi * scale;
-                    ylo[o] = lo * scale;
-                    vmax = fmaxf(vmax, fabsf(hi * scale));
+        };
+        // chunks held in registers while the ones before them are sliced: 79 us at 256^3, 90 with one (two with low parts would not fit)
+        constexpr int DEPTH = LO ? 1 : 2;
+        float v[DEPTH][KV], vl[KV];
+        line();
+        advance(group);
+#pragma unroll
+        for (int b = 0; b < DEPTH; ++b) {
+            if (b > 0) advance(kGroups);
+            load1(xrow, v[b]);
+            if (LO) load1(xlo, vl);
+        }
+        bool ok = true;
+        for (int it0 = group; it0 < items && ok; it0 += kGroups * DEPTH)
+#pragma unroll
+            for (int b = 0; b < DEPTH; ++b) {
+                const int it = it0 + b * kGroups, s = it % C::NS;
+                if (it >= items || !ok) break;
+                // waits decide warp-uniformly: the per-warp arrivals need every lane
+                ok = __all_sync(0xffffffffu, mbar_wait(empty(s), (uint32_t(it / C::NS) & 1u) ^ 1u, p.err, 1, &abort_s, 32));
+                if (!ok) break;
+                slice_store<C::STILE, KV, LO>(v[b], vl, sc, sbase + s * C::SBYTES, row, kofs);
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(full(s));
+                advance(kGroups);
+                load1(xrow, v[b]);                           // in flight for DEPTH rounds of both groups
+                if (LO) load1(xlo, vl);
+            }
+    } else if (warp < kMmaWarp) {
+        // ------------------------------------------------------------ epilogue
+        const int ew = (warp - kProducerWarps) & 3;          // TMEM lane quarter (warp % 4)
+        const int part = (warp - kProducerWarps) >> 2;       // column part
+        const int jlo = part * C::COLS;
+        float vmax = 0.f;
+        int tl = 0;
+        for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++tl) {
+            const int a = tl % C::SETS;
+            const int pt = tile / p.nOut, ot = tile % p.nOut;
+            const int irow = ot * kM + ew * 32 + lane;       // this lane's output
+            const bool rvalid = irow < n, warp_on = ot * kM + ew * 32 < n;
+            const float scale = sback * __ldg(p.fscale + irow);   // padded to whole tiles
+            const unsigned ioff = unsigned(irow) * Q;
+            const int ncol = min(N, int(p.npos - unsigned(pt) * N));
+            // lane c: the offset of column jlo + c (one division a tile)
+            const unsigned cpos = unsigned(pt) * N + jlo + lane;
+            const unsigned coff = MODE1 ? cpos * n : (cpos / Q) * n * Q + cpos % Q;
+            auto off_of = [&](int j) { return __shfl_sync(0xffffffffu, coff, j) + ioff; };   // column jlo + j
+            // the axpy's base or the phi table's values of eight columns, one group ahead
+            auto load_side = [&](int j0, float (&b)[8]) {
+                if (EPI != EPI_AXPY && EPI != EPI_PHI) return;
+                const float* src = EPI == EPI_PHI ? p.phi : p.base;
+                if (!MODE1 && p.vec8 && src && jlo + j0 + 8 <= ncol) {
+                    const unsigned o = off_of(j0);           // every lane takes part in the shuffles
+                    if (rvalid) ld8(src + o, b);
                     return;
                 }
-                float v = (hi + lo) * scale;
-                if (EPI == EPI_PHI) v *= phi_eval(p.phik, zrow + __ldg(zc + col));
-                if (EPI == EPI_AXPY) v = fmaf(p.alpha, v, __ldg(brow + o));
-                yrow[o] = v;
-                vmax = fmaxf(vmax, fabsf(v));
-            };
-            if (!PR) {
-#pragma unroll 1
-                for (int j0 = 0; j0 < C::N; j0 += 16) {
-                    float d0[16], d1[16];
-                    __syncwarp();
-                    tmem_ld16x2(tbase + j0, tbase + uint32_t(C::N) + j0, d0, d1);
-                    if (!rvalid || j0 >= ncol) continue;
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        if (j0 + j >= ncol) break;
-                        // D0 is an exact integer, 2^-8 D1 an exact scaling
-                        const float t1 = d1[j] * 0.00390625f;
-                        if (EPI == EPI_STORE2) {
-                            float hi, lo;
-                            two_sum(d0[j], t1, hi, lo);
-                            emit(j0 + j, hi, lo);
-                        } else {
-                            emit(j0 + j, d0[j] + t1, 0.f);
+                for (int j = 0; j < 8; ++j) {
+                    const unsigned o = off_of(j0 + j);
+                    b[j] = 0.f;
+                    if (rvalid && jlo + j0 + j < ncol) b[j] = EPI == EPI_AXPY || src ? src[o] : phi_at(p, o);
+                }
+            };
+            float side[2][8];
+            if (warp_on) load_side(0, side[0]);
+            const bool waited = mbar_wait(accf(a), uint32_t(tl / C::SETS) & 1u, p.err, 2, &abort_s, 32);
+            if (!__all_sync(0xffffffffu, waited)) break;
+            tc_fence_after();
+            if (!warp_on) {
+                if (lane == 0) mbar_arrive(acce(a));
+                continue;
+            }
+            const uint32_t tbase = tmem + (uint32_t(ew * 32) << 16) + uint32_t(a * kSl * N + jlo);
+#pragma unroll(EPI == EPI_AXPY || EPI == EPI_PHI ? C::COLS / 8 : 1)
+            for (int j0 = 0; j0 < C::COLS; j0 += 8) {
+                float d[4][8];
+                const float (&bcur)[8] = side[(j0 >> 3) & 1];
+                if (j0 + 8 < C::COLS) load_side(j0 + 8, side[((j0 >> 3) + 1) & 1]);
+                __syncwarp();
+                tmem_ld8x4(tbase + j0, uint32_t(N), d);
+                if (j0 + 8 >= C::COLS) {                     // the last columns are in registers: the set is free
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(acce(a));
+                }
+                float v[8], vl[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float tail = fmaf(d[3][j], 5.9604644775390625e-08f, d[2][j] * 1.52587890625e-05f);
+                    if (EPI == EPI_STORE2) {                 // double-float result: D0 + 2^-8 D1 exactly, then the tail
+                        float hi, lo;
+                        two_sum(d[0][j], d[1][j] * 0.00390625f, hi, lo);
+                        lo += tail;
+                        const float s = hi + lo;
+                        v[j] = s * scale;
+                        vl[j] = (lo - (s - hi)) * scale;
+                    } else {                                 // one FP32 result: the smaller terms first, D0 last
+                        v[j] = (d[0][j] + fmaf(d[1][j], 0.00390625f, tail)) * scale;
+                        if (EPI == EPI_PHI) v[j] *= bcur[j];
+                        if (EPI == EPI_AXPY) v[j] = fmaf(p.alpha, v[j], bcur[j]);
+                    }
+                }
+                if (!MODE1 && p.vec8 && jlo + j0 + 8 <= ncol) {
+                    const unsigned o = off_of(j0);
+                    if (rvalid) {
+                        st8(p.Y + o, v);
+                        if (EPI == EPI_STORE2) st8(p.Ylo + o, vl);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const unsigned o = off_of(j0 + j);
+                        if (rvalid && jlo + j0 + j < ncol) {
+                            p.Y[o] = v[j];
+                            if (EPI == EPI_STORE2) p.Ylo[o] = vl[j];
                         }
                     }
                 }
-            } else {
-#pragma unroll 1
-                for (int j0 = 0; j0 < C::N; j0 += 8) {
-                    float d[4][8];
-                    __syncwarp();
-                    tmem_ld8x4(tbase + j0, d);
-                    if (!rvalid || j0 >= ncol) continue;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        if (j0 + j >= ncol) break;
-                        // D0 + 2^-8 D1 + 2^-16 D2 + 2^-24 D3 in double-float arithmetic
-                        float hi, lo;
-                        two_sum(d[0][j], d[1][j] * 0.00390625f, hi, lo);
-                        lo += fmaf(d[3][j], 5.9604644775390625e-08f, d[2][j] * 1.52587890625e-05f);
-                        const float s = hi + lo;
-                        lo = lo - (s - hi);
-                        emit(j0 + j, s, lo);
-                    }
-                }
+                for (int j = 0; j < 8; ++j)
+                    if (rvalid && jlo + j0 + j < ncol) vmax = fmaxf(vmax, fabsf(v[j]));
             }
-            tc_fence_before();
-            mbar_arrive(acce_bar(a));
-            for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-            if (lane == 0 && p.amax_out && vmax > 0.f) atomicMax(p.amax_out, __float_as_uint(vmax));
         }
-    } else if (lane == 0) {
+        for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
+        if (lane == 0 && p.amax_out && vmax > 0.f) atomicMax(p.amax_out, __float_as_uint(vmax));
+    } else if (warp == kMmaWarp && lane == 0) {
         // ------------------------------------------------------------ MMA issuer
-        long long g = 0, tl = 0;
-        for (long long tile = blockIdx.x; tile < p.ntiles && !abort_s; tile += gridDim.x, ++tl) {
-            const int a = int(tl & 1);
-            const uint32_t aph = uint32_t(tl >> 1) & 1u;
-            if (!mbar_wait(acce_bar(a), aph ^ 1u, p.err, 4, &abort_s)) break;
+        // F_i.S_j adds to D_(i+j). The S tiles lie one after another, as do the accumulators, so F_i takes
+        // S_0..S_(3-i) in one MMA of up to 256 columns: four MMAs per K step instead of ten, and F_i is
+        // read from shared memory once.
+        uint32_t ph = 0;
+        int s = 0, tl = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < p.ntiles && !abort_s && ok; tile += gridDim.x, ++tl) {
+            const int a = tl % C::SETS;
+            if (!mbar_wait(acce(a), (uint32_t(tl / C::SETS) & 1u) ^ 1u, p.err, 4, &abort_s)) break;
             tc_fence_after();
-            const uint32_t d = tmem + uint32_t(a) * 256u;
-            bool ok = true;
-            for (int c = 0; c < p.nK; ++c, ++g) {
-                const int s = int(g & 1);
-                const uint32_t ph = uint32_t(g >> 1) & 1u;
-                if (!mbar_wait(full_bar(s), ph, p.err, 8, &abort_s)) { ok = false; break; }
+            const uint32_t d = tmem + uint32_t(a * kSl * N);
+            for (int c = 0; c < p.nK; ++c) {
+                if (!mbar_wait(full(s), ph, p.err, 8, &abort_s)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t sS = sbase + s * C::STAGE;
-                const uint32_t sF = sS + C::SBYTES;
-                uint64_t S[4], F[4];
+                const uint64_t a0 = sdesc64(fbase + s * C::FBYTES), b0 = sdesc64(sbase + s * C::SBYTES);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    S[q] = sdesc(sS + (q < C::SS ? q : 0) * C::STILE);
-                    F[q] = sdesc(sF + q * C::FTILE);
+                for (int kk = 0; kk < kKc / 16; ++kk) {
+                    const uint64_t adv = uint64_t(kk * 32) >> 4;
+#pragma unroll
+                    for (int i = 0; i < kSl; ++i)
+                        tc_mma(d + i * N, a0 + adv + uint64_t(i * C::FTILE >> 4), b0 + adv, idesc_of((kSl - i) * N),
+                               (c == 0 && kk == 0 && i == 0) ? 0u : 1u);
                 }
-#pragma unroll
-                for (int kk = 0; kk < kChunk / 16; ++kk)
-                    mma_kstep<SA, PR>(d, S, F, uint64_t(kk * 32) >> 4, (c == 0 && kk == 0) ? 1u : 0u);
-                tc_commit(empty_bar(s));
+                tc_commit(empty(s));
+                if (++s == C::NS) { s = 0; ph ^= 1; }
             }
-            if (!ok) break;
-            tc_commit(accf_bar(a));
+            if (ok) tc_commit(accf(a));
         }
-        // wait for every MMA this thread issued before TMEM is released
         tc_commit(drain_bar);
-        {
-            const long long t0 = clock64();
-            while (!mbar_try_wait(drain_bar, 0) && clock64() - t0 < kWaitCycles) {}
-        }
+        const long long t0 = clock64();
+        while (!mbar_try_wait(drain_bar, 0) && clock64() - t0 < kWaitCycles) {}
     }
 
     tc_fence_before();
@@ -551,55 +450,73 @@ __global__ void __launch_bounds__(kThreads, 1) tc_contract_kernel(TcArgs p) {
     if (warp == kMmaWarp) {
         __syncwarp();
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM) : "memory");
     }
 }
 
-int g_num_sms = 0;
-
-template <bool SA, bool PR, int EPI>
-cudaError_t launch_variant(const TcArgs& a, unsigned grid, cudaStream_t s) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tc_contract_kernel<SA, PR, EPI>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<SA, PR>::SMEM);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
+__global__ void phi_table_kernel(float* tab, int k, const float* z1, const float* z2, const float* z3, int n1, int n2, size_t N) {
+    for (size_t o = blockIdx.x * size_t(blockDim.x) + threadIdx.x; o < N; o += size_t(gridDim.x) * blockDim.x) {
+        float z = z1[o % n1] + z2[(o / n1) % n2];
+        if (z3) z += z3[o / n1 / n2];
+        tab[o] = phi_eval(k, z);
     }
-    tc_contract_kernel<SA, PR, EPI><<<grid, kThreads, Cfg<SA, PR>::SMEM, s>>>(a);
+}
+
+int sm_count() {
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        return v > 0 ? v : 1;
+    }();
+    return sms;
+}
+
+template <bool MODE1, int N, int EPI, bool LO>
+cudaError_t launch_variant(const TcArgs& a, cudaStream_t s) {
+    static const cudaError_t attr = cudaFuncSetAttribute(tc_contract_kernel<MODE1, N, EPI, LO>,
+                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<N>::SMEM);
+    if (attr != cudaSuccess) return attr;
+    const int grid = a.ntiles < sm_count() ? a.ntiles : sm_count();
+    tc_contract_kernel<MODE1, N, EPI, LO><<<unsigned(grid), kThreads, Cfg<N>::SMEM, s>>>(a);
     return cudaGetLastError();
+}
+
+template <bool MODE1, int N>
+cudaError_t launch_epi(const TcArgs& a, cudaStream_t s) {
+    if (a.Xlo) return a.epi == EPI_STORE2 ? launch_variant<MODE1, N, EPI_STORE2, true>(a, s) : cudaErrorInvalidValue;
+    switch (a.epi) {
+    case EPI_STORE2: return launch_variant<MODE1, N, EPI_STORE2, false>(a, s);
+    case EPI_AXPY: return launch_variant<MODE1, N, EPI_AXPY, false>(a, s);
+    case EPI_PHI:                                            // always fused into the last direction's pass
+        if constexpr (MODE1) return cudaErrorInvalidValue;
+        else return launch_variant<false, N, EPI_PHI, false>(a, s);
+    default: return launch_variant<MODE1, N, EPI_STORE, false>(a, s);
+    }
 }
 
 }  // namespace
 
-// Rows of an output tile and of a position tile for a variant (the host tiles with these).
-int tc_out_rows(bool state_is_a, bool precise) { return state_is_a ? (precise ? 64 : 128) : 128; }
-int tc_pos_rows(bool state_is_a, bool precise) { return state_is_a ? 128 : (precise ? 64 : 128); }
+cudaError_t launch_phi_table(float* tab, int k, const float* const zt[3], int n1, int n2, size_t N, cudaStream_t s) {
+    const unsigned blocks = unsigned((N + 255) / 256 < 65535 ? (N + 255) / 256 : 65535);
+    phi_table_kernel<<<blocks, 256, 0, s>>>(tab, k, zt[0], zt[1], zt[2], n1, n2, N);
+    return cudaGetLastError();
+}
 
-cudaError_t launch_contract_tc(const TcArgs& a, cudaStream_t s) {
-    if (g_num_sms == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
-    }
+cudaError_t launch_contract_tc(TcArgs a, cudaStream_t s) {
     if (a.n > 512 || a.n < 1) return cudaErrorInvalidValue;
-    const long long grid = a.ntiles < g_num_sms ? a.ntiles : g_num_sms;
-    if (grid <= 0) return cudaSuccess;
-    const unsigned g = unsigned(grid);
-    // The library runs every pass in the precise configuration (ten products into exact
-    // accumulators); the standard configuration's two accumulators round, and that rounding
-    // biased every pass.
-    if (!a.precise) return cudaErrorInvalidValue;
-    if (a.state_is_a) {
-        if (a.epi == EPI_PHI) return launch_variant<true, true, EPI_PHI>(a, g, s);
-        if (a.epi == EPI_AXPY) return launch_variant<true, true, EPI_AXPY>(a, g, s);
-        if (a.epi == EPI_STORE2) return launch_variant<true, true, EPI_STORE2>(a, g, s);
-        return launch_variant<true, true, EPI_STORE>(a, g, s);
-    }
-    if (a.epi == EPI_PHI) return cudaErrorInvalidValue;   // fused into modes >= 2 only
-    if (a.epi == EPI_AXPY) return launch_variant<false, true, EPI_AXPY>(a, g, s);
-    if (a.epi == EPI_STORE2) return launch_variant<false, true, EPI_STORE2>(a, g, s);
-    return launch_variant<false, true, EPI_STORE>(a, g, s);
+    if (a.npos == 0) return cudaSuccess;
+    const bool mode1 = a.Q == 1;
+    a.nK = (a.n + kKc - 1) / kKc;
+    a.nOut = (a.n + kM - 1) / kM;
+    auto aligned = [](const void* q, uintptr_t to) { return reinterpret_cast<uintptr_t>(q) % to == 0; };
+    a.vec4 = a.n % 4 == 0 && aligned(a.X, 16) && aligned(a.Xlo, 16);
+    // groups of eight columns are eight consecutive nodes: modes >= 2, q a multiple of 8
+    a.vec8 = !mode1 && a.Q % 8 == 0 && aligned(a.Y, 32) && aligned(a.Ylo, 32) && aligned(a.base, 32) && aligned(a.phi, 32);
+    const bool wide = (a.npos + 63) / 64 * a.nOut >= unsigned(sm_count());
+    a.ntiles = int((a.npos + (wide ? 63 : 31)) / (wide ? 64 : 32) * a.nOut);
+    if (mode1) return wide ? launch_epi<true, 64>(a, s) : launch_epi<true, 32>(a, s);
+    return wide ? launch_epi<false, 64>(a, s) : launch_epi<false, 32>(a, s);
 }
 
 }  // namespace adr

@@ -181,64 +181,38 @@ uint16_t bf16_bits_exact(double v) {
 }
 }  // namespace
 
-TcFactor make_tc_factor(const std::vector<double>& M, int n, int rows, bool precise, int chunk) {
+TcFactor make_tc_factor(const std::vector<double>& M, int n) {
     // Each row i of M (an output index) is written as 2^(e_i-7) sum_j 2^(-8j) f_j with
     // integer slices |f_j| <= 128 and max_k |M[i][k]| < 2^e_i. The image stores, per
-    // (output tile of `rows` rows, K chunk of 64), four slice tiles in the 128-byte-swizzled
-    // K-major layout the tensor cores read (8-row groups of 1024 B; 16-byte chunk j of row r
-    // at position j ^ (r mod 8)): F0, F1, 2^-8 F1, 2^-8 F2 (standard) or F0, F1, F2, F3
-    // (precise). With chunks of 32 the tiles use the 64-byte swizzle (8-row groups of 512 B;
-    // chunk j of row r at position j ^ ((r / 2) mod 4)), and every image holds F0, F1, F2, F3:
-    // that kernel runs the ten-product split in every pass.
-    const int tile = rows * chunk * 2;
+    // (output tile of 128 rows, K chunk of 32), the four slice tiles in the 64-byte-swizzled
+    // K-major layout the tensor cores read (8-row groups of 512 B; 16-byte chunk j of row r
+    // at position j ^ ((r / 2) mod 4)).
+    constexpr int rows = 128, chunk = 32, nq = 4, tile = rows * chunk * 2;
     const int nK = (n + chunk - 1) / chunk, nOut = (n + rows - 1) / rows;
-    const int nq = 4;
     TcFactor out;
     out.img.assign(size_t(nOut) * nK * nq * tile, 0);
     out.fscale.assign(size_t(nOut) * rows, 0.0f);
-    std::vector<double> slices(size_t(n) * n * 4, 0.0);
     for (int i = 0; i < n; ++i) {
         double rmax = 0.0;
         for (int k = 0; k < n; ++k) rmax = std::max(rmax, std::fabs(M[size_t(i) * n + k]));
         int e = 0;
         if (rmax > 0.0) std::frexp(rmax, &e);   // rmax < 2^e
         out.fscale[i] = static_cast<float>(std::ldexp(1.0, e - 7));
+        const int ot = i / rows, r = i % rows;
         for (int k = 0; k < n; ++k) {
-            const double y = std::ldexp(M[size_t(i) * n + k], 7 - e);
-            const double f0 = std::nearbyint(y);
-            const double y1 = (y - f0) * 256.0;
-            const double f1 = std::nearbyint(y1);
-            const double y2 = (y1 - f1) * 256.0;
-            const double f2 = std::nearbyint(y2);
-            const double f3 = std::nearbyint((y2 - f2) * 256.0);
-            double* sl = &slices[(size_t(i) * n + k) * 4];
-            if (precise || chunk == 32) {
-                sl[0] = f0; sl[1] = f1; sl[2] = f2; sl[3] = f3;
-            } else {
-                sl[0] = f0; sl[1] = f1; sl[2] = f1 / 256.0; sl[3] = f2 / 256.0;
+            const int c = k / chunk, j = k % chunk / 8, e2 = k % 8;
+            const size_t off = size_t((r >> 3) * 512 + (r & 7) * 64 + ((j ^ ((r >> 1) & 3)) << 4) + 2 * e2);
+            double y = std::ldexp(M[size_t(i) * n + k], 7 - e);
+            for (int q = 0; q < nq; ++q) {
+                const double f = std::nearbyint(y);
+                y = (y - f) * 256.0;
+                const uint16_t b = bf16_bits_exact(f);
+                uint8_t* t = &out.img[((size_t(ot) * nK + c) * nq + q) * tile];
+                t[off] = uint8_t(b & 0xFF);
+                t[off + 1] = uint8_t(b >> 8);
             }
         }
     }
-    for (int ot = 0; ot < nOut; ++ot)
-        for (int c = 0; c < nK; ++c)
-            for (int q = 0; q < nq; ++q) {
-                uint8_t* t = &out.img[((size_t(ot) * nK + c) * nq + q) * tile];
-                for (int r = 0; r < rows; ++r) {
-                    const int i = ot * rows + r;
-                    if (i >= n) continue;
-                    for (int j = 0; j < chunk / 8; ++j)
-                        for (int e2 = 0; e2 < 8; ++e2) {
-                            const int k = c * chunk + 8 * j + e2;
-                            if (k >= n) continue;
-                            const uint16_t b = bf16_bits_exact(slices[(size_t(i) * n + k) * 4 + q]);
-                            const size_t off = chunk == 64
-                                ? size_t((r >> 3) * 1024 + (r & 7) * 128 + ((j ^ (r & 7)) << 4) + 2 * e2)
-                                : size_t((r >> 3) * 512 + (r & 7) * 64 + ((j ^ ((r >> 1) & 3)) << 4) + 2 * e2);
-                            t[off] = uint8_t(b & 0xFF);
-                            t[off + 1] = uint8_t(b >> 8);
-                        }
-                }
-            }
     return out;
 }
 
