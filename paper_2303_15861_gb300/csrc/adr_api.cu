@@ -138,7 +138,7 @@ struct adr_ctx {
     uint8_t* d_img[kFactorKinds][3] = {{nullptr}};    // sliced image per factor kind and direction
     float* d_fsc[kFactorKinds][3] = {{nullptr}};
     float* d_zt[3] = {nullptr};            // tau * lambda_mu[j] (FP32)
-    float* d_phi32[3] = {nullptr, nullptr, nullptr};   // phi_k(tau (l1 + l2 + l3)) at the nodes, k = 0, 1, 2
+    float* d_phi32[3] = {nullptr, nullptr, nullptr};   // FP32 and mixed: phi_k(tau (l1 + l2 + l3)) at the nodes, k = 0, 1, 2
     unsigned* d_slots = nullptr;           // max-abs slots of the arrays a step produces
     int* d_err = nullptr;                  // device error word (bounded waits)
 
@@ -147,7 +147,7 @@ struct adr_ctx {
     bool f64tc = false;                    // ... and every factor is within its range
     uint8_t* d_img64[kFactorKinds][3] = {{nullptr}};
     int* d_rows64[kFactorKinds][3] = {{nullptr}};
-    double* d_phi64[3] = {nullptr, nullptr, nullptr};   // phi_k(tau (l1 + l2 + l3)) at the nodes, k = 0, 1, 2
+    double* d_phi64[3] = {nullptr, nullptr, nullptr};   // FP64 contexts: phi_k(tau (l1 + l2 + l3)) at the nodes, k = 0, 1, 2
 
     // batched 2-D instances (p.batch > 0)
     std::unique_ptr<adr_batch_state> bs;
@@ -341,10 +341,12 @@ ContractArgs<T> mode_args(const adr_ctx* c, int mu, const T* M, const T* X, T* Y
     if (mu == 1) {
         a.A = X; a.sam = n; a.sak = 1; a.sab = 0;
         a.B = M; a.sbk = 1; a.sbn = n; a.sbb = 0;    // B[k][j] = M[j][k]
+        a.factor = 2;
         a.C = Y; a.scm = n; a.scn = 1; a.scb = 0;
         a.M = int(P); a.N = n; a.K = n; a.batch = 1;
     } else {
         a.A = M; a.sam = n; a.sak = 1; a.sab = 0;
+        a.factor = 1;
         a.B = X; a.sbk = Q; a.sbn = 1; a.sbb = (long long)n * Q;
         a.C = Y; a.scm = Q; a.scn = 1; a.scb = (long long)n * Q;
         a.M = n; a.N = int(Q); a.K = n; a.batch = int(P);
@@ -474,6 +476,16 @@ const unsigned* Sched::consume(const void* buf) {
     return sl;
 }
 
+// The phi argument of a contraction's epilogue.
+template <typename T>
+void phi_fields(const adr_ctx* c, int phik, ContractArgs<T>& a) {
+    a.phik = phik;
+    a.ctau = c->p.tau;
+    for (int m = 0; m < 3; ++m) a.lam[m] = (m < c->dim) ? c->d_lam[m] : nullptr;
+    a.n1 = c->n[0];
+    a.n2 = c->n[1];
+}
+
 // FP64 context on the tensor cores: one mu-mode pass (contract_f64.cu).
 void push_mode_f64(Sched& S, int mu, int kind, const double* x, double* y, int epi, const double* base, double alpha, int phik) {
     const adr_ctx* c = S.c;
@@ -519,8 +531,12 @@ void push_mode(Sched& S, int mu, int kind, const T* x, T* y, int epi = adr::EPI_
     }
     if (!c->tc) {
         auto a = mode_args<T>(c, mu, static_cast<const T*>(dense_factor(c, kind, mu - 1)), x, y);
-        a.epi = epi; a.base = base; a.alpha = alpha; a.phik = phik; a.ctau = c->p.tau;
-        for (int m = 0; m < 3; ++m) a.lam[m] = (m < c->dim) ? c->d_lam[m] : nullptr;
+        a.epi = epi; a.base = base; a.alpha = alpha;
+        phi_fields(c, phik, a);
+        if (epi == adr::EPI_PHI) {
+            if constexpr (sizeof(T) == 8) a.phi = c->d_phi64[phik];
+            else a.phi = c->d_phi32[phik];
+        }
         S.ops.push_back({[a](cudaStream_t s) { return adr::launch_contract(a, s); }, OP_CONTRACT_SIMT});
         return;
     }
@@ -2028,25 +2044,28 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
             c->phi_route = ADR_PHI_DOUBLING;
         } else {
             c->phi_route = ADR_PHI_EIGEN;
-            // the phi factors at the nodes: evaluated in the contraction's epilogue they would take
-            // longer than the contraction
-            for (int k = 1; k <= 2 && c->f64tc; ++k) {
-                if (!c->d_phi64[k]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_phi64[k]), c->N * sizeof(double));
-                if (e == cudaSuccess)
-                    e = adr::launch_f64_phi(c->d_phi64[k], k, c->p.tau, c->d_lam, c->n[0], c->n[1], c->N, nullptr);
-                if (e != cudaSuccess) return cuda_fail(c, e, "phi tables");
+            // the phi factors at the nodes: evaluated in a contraction's epilogue they take longer than
+            // the contraction (FP64: 40 to 60 instructions a node; the series near 0 in every precision)
+            for (int k = 1; k <= 2 && e == cudaSuccess; ++k) {
+                if (c->fp64) {
+                    if (!c->d_phi64[k]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_phi64[k]), c->N * sizeof(double));
+                    ContractArgs<double> a;
+                    phi_fields(c, k, a);
+                    if (e == cudaSuccess) e = adr::launch_phi_nodes(c->d_phi64[k], a, c->N, nullptr);
+                } else {
+                    if (!c->d_phi32[k]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_phi32[k]), c->N * sizeof(float));
+                    ContractArgs<float> a;
+                    phi_fields(c, k, a);
+                    if (e == cudaSuccess)
+                        e = c->tc ? adr::launch_phi_table(c->d_phi32[k], k, c->d_zt, c->n[0], c->n[1], c->N, nullptr)
+                                  : adr::launch_phi_nodes(c->d_phi32[k], a, c->N, nullptr);
+                }
             }
-            for (int k = 1; k <= 2 && c->tc; ++k) {
-                if (!c->d_phi32[k]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_phi32[k]), c->N * sizeof(float));
-                if (e == cudaSuccess) e = adr::launch_phi_table(c->d_phi32[k], k, c->d_zt, c->n[0], c->n[1], c->N, nullptr);
-                if (e != cudaSuccess) return cuda_fail(c, e, "phi tables");
-            }
+            if (e != cudaSuccess) return cuda_fail(c, e, "phi tables");
         }
     }
-    if (c->f64tc || c->tc) {               // the kernels above ran on the legacy stream
-        e = cudaStreamSynchronize(nullptr);
-        if (e != cudaSuccess) return cuda_fail(c, e, "cut factors");
-    }
+    e = cudaStreamSynchronize(nullptr);    // the kernels above ran on the legacy stream
+    if (e != cudaSuccess) return cuda_fail(c, e, "set_coeffs");
     c->coeffs_set = true;
     return ADR_OK;
 }

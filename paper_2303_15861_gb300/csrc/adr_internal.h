@@ -126,6 +126,8 @@ struct ContractArgs {
     int epi = EPI_STORE;
     const T* base = nullptr;  // EPI_AXPY: C = base + alpha * acc
     double alpha = 0;
+    int factor = 0;           // 1: A, 2: B is a context's factor, complete before any launch (0: neither is known to be)
+    const T* phi = nullptr;   // EPI_PHI: phi_k at the nodes, or NULL with the fields below
     int phik = 1;             // EPI_PHI: C = phi_k(ctau * (l1[i1]+l2[i2]+l3[i3])) * acc
     double ctau = 0;
     const double* lam[3] = {nullptr, nullptr, nullptr};
@@ -194,7 +196,6 @@ cudaError_t launch_contract_f64(F64Args a, cudaStream_t s);
 size_t f64_image_bytes(int n);
 int f64_rows(int n);                 // rows of the image (n rounded up to whole tiles)
 cudaError_t launch_f64_factor(const double* M, int n, uint8_t* img, int* rows, cudaStream_t s);
-cudaError_t launch_f64_phi(double* tab, int k, double ctau, const double* const lam[3], int n1, int n2, size_t N, cudaStream_t s);
 
 // Host: slice an FP64 factor into the tensor-core image: per output tile of 128 rows and K chunk of 32, the slice
 // tiles F0..F3 in the 64-byte-swizzled K-major layout.
@@ -212,6 +213,9 @@ cudaError_t launch_f64_faces(const double* a, double* w, double inv_h2, long lon
 cudaError_t launch_stencil(const StencilArgs<float>& a, cudaStream_t s);
 cudaError_t launch_contract(const ContractArgs<double>& a, cudaStream_t s);
 cudaError_t launch_contract(const ContractArgs<float>& a, cudaStream_t s);
+// The phi factor of every node, as an EPI_PHI epilogue of p without a table evaluates it.
+cudaError_t launch_phi_nodes(double* tab, const ContractArgs<double>& p, size_t N, cudaStream_t s);
+cudaError_t launch_phi_nodes(float* tab, const ContractArgs<float>& p, size_t N, cudaStream_t s);
 cudaError_t launch_convert_f64_to_f32(const double* in, float* out, size_t n, cudaStream_t s);
 
 // ---------------------------------------------------------------- batched 2-D instances

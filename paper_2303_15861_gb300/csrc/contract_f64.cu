@@ -556,15 +556,6 @@ __global__ void f64_factor_kernel(const double* M, int n, int nK, uint8_t* img, 
     }
 }
 
-__global__ void f64_phi_kernel(double* tab, int k, double ctau, const double* l1, const double* l2, const double* l3, int n1,
-                               int n2, size_t N) {
-    for (size_t o = blockIdx.x * size_t(blockDim.x) + threadIdx.x; o < N; o += size_t(gridDim.x) * blockDim.x) {
-        double ls = l1[o % n1] + l2[(o / n1) % n2];
-        if (l3) ls += l3[o / n1 / n2];
-        tab[o] = phi_eval(k, ctau * ls);
-    }
-}
-
 int sm_count() {
     static const int sms = [] {
         int dev = 0, v = 0;
@@ -599,12 +590,6 @@ int f64_rows(int n) { return (n + kM - 1) / kM * kM; }
 
 cudaError_t launch_f64_factor(const double* M, int n, uint8_t* img, int* rows, cudaStream_t s) {
     f64_factor_kernel<<<f64_rows(n), 128, 0, s>>>(M, n, (n + kKc - 1) / kKc, img, rows);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_f64_phi(double* tab, int k, double ctau, const double* const lam[3], int n1, int n2, size_t N, cudaStream_t s) {
-    const unsigned blocks = unsigned((N + 255) / 256 < 65535 ? (N + 255) / 256 : 65535);
-    f64_phi_kernel<<<blocks, 256, 0, s>>>(tab, k, ctau, lam[0], lam[1], lam[2], n1, n2, N);
     return cudaGetLastError();
 }
 

@@ -15,6 +15,7 @@
 #include <cstdint>
 
 #include "adr_internal.h"
+#include "launch.cuh"
 #include "stencil_core.cuh"
 
 namespace adr {
@@ -31,6 +32,7 @@ constexpr int ZCHUNK = 4;   // x3 planes per thread
 // by L1, x3 neighbours by registers. DIM = 2 has one plane and no x3 terms.
 template <typename T, int DIM, int ZC, bool HASLO>
 __global__ void __launch_bounds__(TX * TY) stencil_kernel(StencilArgs<T> p, Coefs<T> c, bool needF) {
+    pdl_trigger();
     const int n1 = p.n1, n2 = p.n2, n3 = p.n3;
     const int A1 = p.apitch, A2 = n2 + 2;
     const long long plane_u = (long long)n1 * n2;
@@ -148,6 +150,7 @@ __device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret
 
 template <int DIM, bool HASLO>
 __global__ void __launch_bounds__(256) stencil_vec4_kernel(StencilArgs<float> p, Coefs<float> c, bool needF) {
+    pdl_trigger();
     const int n1 = p.n1, n2 = p.n2, n3 = p.n3;
     const int A1 = p.apitch, A2 = n2 + 2;
     const long long plane_u = (long long)n1 * n2;
@@ -277,6 +280,7 @@ __global__ void __launch_bounds__(256) stencil_vec4_kernel(StencilArgs<float> p,
 // (L1/L2 hits).
 template <bool HASLO, int NX, int NOUT>
 __global__ void __launch_bounds__(256, HASLO ? 2 : 3) stencil_march_kernel(StencilArgs<float> p, Coefs<float> c, bool needF, int zb) {
+    pdl_trigger();
     const int n1 = p.n1, n2 = p.n2, n3 = p.n3;
     const int A1 = p.apitch, A2 = n2 + 2;
     const long long plane_u = (long long)n1 * n2;

@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "adr_internal.h"
+#include "launch.cuh"
 #include "stencil_core.cuh"
 
 namespace adr {
@@ -64,6 +65,7 @@ __global__ void __launch_bounds__(kTX * kTY) stencil_f64_kernel(StencilArgs<doub
     const int n1 = p.n1, n2 = p.n2, n3 = DIM == 3 ? p.n3 : 1;
     const int i1 = (int(blockIdx.x) * kTX + int(threadIdx.x % kTX)) * V;
     const int i2 = int(blockIdx.y) * int(blockDim.x / kTX) + int(threadIdx.x / kTX);
+    pdl_trigger();
     if (i1 >= n1 || i2 >= n2) return;                        // V = 2: n1 is even
     const long long plane_u = (long long)n1 * n2, plane_a = (long long)p.apitch * (n2 + 2);
     const int z0 = DIM == 3 ? int(blockIdx.z) * zb : 0, z1 = DIM == 3 ? min(z0 + zb, n3) : 1;
