@@ -250,8 +250,7 @@ adr_status adr_get_instance_info(const adr_ctx* ctx, int instance, double kappa[
  * by batch_tile), for mode 1 (contraction along x1) or mode 2: the tile edge (32, 64 or
  * 128) of every instance in tile_edge[0..batch-1] (may be NULL) and the number of
  * persistent CTAs of the launch in *grid (may be NULL). Mixed batched contexts report their
- * tensor-core tiles' output extent: 128 in mode 1, 64 in mode 2. ADR_ERR_STATE before every
- * instance is set; ADR_ERR_ARG for a single-grid context. */
+ * tensor-core tiles' output extent, 128. ADR_ERR_STATE before every instance is set; ADR_ERR_ARG for a single-grid context. */
 adr_status adr_get_batch_plan(const adr_ctx* ctx, int mode, int* tile_edge, int* grid);
 
 /* One adr_step with a CUDA event recorded on the context stream around every enqueued

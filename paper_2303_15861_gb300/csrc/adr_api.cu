@@ -1348,9 +1348,9 @@ cudaError_t batch_mixed_instance(adr_ctx* c, int i) {
         for (int m = 0; m < 2 && e == cudaSuccess; ++m) {
             if (!b.roles[r]) continue;
             const double* M = &b.hF[size_t(b.f_off[size_t(i) * 2 * adr::kBatchRoles + r * 2 + m])];
-            img.assign(adr::batch_tc_image_bytes(n[m], m + 1), 0);
+            img.assign(adr::batch_tc_image_bytes(n[m], 1), 0);   // 128-row tiles in both directions
             fsc.assign(size_t(n[m]), 0.0f);
-            adr::make_batch_tc_factor(M, n[m], m + 1, img.data(), fsc.data());
+            adr::make_batch_tc_factor(M, n[m], 1, img.data(), fsc.data());
             e = cudaMemcpy(b.d_img + t.img_off[r][m], img.data(), img.size(), cudaMemcpyHostToDevice);
             if (e == cudaSuccess)
                 e = cudaMemcpy(b.d_fsc + t.fsc_off[r][m], fsc.data(), fsc.size() * sizeof(float), cudaMemcpyHostToDevice);
@@ -1373,8 +1373,7 @@ cudaError_t batch_mixed_instance(adr_ctx* c, int i) {
 
 // Mixed batched context, once every instance is set: the instance table and the work items of
 // the tensor-core passes, instances in order of decreasing size (longest-processing-time order
-// for the persistent CTAs that take items round robin). Mode 1: 64-row x2 tiles x 128 outputs
-// along x1; mode 2: 128-position x1 tiles x 64 outputs along x2.
+// for the persistent CTAs that take items round robin): 64 lines x 128 outputs.
 cudaError_t batch_mixed_plan(adr_ctx* c) {
     adr_batch_state& b = *c->bs;
     cudaError_t e = cudaMemcpy(b.d_tci, b.tci.data(), b.tci.size() * sizeof(adr::BatchTcInst), cudaMemcpyHostToDevice);
@@ -1387,8 +1386,8 @@ cudaError_t batch_mixed_plan(adr_ctx* c) {
         std::vector<int4> items;
         for (int i : order) {
             const int n1 = b.n1[i], n2 = b.n2[i];
-            const int npt = mode == 1 ? (n2 + 63) / 64 : (n1 + 127) / 128;
-            const int nout = mode == 1 ? (n1 + 127) / 128 : (n2 + 63) / 64;
+            const int npt = ((mode == 1 ? n2 : n1) + 63) / 64;
+            const int nout = ((mode == 1 ? n1 : n2) + 127) / 128;
             for (int pt = 0; pt < npt; ++pt)
                 for (int ot = 0; ot < nout; ++ot) items.push_back(make_int4(i, pt, ot, 0));
         }
@@ -1491,7 +1490,7 @@ adr_status create_batch(const adr_params* p, void* cuda_stream, adr_ctx** out) {
                     if (!b.roles[r]) continue;
                     const int nm = m == 0 ? n1 : n2;
                     t.img_off[r][m] = img_len;
-                    img_len += (long long)adr::batch_tc_image_bytes(nm, m + 1);
+                    img_len += (long long)adr::batch_tc_image_bytes(nm, 1);
                     t.fsc_off[r][m] = fsc_len;
                     fsc_len += (nm + 3) / 4 * 4;
                 }
@@ -2355,8 +2354,8 @@ adr_status adr_get_batch_plan(const adr_ctx* c, int mode, int* tile_edge, int* g
     const adr_batch_state& b = *c->bs;
     if (!b.tuned) return ADR_ERR_STATE;
     if (tile_edge)
-        for (int i = 0; i < b.B; ++i)   // mixed: the tensor-core tiles' output extent (128 along x1, 64 along x2)
-            tile_edge[i] = b.mixed ? (mode == 1 ? 128 : 64) : adr::batch_tile_edge(b.tile[mode - 1][i]);
+        for (int i = 0; i < b.B; ++i)   // mixed: the tensor-core tiles' output extent
+            tile_edge[i] = b.mixed ? 128 : adr::batch_tile_edge(b.tile[mode - 1][i]);
     if (grid) *grid = b.grid[mode - 1];
     return ADR_OK;
 }

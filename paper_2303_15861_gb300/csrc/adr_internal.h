@@ -316,8 +316,8 @@ struct BatchTcInst {
 };
 
 // One mu-mode pass over every instance on the tensor cores. items[i] = {instance, position
-// tile, output tile, 0}: mode 1 (Y_i = X_i M^T, K = n1): 64 rows (x2 fibres) x 128 outputs;
-// mode 2 (Y_i = M X_i, K = n2): 128 positions (x1) x 64 outputs. Inputs and outputs are
+// tile, output tile, 0}: 64 lines (mode 1, Y_i = X_i M^T, K = n1: x2 rows; mode 2, Y_i = M X_i, K = n2: x1
+// positions) x 128 outputs. Inputs and outputs are
 // double-float pairs (a NULL low part reads as zero / is not written).
 //   EPI_STORE: Y (+ Ylo) = the product;  EPI_PHI (mode 2): times the double-float table
 //   phi = (hi, lo) pairs, one per node of the instance;  EPI_AXPY: base (+ base_lo) + alpha
@@ -345,11 +345,12 @@ struct BatchTcArgs {
     unsigned* amax_out = nullptr;
     int* err = nullptr;
     int grid = 0;
+    bool al16 = false;               // set by the launcher: the arrays start on 16 bytes
 };
-cudaError_t launch_batch_tc(const BatchTcArgs& a, cudaStream_t s);
+cudaError_t launch_batch_tc(BatchTcArgs a, cudaStream_t s);
 // Bytes of the sliced image of an n x n factor in a pass of the given mode, and the host
 // slicing: per (output tile, K chunk of 32), seven 64-byte-swizzled K-major BF16 tiles
-// F0, F1, F2, F3, 2^-8 F1, 2^-8 F2, 2^-8 F3 of 64 (mode 2) or 128 (mode 1) rows; row i of
+// F0, F1, F2, F3, 2^-8 F1, 2^-8 F2, 2^-8 F3 of 64 (mode 2) or 128 (mode 1) rows (batch_tc.cu takes 128 rows in both modes); row i of
 // the factor is 2^(e_i-7) sum_j 2^(-8j) F_j with integer |F_j| <= 128.
 constexpr int kBatchTcRows1 = 128;         // output rows of a mode-1 factor tile (UMMA M)
 constexpr int kBatchTcRows2 = 64;          // output rows of a mode-2 factor tile (UMMA N)

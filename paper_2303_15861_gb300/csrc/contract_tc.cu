@@ -94,9 +94,6 @@ __device__ __forceinline__ void tmem_ld8x4(uint32_t t0, uint32_t stride, float (
         for (int j = 0; j < 8; ++j) d[k][j] = __uint_as_float(r[8 * k + j]);
 }
 
-// Round to the nearest integer (|y| < 2^22) by two additions; a rounding instruction runs at an eighth of their rate.
-__device__ __forceinline__ float rint_small(float y) { return (y + 12582912.f) - 12582912.f; }
-
 // Integer slices of y + ylo: the residuals y - s0 and y1 - s1 are exact, and the low part enters once,
 // after the leading slice.
 __device__ __forceinline__ void split(float y, float ylo, float (&s)[kSl]) {
@@ -133,24 +130,6 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
     const float bb = s - a;
     e = (a - (s - bb)) + (b - bb);
-}
-
-// Loads that stay where they are written (the compiler sinks plain ones to their first use), 0 where `on` is false.
-__device__ __forceinline__ float ld1_or_0(const float* p, bool on) {
-    float v;
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %2, 0;\n mov.b32 %0, 0;\n @p ld.global.nc.f32 %0, [%1];\n}\n"
-                 : "=f"(v)
-                 : "l"(p), "r"(int(on)));
-    return v;
-}
-__device__ __forceinline__ float4 ld4_or_0(const float* p, bool on) {
-    float4 v;
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %5, 0;\n mov.b32 %0, 0;\n mov.b32 %1, 0;\n mov.b32 %2, 0;\n mov.b32 %3, 0;\n"
-        " @p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n}\n"
-        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-        : "l"(p), "r"(int(on)));
-    return v;
 }
 
 // 32-byte (256-bit) accesses: eight consecutive floats.

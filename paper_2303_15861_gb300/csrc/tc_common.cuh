@@ -86,6 +86,27 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint4 v) {
                  : "memory");
 }
 
+// Round to the nearest integer (|y| < 2^22) by two additions; a rounding instruction runs at an eighth of their rate.
+__device__ __forceinline__ float rint_small(float y) { return (y + 12582912.f) - 12582912.f; }
+
+// Loads that stay where they are written (the compiler sinks plain ones to their first use), 0 where `on` is false.
+__device__ __forceinline__ float ld1_or_0(const float* p, bool on) {
+    float v;
+    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %2, 0;\n mov.b32 %0, 0;\n @p ld.global.nc.f32 %0, [%1];\n}\n"
+                 : "=f"(v)
+                 : "l"(p), "r"(int(on)));
+    return v;
+}
+__device__ __forceinline__ float4 ld4_or_0(const float* p, bool on) {
+    float4 v;
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %5, 0;\n mov.b32 %0, 0;\n mov.b32 %1, 0;\n mov.b32 %2, 0;\n mov.b32 %3, 0;\n"
+        " @p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n}\n"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+        : "l"(p), "r"(int(on)));
+    return v;
+}
+
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
