@@ -85,6 +85,7 @@ struct adr_batch_state {
     int4* d_items[2] = {nullptr, nullptr};
     int nitems[2] = {0, 0};
     int grid[2] = {0, 0};                  // persistent CTAs of the contraction, per mode
+    int max_tile[2] = {adr::BT_128, adr::BT_128};   // the largest tile shape among the items
     int sgrid = 0;                         // persistent CTAs of the stencil
     std::vector<int> tile[2];              // BatchTile per instance, per mode
     bool uploaded = false, tuned = false;
@@ -414,6 +415,7 @@ void push_mode_batch(Sched& S, int mu, int kind, const T* x, T* y, int epi, cons
     a.inst = static_cast<const adr::BatchInst<T>*>(b.d_inst);
     a.items = b.d_items[mu - 1];
     a.nitems = b.nitems[mu - 1];
+    a.max_tile = b.max_tile[mu - 1];
     a.mode = mu;
     a.role = kind == FK_EXP_ALPHA ? adr::BR_EXP_ALPHA : kind;
     a.factors = static_cast<const T*>(b.d_f);
@@ -1191,8 +1193,8 @@ void append_items(const adr_batch_state& b, const std::vector<int>& insts, int t
 // Autotuner. Per instance size (n1, n2) and mode it times each candidate tile shape on the
 // items of that size class and keeps the fastest; the full item list of a mode is then
 // ordered by the measured cost per item, largest first (longest-processing-time order for
-// the persistent CTAs that take items round robin); last it times the full list at 1-4
-// CTAs per SM, and the stencil at 4, 8 and 16 CTAs per SM.
+// the persistent CTAs that take items round robin); last it times the full list at 1 CTA per SM up to what
+// an SM holds (at least 4), and the stencil at 4, 8 and 16 CTAs per SM.
 template <typename T>
 adr_status batch_tune(adr_ctx* c) {
     adr_batch_state& b = *c->bs;
@@ -1244,8 +1246,10 @@ adr_status batch_tune(adr_ctx* c) {
     base.X = static_cast<const T*>(c->ws[0]);
     base.Y = static_cast<T*>(c->ws[1]);
     base.epi = adr::EPI_STORE;
+    auto resident = [&](int t) { return adr::batch_contract_blocks_per_sm(t, sizeof(T) == 8) * sms; };
     for (int mode = 1; mode <= 2 && e == cudaSuccess; ++mode) {
         std::vector<std::pair<double, int4>> all;
+        int max_tile = adr::BT_32;
         for (const auto& cl : classes) {
             int best_t = b.tile_force >= 0 ? b.tile_force : adr::BT_64;
             float best_ms = 1e30f;
@@ -1258,14 +1262,16 @@ adr_status batch_tune(adr_ctx* c) {
                 a.items = d_tmp;
                 a.nitems = int(items.size());
                 a.mode = mode;
-                a.grid = std::min(int(items.size()), 2 * sms);
+                a.max_tile = t;
+                a.grid = std::min(int(items.size()), resident(t));
                 float ms = 0.f;
                 if (e == cudaSuccess) e = best_of([a](cudaStream_t s) { return adr::launch_batch_contract(a, s); }, ms);
                 if (e == cudaSuccess && ms < best_ms) { best_ms = ms; best_t = t; }
             }
             std::vector<int4> items;
             append_items(b, cl.second, best_t, items);
-            const double g = double(std::min(int(items.size()), 2 * sms));
+            const double g = double(std::min(int(items.size()), resident(best_t)));
+            max_tile = std::max(max_tile, best_t);
             const double per_item = double(best_ms) * g / double(items.size());
             for (int i : cl.second) b.tile[mode - 1][i] = best_t;
             for (const auto& it : items) all.push_back({per_item, it});
@@ -1283,9 +1289,11 @@ adr_status batch_tune(adr_ctx* c) {
             e = cudaMemcpy(b.d_items[mode - 1], items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice);
         b.nitems[mode - 1] = int(items.size());
         float best_ms = 1e30f;
-        b.grid[mode - 1] = std::min(b.nitems[mode - 1], 2 * sms);
-        for (int per_sm = 1; per_sm <= 4 && e == cudaSuccess; ++per_sm) {
+        b.max_tile[mode - 1] = max_tile;
+        b.grid[mode - 1] = std::min(b.nitems[mode - 1], resident(max_tile));
+        for (int per_sm = 1; per_sm <= std::max(4, resident(max_tile) / sms) && e == cudaSuccess; ++per_sm) {
             auto a = base;
+            a.max_tile = max_tile;
             a.items = b.d_items[mode - 1];
             a.nitems = b.nitems[mode - 1];
             a.mode = mode;

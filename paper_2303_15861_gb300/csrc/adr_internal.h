@@ -288,9 +288,11 @@ struct BatchContractArgs {
     double alpha = 0;
     int phik = 1;
     bool aligned = false;          // X, Y (and base) 16-byte aligned: vector loads where vec
+    int max_tile = BT_128;         // the largest tile shape among the items
     int grid = 0;
 };
 
+int batch_contract_blocks_per_sm(int max_tile, bool fp64);
 cudaError_t launch_batch_stencil(const BatchStencilArgs<double>& a, cudaStream_t s);
 cudaError_t launch_batch_stencil(const BatchStencilArgs<float>& a, cudaStream_t s);
 cudaError_t launch_batch_contract(const BatchContractArgs<double>& a, cudaStream_t s);

@@ -303,12 +303,11 @@ __global__ void __launch_bounds__(256) batch_stencil2_march_kernel(BatchStencil2
 constexpr int kThreads = 256;      // 16 x 16 threads per tile of every shape
 constexpr int kBK = 16;            // K per shared-memory stage
 constexpr int kPad = 4;            // row padding: keeps 16-byte alignment of 4-wide groups
-constexpr int kMaxEdge = 128;
 
-template <typename T>
+template <typename T, int MAXE>
 struct TileSmem {
-    alignas(16) T A[kBK][kMaxEdge + kPad];   // A^T slice: [k][m]
-    alignas(16) T B[kBK][kMaxEdge + kPad];   // B slice:   [k][n]
+    alignas(16) T A[kBK][MAXE + kPad];       // A^T slice: [k][m]
+    alignas(16) T B[kBK][MAXE + kPad];       // B slice:   [k][n]
 };
 
 // G consecutive values from shared or global memory (16-byte aligned when G * sizeof(T) >= 16).
@@ -385,7 +384,8 @@ struct Slice {
         }
     }
 
-    __device__ __forceinline__ void store(T (*S)[kMaxEdge + kPad]) const {
+    template <int PITCH>
+    __device__ __forceinline__ void store(T (*S)[PITCH]) const {
         const int tid = threadIdx.x;
         if constexpr (VEC) {
 #pragma unroll
@@ -421,8 +421,8 @@ __device__ __noinline__ T phi_factor(int k, T z) { return phi_eval(k, z); }
 // A(m, k) = A[m * sam + k]; B(k, n) = B[n * sb + k] in mode 1 (the factor, k contiguous)
 // and B[k * sb + n] in mode 2 (the state, n contiguous). A thread owns TM x TM outputs in
 // groups of G consecutive rows and columns: row (i / G) * 16G + ty G + i % G.
-template <typename T, int E, int MODE, bool VEC>
-__device__ __forceinline__ void tile_gemm(TileSmem<T>& sm, const T* __restrict__ A, long long sam,
+template <typename T, int E, int MODE, bool VEC, int MAXE>
+__device__ __forceinline__ void tile_gemm(TileSmem<T, MAXE>& sm, const T* __restrict__ A, long long sam,
                                           const T* __restrict__ B, long long sb, int M, int N, int K, int m0, int n0,
                                           const BatchContractArgs<T>& p, const BatchInst<T>& in) {
     constexpr int TM = E / 16;
@@ -514,9 +514,17 @@ __device__ __forceinline__ void tile_gemm(TileSmem<T>& sm, const T* __restrict__
     }
 }
 
-template <typename T, int MODE>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1) batch_contract_kernel(BatchContractArgs<T> p) {
-    __shared__ TileSmem<T> sm;
+// Blocks that an SM holds of the kernel for tiles up to MAXE: what bounds a tile is the latency of its stages of 16 of K
+// (the next one in flight during 16 x TM^2 FMAs), so the registers and shared memory that only larger
+// tiles need are left to more blocks.
+// One kernel for all three shapes (two blocks per SM in FP32, one in FP64) -> these, same bits: 96 instances of 24 to 160 nodes
+// a direction, Lawson4 FP32, six steps on each of three streams 1112 -> 781 us; 200 of 24 to 120, Lawson2a FP64 11.07 ->
+// 9.50 ms; 40 of 100 to 250, Lawson4 FP64 28.9 -> 26.3 ms.
+constexpr int blocks_per_sm(int maxe, bool fp64) { return maxe == 32 ? (fp64 ? 4 : 6) : maxe == 64 ? (fp64 ? 2 : 4) : (fp64 ? 1 : 2); }
+
+template <typename T, int MODE, int MAXE>
+__global__ void __launch_bounds__(kThreads, blocks_per_sm(MAXE, sizeof(T) == 8)) batch_contract_kernel(BatchContractArgs<T> p) {
+    __shared__ TileSmem<T, MAXE> sm;
     for (int it = blockIdx.x; it < p.nitems; it += gridDim.x) {
         const int4 item = __ldg(p.items + it);
         const BatchInst<T>& in = p.inst[item.x];
@@ -532,12 +540,14 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1) batch_contra
         const long long sb = n1;
         const int K = MODE == 1 ? n1 : n2;
         const bool vec = in.vec && p.aligned;
-        if (item.w == BT_32) {
+        if (MAXE == 32 || item.w == BT_32) {
             tile_gemm<T, 32, MODE, false>(sm, A, sam, B, sb, n2, n1, K, m0, n0, p, in);
-        } else if (item.w == BT_64) {
-            if (vec) tile_gemm<T, 64, MODE, true>(sm, A, sam, B, sb, n2, n1, K, m0, n0, p, in);
-            else     tile_gemm<T, 64, MODE, false>(sm, A, sam, B, sb, n2, n1, K, m0, n0, p, in);
-        } else {
+        } else if (MAXE == 64 || item.w == BT_64) {
+            if constexpr (MAXE >= 64) {
+                if (vec) tile_gemm<T, 64, MODE, true>(sm, A, sam, B, sb, n2, n1, K, m0, n0, p, in);
+                else     tile_gemm<T, 64, MODE, false>(sm, A, sam, B, sb, n2, n1, K, m0, n0, p, in);
+            }
+        } else if constexpr (MAXE >= 128) {
             if (vec) tile_gemm<T, 128, MODE, true>(sm, A, sam, B, sb, n2, n1, K, m0, n0, p, in);
             else     tile_gemm<T, 128, MODE, false>(sm, A, sam, B, sb, n2, n1, K, m0, n0, p, in);
         }
@@ -584,8 +594,12 @@ cudaError_t contract_launch(const BatchContractArgs<T>& p, cudaStream_t s) {
     if (p.epi == EPI_AXPY && !p.base) return cudaErrorInvalidValue;
     long long grid = p.grid > 0 ? p.grid : 2LL * sm_count();
     if (grid > p.nitems) grid = p.nitems;
-    if (p.mode == 1) batch_contract_kernel<T, 1><<<unsigned(grid), kThreads, 0, s>>>(p);
-    else             batch_contract_kernel<T, 2><<<unsigned(grid), kThreads, 0, s>>>(p);
+    const bool m1 = p.mode == 1;
+    switch (p.max_tile) {
+    case BT_32: (m1 ? batch_contract_kernel<T, 1, 32> : batch_contract_kernel<T, 2, 32>)<<<unsigned(grid), kThreads, 0, s>>>(p); break;
+    case BT_64: (m1 ? batch_contract_kernel<T, 1, 64> : batch_contract_kernel<T, 2, 64>)<<<unsigned(grid), kThreads, 0, s>>>(p); break;
+    default: (m1 ? batch_contract_kernel<T, 1, 128> : batch_contract_kernel<T, 2, 128>)<<<unsigned(grid), kThreads, 0, s>>>(p); break;
+    }
     return cudaGetLastError();
 }
 
@@ -631,5 +645,6 @@ cudaError_t launch_batch_stencil(const BatchStencilArgs<float>& a, cudaStream_t 
 cudaError_t launch_batch_contract(const BatchContractArgs<double>& a, cudaStream_t s) { return contract_launch(a, s); }
 cudaError_t launch_batch_contract(const BatchContractArgs<float>& a, cudaStream_t s) { return contract_launch(a, s); }
 cudaError_t launch_batch_stencil2(const BatchStencil2Args& a, cudaStream_t s) { return stencil2_launch(a, s); }
+int batch_contract_blocks_per_sm(int max_tile, bool fp64) { return blocks_per_sm(batch_tile_edge(max_tile), fp64); }
 
 }  // namespace adr
