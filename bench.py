@@ -35,7 +35,7 @@ UNIT = "DOF*steps/s"
 
 
 def split_products(ctx):
-    """BF16 products per multiply-add of the TMA-fed tensor-core contraction: four state slices
+    """BF16 products per multiply-add of the mixed tensor-core contraction: four state slices
     against four factor slices, the products below 2^-24 left out (ten)."""
     return {4: 10.0}[ctx.tc_factor_slices()]
 
@@ -66,11 +66,11 @@ def parse():
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per standard pass of the
 # tensor-core contraction at 256^3, averaged over the six standard passes of the second step
-# of `python bench.py --ncu-steps 2` (ncu -k regex:tma_contract -s 12 -c 6). The figure holds only for the
+# of `python bench.py --ncu-steps 2` (ncu -k regex:tc_contract -s 12 -c 6). The figure holds only for the
 # kernel source it was taken from, identified by the hash below; after any change to that
 # source the bench reports null until the kernel is captured again.
-_TRAFFIC_CAPTURE = {"n": 256, "bytes_per_launch": 86.1e6,
-                    "source_sha256": "78dffd3a19003a8c961d823307beb2ea5ce7aebd44e43612de628f34843851e9"}
+_TRAFFIC_CAPTURE = {"n": 256, "bytes_per_launch": 88.3e6,
+                    "source_sha256": "b13d598ee28cbbca751feaf66f3c27e5c8f66c8b37b4880253b71b0b9ff4d8f0"}
 _TRAFFIC_SOURCES = ("paper_2303_15861_gb300/csrc/contract_tc.cu", "paper_2303_15861_gb300/csrc/tc_common.cuh",
                     "paper_2303_15861_gb300/csrc/host_setup.cpp")
 
@@ -353,7 +353,7 @@ def ours(args):
         tflops = flops / (tc_ms * 1e-3) / 1e12
         roof = {"bound": "tensor", "achieved": tflops, "peak": bf16_peak, "unit": "TFLOP/s",
                 "frac": tflops / bf16_peak, "traffic": _captured_traffic(n),
-                "kernel": "tma_contract_kernel standard pass (mu-mode contraction, TMA-fed tcgen05 kind::f16)",
+                "kernel": "tc_contract_kernel standard pass (mu-mode contraction, tcgen05 kind::f16)",
                 "algorithmic_flops_per_launch": flops, "launch_ms": tc_ms,
                 "issued_bf16_tflops": products * tflops, "issued_frac": products * tflops / bf16_peak,
                 "products_per_multiply_add": products, "hbm_gbs": hbm_gbs, "hbm_frac": hbm_gbs / hbm_peak,
@@ -585,17 +585,17 @@ def ours_grid(args):
         # N-point transform (5 N log2 N flops each), the complex product (6 N) and the epilogue
         # (2 N). The state is L2-resident at this size, so the bound is arithmetic: the FP64 pipe
         # in FP64, otherwise latency (reported against the FP32 lanes).
-        # A stage kept in Fourier space (2-D; four or five launches) takes seven
-        # complex N-point transforms (u forward, two derivatives back, two fluxes and the
-        # pointwise part forward, the result back), 35 N log2 N flops, and about 50 N pointwise.
+        # A stage kept in Fourier space (2-D; four or five launches) takes seven N-point transforms of real data (u
+        # forward, two derivatives back, two fluxes and the pointwise part forward, the result back), half the work of
+        # complex ones: 17.5 N log2 N flops, and about 50 N pointwise.
         peak, src = alu_peak(prec)
         if 8 in kinds:
             c_ms = statistics.mean(kinds[8])
-            flops = 35.0 * N * math.log2(N) + 50.0 * N
+            flops = 17.5 * N * math.log2(N) + 50.0 * N
             kname = "Fourier-space stage (four or five fourier_pass_kernel launches)"
         else:
             c_ms = statistics.mean(kinds.get(7, [float("nan")]))
-            flops = 10.0 * N * math.log2(N) + 8.0 * N
+            flops = 5.0 * N * math.log2(N) + 8.0 * N
             kname = "Fourier multiplier (three fourier_pass_kernel launches)"
         ach = flops / (c_ms * 1e-3) / 1e12
         roof = {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
@@ -607,9 +607,18 @@ def ours_grid(args):
             peak = json.load(f)["bf16_tflops_sustained"]
         ach = 2.0 * n * N / (c_ms * 1e-3) / 1e12      # algorithmic: 2 n flops per element per pass
         roof = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-                "traffic": None, "kernel": "tma_contract_kernel standard pass", "launch_ms": c_ms,
+                "traffic": None, "kernel": "tc_contract_kernel standard pass", "launch_ms": c_ms,
                 "issued_frac": products * ach / peak, "products_per_multiply_add": products,
                 "peak_source": "measured bf16 sustained"}
+    elif prec == "fp64" and kinds.get(4):
+        # seven BF16 digits per operand, 28 products per FP64 multiply-add
+        c_ms = statistics.mean(kinds[4])
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            peak = json.load(f)["bf16_tflops_sustained"]
+        ach = 2.0 * n * N / (c_ms * 1e-3) / 1e12
+        roof = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
+                "traffic": None, "kernel": "f64_contract_kernel pass", "launch_ms": c_ms, "issued_frac": 28.0 * ach / peak,
+                "products_per_multiply_add": 28.0, "peak_source": "measured bf16 sustained"}
     else:
         c_ms = statistics.mean(kinds.get(3, [float("nan")]))
         ach = 2.0 * n * N / (c_ms * 1e-3) / 1e12

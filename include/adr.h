@@ -57,7 +57,7 @@ typedef enum {
 } adr_status;
 
 typedef enum {
-    ADR_FP64 = 0,          /* FP64 state, stencil and contractions (FP64 FMA)            */
+    ADR_FP64 = 0,          /* FP64 state, stencil and contractions (FP64 FMA, large ones exact digits on tensor cores) */
     ADR_FP32 = 1,          /* FP32 state, stencil and contractions (FP32 FMA)            */
     ADR_MIXED_TF32X3 = 2,  /* reserved: not implemented (returns ADR_ERR_UNSUPPORTED)    */
     ADR_MIXED_BF16X3 = 3   /* FP32 state and stencil; mu-mode contractions on the tensor
@@ -326,7 +326,7 @@ adr_status adr_measure_peak(int kind, int iters, double* tflops);
 int adr_kernels_per_step(const adr_ctx* ctx);
 
 /* Mixed-precision contexts after adr_set_coeffs: the number of slices (4) in which the standard
- * tensor-core images of the TMA-fed contraction write a factor; 0 for FP64 and FP32 contexts,
+ * tensor-core images of the mixed contraction write a factor; 0 for FP64 and FP32 contexts,
  * periodic and batched contexts, and before adr_set_coeffs. The exact-slice split of the
  * mu-mode products (Section 1) writes each factor row as 2^(e_i-7) sum_j 2^(-8j) f_j with
  * integer slices: four slices make a 32-bit factor, and the standard contraction then issues
