@@ -1262,15 +1262,14 @@ adr_status batch_tune(adr_ctx* c) {
                 a.items = d_tmp;
                 a.nitems = int(items.size());
                 a.mode = mode;
-                a.max_tile = t;
-                a.grid = std::min(int(items.size()), resident(t));
+                a.grid = std::min(int(items.size()), 2 * sms);   // the kernel for all shapes, as a mixed list runs
                 float ms = 0.f;
                 if (e == cudaSuccess) e = best_of([a](cudaStream_t s) { return adr::launch_batch_contract(a, s); }, ms);
                 if (e == cudaSuccess && ms < best_ms) { best_ms = ms; best_t = t; }
             }
             std::vector<int4> items;
             append_items(b, cl.second, best_t, items);
-            const double g = double(std::min(int(items.size()), resident(best_t)));
+            const double g = double(std::min(int(items.size()), 2 * sms));
             max_tile = std::max(max_tile, best_t);
             const double per_item = double(best_ms) * g / double(items.size());
             for (int i : cl.second) b.tile[mode - 1][i] = best_t;
