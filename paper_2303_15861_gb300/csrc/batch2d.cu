@@ -518,7 +518,7 @@ __device__ __forceinline__ void tile_gemm(TileSmem<T, MAXE>& sm, const T* __rest
 // (the next one in flight during 16 x TM^2 FMAs), so the registers and shared memory that only larger
 // tiles need are left to more blocks.
 // One kernel for all three shapes (two blocks per SM in FP32, one in FP64) -> these, same bits: 96 instances of 24 to 160 nodes
-// a direction, Lawson4 FP32, six steps on each of three streams 1112 -> 781 us; 200 of 24 to 120, Lawson2a FP64 11.07 ->
+// a direction, Lawson4 FP32, six steps on each of three streams 1103 -> 796 us; 200 of 24 to 120, Lawson2a FP64 11.07 ->
 // 9.50 ms; 40 of 100 to 250, Lawson4 FP64 28.9 -> 26.3 ms.
 constexpr int blocks_per_sm(int maxe, bool fp64) { return maxe == 32 ? (fp64 ? 4 : 6) : maxe == 64 ? (fp64 ? 2 : 4) : (fp64 ? 1 : 2); }
 
