@@ -211,6 +211,25 @@ void drop_graph(adr_ctx* c) {
     c->graph_u = nullptr;
 }
 
+// New coefficients go, through the legacy stream, into the buffers that the steps of the old ones read, and a
+// non-blocking stream is not ordered against that one: what is in flight on the context's stream ends first ...
+adr_status settle(adr_ctx* c) {
+    const cudaError_t e = c->coeffs_set ? cudaStreamSynchronize(c->stream) : cudaSuccess;   // else no step can be in flight
+    if (e != cudaSuccess) return cuda_fail(c, e, "steps before the new coefficients");
+    drop_graph(c);
+    c->coeffs_set = false;
+    return ADR_OK;
+}
+
+// ... and the steps of the new ones start when the uploads (a copy from pageable memory may return before its last
+// bytes arrive) and the kernels on the legacy stream have.
+adr_status publish(adr_ctx* c) {
+    const cudaError_t e = cudaStreamSynchronize(nullptr);
+    if (e != cudaSuccess) return cuda_fail(c, e, "new coefficients");
+    c->coeffs_set = true;
+    return ADR_OK;
+}
+
 // Upload an FP64 host array in the working precision.
 cudaError_t upload(adr_ctx* c, void** dst, const std::vector<double>& src) {
     const size_t bytes = src.size() * c->esize;
@@ -1580,8 +1599,7 @@ adr_status batch_set_coeffs(adr_ctx* c, int i, const double* a_nodes, const doub
     const size_t nodes = size_t(n[0] + 2) * (n[1] + 2);
     for (size_t k = 0; k < nodes; ++k)
         if (!std::isfinite(a_nodes[k])) return fail(c, ADR_ERR_ARG, "a_nodes has a non-finite value");
-    drop_graph(c);
-    c->coeffs_set = false;
+    if (const adr_status st = settle(c); st != ADR_OK) return st;
     // Eq. (amaxbeta), per instance
     const double abar = c->p.abar_override > 0 ? c->p.abar_override : c->p.lambda * adr::nodal_max(a_nodes, nodes);
     if (!(abar > 0)) return fail(c, ADR_ERR_ARG, "lambda * a_max must be positive");
@@ -1655,15 +1673,13 @@ adr_status batch_set_coeffs(adr_ctx* c, int i, const double* a_nodes, const doub
             if (e != cudaSuccess) return cuda_fail(c, e, "mixed batch plan");
             b.tuned = true;
         }
-        c->coeffs_set = true;
-        return ADR_OK;
+        return publish(c);
     }
     if (!b.tuned) {
         const adr_status st = c->fp64 ? batch_tune<double>(c) : batch_tune<float>(c);
         if (st != ADR_OK) return st;
     }
-    c->coeffs_set = true;
-    return ADR_OK;
+    return publish(c);
 }
 
 }  // namespace
@@ -1930,8 +1946,7 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
     if (!a_nodes || !b || !r_poly) return fail(c, ADR_ERR_ARG, "NULL coefficient pointer");
     for (size_t i = 0; i < c->nodes; ++i)
         if (!std::isfinite(a_nodes[i])) return fail(c, ADR_ERR_ARG, "a_nodes has a non-finite value");
-    drop_graph(c);
-    c->coeffs_set = false;
+    if (const adr_status st = settle(c); st != ADR_OK) return st;
     for (int m = 0; m < 3; ++m) c->b[m] = (m < c->dim) ? b[m] : 0.0;
     for (int i = 0; i < 4; ++i) c->r[i] = r_poly[i];
     // Eq. (amaxbeta)
@@ -2070,10 +2085,7 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
             if (e != cudaSuccess) return cuda_fail(c, e, "phi tables");
         }
     }
-    e = cudaStreamSynchronize(nullptr);    // the kernels above ran on the legacy stream
-    if (e != cudaSuccess) return cuda_fail(c, e, "set_coeffs");
-    c->coeffs_set = true;
-    return ADR_OK;
+    return publish(c);
 }
 
 adr_status adr_set_coeffs_periodic(adr_ctx* c, const double* a_diag, const double* b_field, const double r_poly[4]) {
@@ -2087,8 +2099,7 @@ adr_status adr_set_coeffs_periodic(adr_ctx* c, const double* a_diag, const doubl
             return fail(c, ADR_ERR_ARG, "a_diag or b_field has a non-finite value");
     for (int i = 0; i < 4; ++i)
         if (!std::isfinite(r_poly[i])) return fail(c, ADR_ERR_ARG, "r_poly has a non-finite value");
-    drop_graph(c);
-    c->coeffs_set = false;
+    if (const adr_status st = settle(c); st != ADR_OK) return st;
     for (int i = 0; i < 4; ++i) c->r[i] = r_poly[i];
     // Eq. (amaxbeta): a^max_mu = lambda max a_mumu, beta_mu = mean of b_mu (the mean of d_mu a_mumu
     // over a period is zero)
@@ -2140,8 +2151,7 @@ adr_status adr_set_coeffs_periodic(adr_ctx* c, const double* a_diag, const doubl
     for (int q = 0; q < 5 && e == cudaSuccess; ++q) e = upload(c, &c->d_pm[q], mult[q]);
     if (e != cudaSuccess) return cuda_fail(c, e, "upload Fourier multipliers");
     c->phi_route = needs_phi(c->p.scheme) ? ADR_PHI_FOURIER : 0;
-    c->coeffs_set = true;
-    return ADR_OK;
+    return publish(c);
 }
 
 adr_status adr_step(adr_ctx* c, void* u, double t) {
