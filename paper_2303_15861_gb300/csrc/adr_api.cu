@@ -148,6 +148,8 @@ struct adr_ctx {
     bool f64tc = false;                    // ... and every factor is within its range
     uint8_t* d_img64[kFactorKinds][3] = {{nullptr}};
     int* d_rows64[kFactorKinds][3] = {{nullptr}};
+    int* d_cexp64[kFactorKinds][3] = {{nullptr}};        // column exponents, of the factors that have any (eq64)
+    bool eq64[kFactorKinds][3] = {{false}};
     double* d_phi64[3] = {nullptr, nullptr, nullptr};   // FP64 contexts: phi_k(tau (l1 + l2 + l3)) at the nodes, k = 0, 1, 2
 
     // batched 2-D instances (p.batch > 0)
@@ -270,9 +272,14 @@ cudaError_t upload_f64(adr_ctx* c, int kind, int m, const std::vector<double>& M
     if (!c->d_img64[kind][m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_img64[kind][m]), adr::f64_image_bytes(n));
     if (e == cudaSuccess && !c->d_rows64[kind][m])
         e = cudaMalloc(reinterpret_cast<void**>(&c->d_rows64[kind][m]), adr::f64_rows(n) * sizeof(int));
+    const std::vector<int> cexp = adr::f64_column_exps(M, n);
+    int*& d_cexp = c->d_cexp64[kind][m];
+    const bool eq = c->eq64[kind][m] = !cexp.empty();
+    if (e == cudaSuccess && eq && !d_cexp) e = cudaMalloc(reinterpret_cast<void**>(&d_cexp), cexp.size() * sizeof(int));
+    if (e == cudaSuccess && eq) e = cudaMemcpy(d_cexp, cexp.data(), cexp.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-        e = adr::launch_f64_factor(static_cast<const double*>(dense_factor(c, kind, m)), n, c->d_img64[kind][m],
-                                   c->d_rows64[kind][m], nullptr);
+        e = adr::launch_f64_factor(static_cast<const double*>(dense_factor(c, kind, m)), n, eq ? d_cexp : nullptr,
+                                   c->d_img64[kind][m], c->d_rows64[kind][m], nullptr);
     return e;
 }
 
@@ -516,6 +523,7 @@ void push_mode_f64(Sched& S, int mu, int kind, const double* x, double* y, int e
     a.factor = static_cast<const double*>(dense_factor(c, kind, mu - 1));
     a.fimg = c->d_img64[kind][mu - 1];
     a.rows = c->d_rows64[kind][mu - 1];
+    a.cexp = c->eq64[kind][mu - 1] ? c->d_cexp64[kind][mu - 1] : nullptr;
     a.n = c->n[mu - 1];
     for (int nu = 1; nu < mu; ++nu) a.Q *= c->n[nu - 1];
     a.npos = static_cast<long long>(c->N) / a.n;
@@ -2470,6 +2478,7 @@ void adr_destroy(adr_ctx* c) {
     for (auto& p : c->d_phi32) { void* q = p; free_dev(q); p = nullptr; }
     for (auto& row : c->d_img64) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
     for (auto& row : c->d_rows64) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
+    for (auto& row : c->d_cexp64) for (auto& p : row) { void* q = p; free_dev(q); p = nullptr; }
     for (auto& p : c->d_phi64) { void* q = p; free_dev(q); p = nullptr; }
     for (auto& p : c->d_zt) { void* q = p; free_dev(q); p = nullptr; }
     { void* q = c->d_slots; free_dev(q); c->d_slots = nullptr; }

@@ -176,6 +176,7 @@ struct F64Args {
     const double* factor = nullptr;  // dense, row-major (for lines contracted with plain FMAs)
     const uint8_t* fimg = nullptr;   // its slices
     const int* rows = nullptr;       // per factor row: exponent of the result's unit less that of the line
+    const int* cexp = nullptr;       // c_k <= 0 per K position, padded to whole chunks: x_k 2^c_k meets f_k 2^-c_k (NULL: all 0)
     int n = 0;
     long long Q = 1, npos = 0;       // npos: positions P Q (modes >= 2) or fibres P (mode 1, Q = 1)
     int epi = EPI_STORE;
@@ -195,7 +196,8 @@ struct F64Args {
 cudaError_t launch_contract_f64(F64Args a, cudaStream_t s);
 size_t f64_image_bytes(int n);
 int f64_rows(int n);                 // rows of the image (n rounded up to whole tiles)
-cudaError_t launch_f64_factor(const double* M, int n, uint8_t* img, int* rows, cudaStream_t s);
+std::vector<int> f64_column_exps(const std::vector<double>& M, int n);   // c_k of a factor, or nothing where all are 0 (host_setup.cpp)
+cudaError_t launch_f64_factor(const double* M, int n, const int* cexp, uint8_t* img, int* rows, cudaStream_t s);
 
 // Host: slice an FP64 factor into the tensor-core image: per output tile of 128 rows and K chunk of 32, the slice
 // tiles F0..F3 in the 64-byte-swizzled K-major layout.

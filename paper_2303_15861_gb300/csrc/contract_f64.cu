@@ -5,8 +5,8 @@
 // takes 7.4 ms there. The tensor cores do 1.9 PFLOP/s in BF16. So x and the factor are cut into
 // integer slices whose products the tensor cores sum exactly, and the slices of the result are put
 // together in 64-bit integers:
-//   X = rint(x 2^(56 - es)) = sum_i S_i 2^(8 (6 - i)),  |S_0| <= 256, |S_1..S_6| <= 128, |x| < 2^es,
-//   F = rint(f 2^(56 - ef)) = sum_j F_j 2^(8 (6 - j)),  the same, ef per factor row,
+//   X_k = rint(x_k 2^(c_k + 56 - es)) = sum_i S_i 2^(8 (6 - i)),  |S_0| <= 256, |S_1..S_6| <= 128, |x_k| 2^c_k < 2^es,
+//   F_k = rint(f_k 2^(-c_k + 56 - ef)) = sum_j F_j 2^(8 (6 - j)),  the same, ef per factor row, c_k per factor column,
 //   D_s = sum_{i + j = s} S_i . F_j,  s = 0..6  (28 products),
 //   T = sum_s D_s 2^(8 (6 - s)),   x . f = T 2^(es + ef - 64).
 // The seven D_s are TMEM accumulators. They are sums of integers, exact in FP32 up to 2^24: with
@@ -16,8 +16,14 @@
 // signs: the digits past the first of a varying row or state average out (the sums are then near 2^19).
 // Errors: 2^-57 of 2^es and 2^ef for the two representations, about sqrt(K) 2^-57 of 2^(es + ef) for
 // the slice products left out (i + j > 6), and one rounding of the result to FP64. A chain of K FMAs rounds
-// K times. Against exact sums, e^{c tau A}, V and V^-1 for n = 24..300, b = 1..50, smooth and random
-// states: relative l2 4e-17 to 1.6e-16, where the FMA kernel has 9e-17 to 6.3e-16, and the smaller of the two in every case.
+// K times, but each time at the size of its own terms, so what decides is whether 2^(es + ef) is the size of the largest
+// term. The columns of V_mu^-1 differ by rho^n (5e8 at n = 128 and b = 40 abar): the c_k give them one
+// size. Without them, a pulse of width 0.05 that lies where the columns are small (128^2, b = 50, 60, 80 along x1, abar = 1.5)
+// left a phi action 3e-12, 9e-12 and 7e-10 off; with them pulses at b = 30 and 60 are 1e-15 to 4e-15 off and within 4%
+// of the FMA chain. Over 162 exponentials and phi actions
+// (n = 64..520, b = 3..60, smooth, random, pulses, single points) against 80-bit sums the relative l2 error
+// is 0.37 to 1.6 times that of the FMA kernel, 0.92 in the mean. It is an error of the line: results more than 2^-53 below the
+// line's largest are noise of that size, of either sign, where a chain of positive terms would keep their digits.
 // Time of a pass, FMA kernel -> this one: 256^3 6.9 ms -> 0.24 ms, 128^3 526 -> 31 us (39 with the phi table), 60^3
 // 33 -> 12 us. At the BF16 rate the products of a 256^3 pass take 0.13 ms; the rest is the assembly of a tile,
 // which cannot overlap its MMAs (the accumulators fill TMEM), and the producers just behind them.
@@ -86,12 +92,12 @@ __device__ __forceinline__ uint32_t idesc_of(int ncols) {   // FP32 accumulator,
     return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(ncols >> 3) << 17) | (uint32_t(kM >> 4) << 24);
 }
 
-// Cut x into its seven digits: d = es + 1022 - exponent(x) >= 0 places below the leading one. Digits
+// Cut x 2^c into its seven digits: d = etop - c - exponent(x) >= 0 places below the leading one. Digits
 // 1..6 are bytes of X + 0x808080808080 less 128, digit 0 what is above them. Returned as FP32 values
 // whose upper halves are their BF16 forms (integers of at most 8 bits).
-__device__ __forceinline__ void cut(double x, int etop, float (&s)[kSl]) {
+__device__ __forceinline__ void cut(double x, int etop, int c, float (&s)[kSl]) {
     const uint32_t hi = uint32_t(__double2hiint(x)), lo = uint32_t(__double2loint(x));
-    const int d = min(etop - int((hi >> 20) & 0x7FFu), 63);
+    const int d = min(etop - c - int((hi >> 20) & 0x7FFu), 63);
     const unsigned long long m = (static_cast<unsigned long long>((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
     long long v = static_cast<long long>((((m << 4) >> d) + 1ull) >> 1);
     const long long sg = static_cast<long long>(int(hi) >> 31);
@@ -106,15 +112,15 @@ __device__ __forceinline__ void cut(double x, int etop, float (&s)[kSl]) {
     s[6] = __uint_as_float(__byte_perm(vl, 0x4B000000u, 0x7440)) - 8388736.f;
 }
 
-// Cut KV (4 or 8) values along K and store them at K position k of row r of the seven slice tiles.
+// Cut KV (4 or 8) values along K, of exponents c, and store them at K position k of row r of the seven slice tiles.
 template <int TILE, int KV>
-__device__ __forceinline__ void cut_store(const double (&v)[KV], int etop, uint32_t tile0, int r, int k) {
+__device__ __forceinline__ void cut_store(const double (&v)[KV], int etop, const int (&c)[KV], uint32_t tile0, int r, int k) {
     uint32_t w[kSl][KV / 2];
 #pragma unroll
     for (int e = 0; e < KV / 2; ++e) {
         float a[kSl], b[kSl];
-        cut(v[2 * e], etop, a);
-        cut(v[2 * e + 1], etop, b);
+        cut(v[2 * e], etop, c[2 * e], a);
+        cut(v[2 * e + 1], etop, c[2 * e + 1], b);
 #pragma unroll
         for (int q = 0; q < kSl; ++q) w[q][e] = __byte_perm(__float_as_uint(a[q]), __float_as_uint(b[q]), 0x7632);
     }
@@ -185,11 +191,8 @@ __device__ __noinline__ double fma_dot(const double* f, const double* x, int n, 
     return acc;
 }
 
-// |v| as an unsigned that orders like |v|: the upper word, with its last bit set where the lower
-// word is not zero (so it is 0 only for v = 0). NaN orders above infinity.
-__device__ __forceinline__ unsigned f64_amax_bits(double v) {
-    return (unsigned(__double2hiint(v)) & 0x7FFFFFFFu) | (__double2loint(v) != 0 ? 1u : 0u);
-}
+// The upper word of |v|. NaN orders above infinity.
+__device__ __forceinline__ int f64_abs_hi(double v) { return __double2hiint(v) & 0x7FFFFFFF; }
 
 // The phi factor of node o, where the context keeps no table.
 __device__ __noinline__ double f64_phi_eval(const F64Args& p, long long o) {
@@ -200,7 +203,7 @@ __device__ __noinline__ double f64_phi_eval(const F64Args& p, long long o) {
 
 constexpr int kNoCut = 1 << 20;          // es of a line that fma_dot contracts
 
-template <bool MODE1, int N, int EPI>
+template <bool MODE1, int N, int EPI, bool EQ>
 __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_constant__ F64Args p) {
     using C = Cfg<N>;
     extern __shared__ uint8_t smem_raw[];
@@ -212,7 +215,15 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
     // per line of the last tiles: its exponent es, and its offset in the state (k = 0)
     __shared__ int es_s[kTileBufs][N];
     __shared__ long long off_s[kTileBufs][N];
-    __shared__ unsigned part_s[2][C::KG][N];                 // modes >= 2: the parts of a line's max|x|
+    __shared__ int part_s[2][C::KG][N];                      // modes >= 2: the parts of a line's max|x|
+    __shared__ __align__(16) int cexp_s[EQ ? kF64MaxN : 4];  // c_k (EQ: the factor has any)
+
+    static_assert(kF64MaxN <= 2 * kThreads, "two column exponents a thread");
+    int c0 = 0, c1 = 0;                                      // on their way during the set-up
+    if (EQ) {
+        if (threadIdx.x < p.nK * kKc) c0 = p.cexp[threadIdx.x];
+        if (threadIdx.x + kThreads < p.nK * kKc) c1 = p.cexp[threadIdx.x + kThreads];
+    }
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;     // state-slice ring
@@ -244,6 +255,10 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
                      "r"(C::TMEM)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (EQ) {
+        if (threadIdx.x < p.nK * kKc) cexp_s[threadIdx.x] = c0;
+        if (threadIdx.x + kThreads < p.nK * kKc) cexp_s[threadIdx.x + kThreads] = c1;
     }
     tc_fence_before();
     __syncthreads();
@@ -307,26 +322,43 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
                 for (int e = 0; e < KV; ++e) w[e] = (lrow && k0 + kofs + e < n) ? __ldg(x + e * Q) : 0.0;
             }
         };
-        auto amax = [&](const double (&w)[KV], unsigned m) {
+        auto exps = [&](int k0, int (&c)[KV]) {
 #pragma unroll
-            for (int e = 0; e < KV; ++e) m = max(m, f64_amax_bits(w[e]));
-            return m;
+            for (int e = 0; e < KV; e += 4) {
+                const int4 q = EQ ? *reinterpret_cast<const int4*>(&cexp_s[k0 + kofs + e]) : make_int4(0, 0, 0, 0);
+                c[e] = q.x; c[e + 1] = q.y; c[e + 2] = q.z; c[e + 3] = q.w;
+            }
+        };
+        // upper word of the largest |x_k| 2^c_k (0 below the normal range), and whether any value is not zero
+        int m = 0, any = 0;
+        auto amax = [&](const double (&w)[KV], int k0) {
+            int c[KV];
+            exps(k0, c);
+#pragma unroll
+            for (int e = 0; e < KV; ++e) {
+                const int h = f64_abs_hi(w[e]);
+                m = max(m, h + c[e] * (1 << 20));
+                any |= h | __double2loint(w[e]);
+            }
         };
         // es of this thread's line, of which v holds the first chunk
         auto line_scale = [&](int tl) {
-            unsigned m = amax(v, 0u);
+            m = any = 0;
+            amax(v, 0);
             int c = 1;
             for (; c + 1 < p.nK; c += 2) {                   // two chunks of loads in flight
                 double w[KV], u[KV];
                 load(c * kKc, w);
                 load((c + 1) * kKc, u);
-                m = amax(u, amax(w, m));
+                amax(w, c * kKc);
+                amax(u, (c + 1) * kKc);
             }
             if (c < p.nK) {
                 double w[KV];
                 load(c * kKc, w);
-                m = amax(w, m);
+                amax(w, c * kKc);
             }
+            if (any) m = max(m, 1);
             if (MODE1) {
 #pragma unroll
                 for (int o = 1; o < KG; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -336,8 +368,8 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
 #pragma unroll
                 for (int o = 0; o < KG; ++o) m = max(m, part_s[tl & 1][o][row]);
             }
-            const int eb = int(m >> 20);
-            live = m == 0u || (eb >= 1023 - 500 && eb <= 1023 + 500);
+            const int eb = m >> 20;
+            live = m == 0 || (eb >= 1023 - 500 && eb <= 1023 + 500);
             etop = m ? eb : 1022;                            // es + 1022
             if (kg == 0) {
                 es_s[tl & (kTileBufs - 1)][row] = live ? etop - 1022 : kNoCut;
@@ -352,6 +384,8 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
             // still meets the others at line_scale's barrier
             mbar_wait(sempty(ss), sph, p.err, 1, &abort_s, 32);
             __syncwarp();
+            int ce[KV];
+            exps(lc * kKc, ce);
             const bool next_tile = ++lc == p.nK;
             if (next_tile) {
                 lc = 0;
@@ -362,7 +396,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
 #pragma unroll
                 for (int e = 0; e < KV; ++e) v[e] = 0.0;
             }
-            cut_store<C::STILE, KV>(v, etop, sbase + ss * C::SBYTES, row, kofs);
+            cut_store<C::STILE, KV>(v, etop, ce, sbase + ss * C::SBYTES, row, kofs);
             load(lc * kKc, v);                               // in flight until the next chunk is cut
             fence_proxy_async();
             __syncwarp();
@@ -527,27 +561,30 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
     }
 }
 
-// Cut the dense factor (n x n, row-major) into its image: per (tile of 128 rows, K chunk of 32)
-// seven 64-byte-swizzled K-major tiles; and per row the exponent of the result's unit, less es. One block per
-// padded row.
-__global__ void f64_factor_kernel(const double* M, int n, int nK, uint8_t* img, int* rows) {
+// Cut the dense factor (n x n, row-major), its column k times 2^-c_k, into its image: per (tile of 128 rows, K chunk of
+// 32) seven 64-byte-swizzled K-major tiles; and per row the exponent of the result's unit, less es. One block
+// per padded row.
+__global__ void f64_factor_kernel(const double* M, int n, int nK, const int* cexp, uint8_t* img, int* rows) {
     const int i = blockIdx.x;
-    __shared__ unsigned smax;
+    __shared__ int smax;
     if (threadIdx.x == 0) smax = 0;
     __syncthreads();
-    unsigned m = 0;
+    int m = 0;                                               // exponent field of the largest entry; 0: no entry
     if (i < n)
-        for (int k = threadIdx.x; k < n; k += blockDim.x) m = max(m, f64_amax_bits(M[(size_t)i * n + k]));
+        for (int k = threadIdx.x; k < n; k += blockDim.x) {
+            const int h = f64_abs_hi(M[(size_t)i * n + k]) >> 20;
+            if (h) m = max(m, h - (cexp ? cexp[k] : 0));
+        }
     atomicMax(&smax, m);
     __syncthreads();
     // max|f| < 2^ef; rows below 2^-500 keep that scale (their digits are then smaller)
-    const int ef = smax ? max(int(smax >> 20) - 1022, -500) : 0;
+    const int ef = smax ? max(smax - 1022, -500) : 0;
     if (threadIdx.x == 0) rows[i] = ef - 64;
     uint8_t* tile = img + (size_t)(i / kM) * nK * kSl * kM * 64;
     for (int k = threadIdx.x; k < nK * kKc; k += blockDim.x) {
         const double f = (i < n && k < n) ? M[(size_t)i * n + k] : 0.0;
         float s[kSl];
-        cut(f, ef + 1022, s);
+        cut(f, ef + 1022, cexp ? -cexp[k] : 0, s);
         const int kc = k % kKc;
         uint8_t* dst = tile + (size_t)(k / kKc) * kSl * kM * 64 + swz64(i % kM, kc / 8) + (kc % 8) * 2;
 #pragma unroll
@@ -566,21 +603,25 @@ int sm_count() {
     return sms;
 }
 
-template <bool MODE1, int N, int EPI>
+template <bool MODE1, int N, int EPI, bool EQ>
 cudaError_t launch_variant(const F64Args& a, cudaStream_t s) {
-    static const cudaError_t attr = cudaFuncSetAttribute(f64_contract_kernel<MODE1, N, EPI>,
+    static const cudaError_t attr = cudaFuncSetAttribute(f64_contract_kernel<MODE1, N, EPI, EQ>,
                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<N>::SMEM);
     if (attr != cudaSuccess) return attr;
     const int grid = a.ntiles < sm_count() ? a.ntiles : sm_count();
-    f64_contract_kernel<MODE1, N, EPI><<<unsigned(grid), kThreads, Cfg<N>::SMEM, s>>>(a);
+    f64_contract_kernel<MODE1, N, EPI, EQ><<<unsigned(grid), kThreads, Cfg<N>::SMEM, s>>>(a);
     return cudaGetLastError();
 }
 
-template <bool MODE1, int N>
+template <bool MODE1, int N, bool EQ>
 cudaError_t launch_epi(const F64Args& a, cudaStream_t s) {
-    if (a.epi == EPI_PHI) return launch_variant<MODE1, N, EPI_PHI>(a, s);
-    if (a.epi == EPI_AXPY) return launch_variant<MODE1, N, EPI_AXPY>(a, s);
-    return launch_variant<MODE1, N, EPI_STORE>(a, s);
+    if (a.epi == EPI_PHI) return launch_variant<MODE1, N, EPI_PHI, EQ>(a, s);
+    if (a.epi == EPI_AXPY) return launch_variant<MODE1, N, EPI_AXPY, EQ>(a, s);
+    return launch_variant<MODE1, N, EPI_STORE, EQ>(a, s);
+}
+template <bool MODE1, int N>
+cudaError_t launch_eq(const F64Args& a, cudaStream_t s) {
+    return a.cexp ? launch_epi<MODE1, N, true>(a, s) : launch_epi<MODE1, N, false>(a, s);
 }
 
 }  // namespace
@@ -588,8 +629,9 @@ cudaError_t launch_epi(const F64Args& a, cudaStream_t s) {
 size_t f64_image_bytes(int n) { return size_t((n + kM - 1) / kM) * kM * ((n + kKc - 1) / kKc) * kKc * 2 * kSl; }
 int f64_rows(int n) { return (n + kM - 1) / kM * kM; }
 
-cudaError_t launch_f64_factor(const double* M, int n, uint8_t* img, int* rows, cudaStream_t s) {
-    f64_factor_kernel<<<f64_rows(n), 128, 0, s>>>(M, n, (n + kKc - 1) / kKc, img, rows);
+
+cudaError_t launch_f64_factor(const double* M, int n, const int* cexp, uint8_t* img, int* rows, cudaStream_t s) {
+    f64_factor_kernel<<<f64_rows(n), 128, 0, s>>>(M, n, (n + kKc - 1) / kKc, cexp, img, rows);
     return cudaGetLastError();
 }
 
@@ -604,8 +646,8 @@ cudaError_t launch_contract_f64(F64Args a, cudaStream_t s) {
     a.vec4 = !mode1 && a.Q % 4 == 0 && aligned(a.Y, 32) && aligned(a.base, 32) && aligned(a.phi, 32);
     const bool wide = (a.npos + 63) / 64 * a.nOut >= sm_count();
     a.ntiles = int((a.npos + (wide ? 63 : 31)) / (wide ? 64 : 32) * a.nOut);
-    if (mode1) return wide ? launch_epi<true, 64>(a, s) : launch_epi<true, 32>(a, s);
-    return wide ? launch_epi<false, 64>(a, s) : launch_epi<false, 32>(a, s);
+    if (mode1) return wide ? launch_eq<true, 64>(a, s) : launch_eq<true, 32>(a, s);
+    return wide ? launch_eq<false, 64>(a, s) : launch_eq<false, 32>(a, s);
 }
 
 }  // namespace adr

@@ -1,6 +1,7 @@
 // Host-side operator setup in FP64: the 1-D factors A_mu of the extracted operator,
 // their exponentials and their closed-form eigenpairs (Sections 3 and 5.2).
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <stdexcept>
@@ -180,6 +181,26 @@ uint16_t bf16_bits_exact(double v) {
     return static_cast<uint16_t>(u >> 16);
 }
 }  // namespace
+
+// c_k of the FP64 tensor-core contraction (contract_f64.cu): the exponent of column k's largest entry less the
+// largest such exponent, so that f_k 2^-c_k has columns of one size. Columns within a factor of 8 of each other stay as they
+// are: the digits hold three bits more than an FP64 value.
+std::vector<int> f64_column_exps(const std::vector<double>& M, int n) {
+    std::vector<double> mx(size_t(n), 0.0);
+    for (int i = 0; i < n; ++i)
+        for (int k = 0; k < n; ++k) mx[k] = std::max(mx[k], std::fabs(M[size_t(i) * n + k]));
+    std::vector<int> c(size_t((n + kF64Chunk - 1) / kF64Chunk * kF64Chunk), 0);   // whole chunks
+    int top = INT_MIN, low = INT_MAX;
+    for (int k = 0; k < n; ++k) {
+        if (mx[k] == 0.0) continue;
+        c[k] = std::ilogb(mx[k]);
+        top = std::max(top, c[k]);
+        low = std::min(low, c[k]);
+    }
+    if (top == INT_MIN || low >= top - 2) return {};
+    for (int k = 0; k < n; ++k) c[k] = std::max((mx[k] == 0.0 ? low : c[k]) - top, -400);
+    return c;
+}
 
 TcFactor make_tc_factor(const std::vector<double>& M, int n) {
     // Each row i of M (an output index) is written as 2^(e_i-7) sum_j 2^(-8j) f_j with
