@@ -168,6 +168,7 @@ cudaError_t launch_phi_table(float* tab, int k, const float* const zt[3], int n1
 // contracted along n with a factor cut into seven slices.
 constexpr int kF64Slices = 7;
 constexpr int kF64Chunk = 32;        // K per factor tile
+constexpr int kF64MinExp = -400;     // the lowest column exponent
 constexpr int kF64MaxN = 1024;       // longest line (the cut factor takes 14 n^2 bytes)
 
 struct F64Args {
@@ -175,7 +176,7 @@ struct F64Args {
     double* Y = nullptr;
     const double* factor = nullptr;  // dense, row-major (for lines contracted with plain FMAs)
     const uint8_t* fimg = nullptr;   // its slices
-    const int* rows = nullptr;       // per factor row: exponent of the result's unit less that of the line
+    const int* rows = nullptr;       // per factor row: exponent of the result's unit less that of the line (offset: contract_f64.cu)
     const int* cexp = nullptr;       // c_k <= 0 per K position, padded to whole chunks: x_k 2^c_k meets f_k 2^-c_k (NULL: all 0)
     int n = 0;
     long long Q = 1, npos = 0;       // npos: positions P Q (modes >= 2) or fibres P (mode 1, Q = 1)

@@ -32,9 +32,9 @@
 // once for their largest exponents and a second time, from L2, to cut them. One es for the whole array would
 // save that read, but each pass would then lose what the array varies by: through the eigenbasis
 // (V_mu scaled by rho^i, 28-fold from end to end per direction at b = 10) a 100 x 72 x 64 ETD2RK run was
-// 1.2e-14 off instead of 5e-16. Lines with a NaN or an infinity, or with max|x| outside
-// 2^-500..2^500, are contracted with plain FMAs by the epilogue, so that such values propagate as
-// in any FP64 sum.
+// 1.2e-14 off instead of 5e-16. Lines with a NaN or an infinity, or with max|x| below 2^-958 (or, where the factor has
+// column exponents, above 2^624), are contracted with plain FMAs by the epilogue, so that such values propagate as
+// in any FP64 sum. That costs 1.2 ms a pass at 128^3 where the FMA kernel takes 0.53.
 //
 // Work split. The factor is the A operand, 128 outputs (TMEM lanes) a tile; the lines are the B operand,
 // N = 64 of them (448 of the 512 TMEM columns), or 32 where 64 would leave SMs without a tile. For modes >= 2
@@ -167,8 +167,10 @@ __device__ __forceinline__ void tmem_ld4x7(uint32_t t0, uint32_t stride, float (
         for (int j = 0; j < 4; ++j) d[k][j] = __uint_as_float(r[4 * k + j]);
 }
 
-// The result from its seven sums, in units of 2^e: T = 2^24 h + l, shifted right (rounding) by the ex >= 0 places that
-// leave it 62 bits; the conversion to FP64 rounds to nearest, and the unit goes into the exponent.
+// The result from its seven sums, in units of 2^(e - kUnit): T = 2^24 h + l, shifted right (rounding) by the ex >= 0 places
+// that leave it 62 bits; the conversion to FP64 rounds to nearest, and the unit goes into the exponent, which
+// takes it for 0 <= e <= kUnitTop (1 <= |T| < 2^88).
+constexpr int kUnit = 1022, kUnitTop = kUnit + 1023 - 88;
 __device__ __forceinline__ double assemble(const float (&d)[kSl][4], int c, int e) {
     int v[kSl];
 #pragma unroll
@@ -180,9 +182,11 @@ __device__ __forceinline__ double assemble(const float (&d)[kSl][4], int c, int 
     const int ex = max(26 - __clz(top ^ (top >> 31)), 0);
     const long long t = (h << (24 - ex)) + ((l + ((1 << ex) >> 1)) >> ex);
     const double r = static_cast<double>(t);
-    const int up = t ? (e + ex) << 20 : 0;
+    const int up = t ? (e - kUnit + ex) * (1 << 20) : 0;
     return __hiloint2double(__double2hiint(r) + up, __double2loint(r));
 }
+
+__device__ __noinline__ double scale_by(double r, int e) { return ldexp(r, e); }
 
 // One output by plain FMAs, k ascending (lines whose values do not fit the slices).
 __device__ __noinline__ double fma_dot(const double* f, const double* x, int n, long long stride) {
@@ -341,6 +345,9 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
                 any |= h | __double2loint(w[e]);
             }
         };
+        // Lines that are cut, by the exponent field of their largest value: below kLiveLow a value outside the normal
+        // range, which cut() does not know, could still reach a digit; an infinity or a NaN has at least 2047 + min c_k
+        constexpr int kLiveLow = 64, kLiveHigh = 2047 + (EQ ? kF64MinExp : 0);
         // es of this thread's line, of which v holds the first chunk
         auto line_scale = [&](int tl) {
             m = any = 0;
@@ -369,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
                 for (int o = 0; o < KG; ++o) m = max(m, part_s[tl & 1][o][row]);
             }
             const int eb = m >> 20;
-            live = m == 0 || (eb >= 1023 - 500 && eb <= 1023 + 500);
+            live = m == 0 || (eb >= kLiveLow && eb < kLiveHigh);
             etop = m ? eb : 1022;                            // es + 1022
             if (kg == 0) {
                 es_s[tl & (kTileBufs - 1)][row] = live ? etop - 1022 : kNoCut;
@@ -470,14 +477,21 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
                         if (lane == 0) mbar_arrive(acce);
                     }
                     double v[4];
+                    unsigned unit[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) v[j] = assemble(d, j, rexp + es[j]);
-                    if (max(max(es[0], es[1]), max(es[2], es[3])) == kNoCut) {
+                    for (int j = 0; j < 4; ++j) unit[j] = unsigned(rexp + es[j]);
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
+                    for (int j = 0; j < 4; ++j) v[j] = assemble(d, j, int(min(unit[j], unsigned(kUnitTop))));
+                    // results that may leave the normal range, lines that were not cut (nothing of the sums is
+                    // needed any more: assembled anew here, they cost 8% of 128^3 ETD2RK)
+                    if (max(max(unit[0], unit[1]), max(unit[2], unit[3])) > unsigned(kUnitTop)) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            if (unit[j] > unsigned(kUnitTop)) v[j] = scale_by(v[j], int(unit[j]) - kUnitTop);
                             if (es[j] == kNoCut)
                                 v[j] = first && rvalid && j0 + j < ncol
                                            ? fma_dot(p.factor + (long long)irow * n, p.X + off[j] - ioff, n, Q) : 0.0;
+                        }
                     }
                     if (EPI == EPI_PHI) {
 #pragma unroll
@@ -561,30 +575,38 @@ __global__ void __launch_bounds__(kThreads, 1) f64_contract_kernel(const __grid_
     }
 }
 
+// A factor entry as a normal number times 2^sh.
+__device__ __forceinline__ double normal_part(double f, int& sh) {
+    sh = (f64_abs_hi(f) >> 20) ? 0 : -64;
+    return sh ? f * 18446744073709551616.0 : f;
+}
+
 // Cut the dense factor (n x n, row-major), its column k times 2^-c_k, into its image: per (tile of 128 rows, K chunk of
-// 32) seven 64-byte-swizzled K-major tiles; and per row the exponent of the result's unit, less es. One block
+// 32) seven 64-byte-swizzled K-major tiles; and per row the exponent of the result's unit, less es, plus kUnit. One block
 // per padded row.
 __global__ void f64_factor_kernel(const double* M, int n, int nK, const int* cexp, uint8_t* img, int* rows) {
     const int i = blockIdx.x;
     __shared__ int smax;
-    if (threadIdx.x == 0) smax = 0;
+    constexpr int kNone = -(1 << 20);                        // a row of zeros
+    if (threadIdx.x == 0) smax = kNone;
     __syncthreads();
-    int m = 0;                                               // exponent field of the largest entry; 0: no entry
+    int m = kNone;                                           // exponent field of the largest entry
     if (i < n)
         for (int k = threadIdx.x; k < n; k += blockDim.x) {
-            const int h = f64_abs_hi(M[(size_t)i * n + k]) >> 20;
-            if (h) m = max(m, h - (cexp ? cexp[k] : 0));
+            int sh;
+            const double f = normal_part(M[(size_t)i * n + k], sh);
+            if (f != 0.0) m = max(m, (f64_abs_hi(f) >> 20) + sh - (cexp ? cexp[k] : 0));
         }
     atomicMax(&smax, m);
     __syncthreads();
-    // max|f| < 2^ef; rows below 2^-500 keep that scale (their digits are then smaller)
-    const int ef = smax ? max(smax - 1022, -500) : 0;
-    if (threadIdx.x == 0) rows[i] = ef - 64;
+    const int ef = smax == kNone ? 0 : smax - 1022;          // max|f_k| 2^-c_k < 2^ef
+    if (threadIdx.x == 0) rows[i] = ef - 64 + kUnit;
     uint8_t* tile = img + (size_t)(i / kM) * nK * kSl * kM * 64;
     for (int k = threadIdx.x; k < nK * kKc; k += blockDim.x) {
-        const double f = (i < n && k < n) ? M[(size_t)i * n + k] : 0.0;
-        float s[kSl];
-        cut(f, ef + 1022, cexp ? -cexp[k] : 0, s);
+        int sh;
+        const double f = normal_part((i < n && k < n) ? M[(size_t)i * n + k] : 0.0, sh);
+        float s[kSl] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (f != 0.0) cut(f, ef + 1022, (cexp ? -cexp[k] : 0) + sh, s);
         const int kc = k % kKc;
         uint8_t* dst = tile + (size_t)(k / kKc) * kSl * kM * 64 + swz64(i % kM, kc / 8) + (kc % 8) * 2;
 #pragma unroll

@@ -198,7 +198,7 @@ std::vector<int> f64_column_exps(const std::vector<double>& M, int n) {
         low = std::min(low, c[k]);
     }
     if (top == INT_MIN || low >= top - 2) return {};
-    for (int k = 0; k < n; ++k) c[k] = std::max((mx[k] == 0.0 ? low : c[k]) - top, -400);
+    for (int k = 0; k < n; ++k) c[k] = std::max((mx[k] == 0.0 ? low : c[k]) - top, kF64MinExp);
     return c;
 }
 
