@@ -37,6 +37,7 @@
 #include <cstring>
 
 #include "adr_internal.h"
+#include "smem_limit.h"
 #include "tc_common.cuh"
 
 namespace adr {
@@ -573,9 +574,9 @@ int g_sms = 0;
 
 template <bool MODE1, int EPI>
 cudaError_t launch_variant(const BatchTcArgs& a, unsigned grid, cudaStream_t s) {
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(batch_tc_kernel<MODE1, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-    if (attr != cudaSuccess) return attr;
+    static SmemLimit smem;
+    const cudaError_t e = smem.allow(reinterpret_cast<const void*>(batch_tc_kernel<MODE1, EPI>), kSmem);
+    if (e != cudaSuccess) return e;
     batch_tc_kernel<MODE1, EPI><<<grid, kThreads, kSmem, s>>>(a);
     return cudaGetLastError();
 }

@@ -53,6 +53,7 @@
 
 #include "adr_internal.h"
 #include "phi_device.cuh"
+#include "smem_limit.h"
 #include "tc_common.cuh"
 
 namespace adr {
@@ -627,9 +628,9 @@ int sm_count() {
 
 template <bool MODE1, int N, int EPI, bool EQ>
 cudaError_t launch_variant(const F64Args& a, cudaStream_t s) {
-    static const cudaError_t attr = cudaFuncSetAttribute(f64_contract_kernel<MODE1, N, EPI, EQ>,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<N>::SMEM);
-    if (attr != cudaSuccess) return attr;
+    static SmemLimit smem;
+    const cudaError_t e = smem.allow(reinterpret_cast<const void*>(f64_contract_kernel<MODE1, N, EPI, EQ>), Cfg<N>::SMEM);
+    if (e != cudaSuccess) return e;
     const int grid = a.ntiles < sm_count() ? a.ntiles : sm_count();
     f64_contract_kernel<MODE1, N, EPI, EQ><<<unsigned(grid), kThreads, Cfg<N>::SMEM, s>>>(a);
     return cudaGetLastError();

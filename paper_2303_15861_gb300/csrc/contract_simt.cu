@@ -14,6 +14,7 @@
 #include "adr_internal.h"
 #include "launch.cuh"
 #include "phi_device.cuh"
+#include "smem_limit.h"
 
 namespace adr {
 namespace {
@@ -165,9 +166,10 @@ cudaError_t launch_tiled(const ContractArgs<T>& p, cudaStream_t s) {
 
 template <typename T, int W, int KS>
 cudaError_t launch_small(const ContractArgs<T>& p, cudaStream_t s) {
-    static const cudaError_t attr = cudaFuncSetAttribute(contract_small_kernel<T, W, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         int(2 * W * (kSmallK + 1) * sizeof(T)));
-    if (attr != cudaSuccess) return attr;
+    static SmemLimit smem;
+    const cudaError_t e = smem.allow(reinterpret_cast<const void*>(contract_small_kernel<T, W, KS>),
+                                     int(2 * W * (kSmallK + 1) * sizeof(T)));
+    if (e != cudaSuccess) return e;
     const dim3 grid((p.N + W - 1) / W, (p.M + W - 1) / W, p.batch);
     return launch_pdl(contract_small_kernel<T, W, KS>, grid, W * W * KS, size_t(2 * W) * (p.K + 1) * sizeof(T), s, p);
 }

@@ -37,6 +37,7 @@
 
 #include "adr_internal.h"
 #include "phi_device.cuh"
+#include "smem_limit.h"
 #include "tc_common.cuh"
 
 namespace adr {
@@ -453,9 +454,9 @@ int sm_count() {
 
 template <bool MODE1, int N, int EPI, bool LO>
 cudaError_t launch_variant(const TcArgs& a, cudaStream_t s) {
-    static const cudaError_t attr = cudaFuncSetAttribute(tc_contract_kernel<MODE1, N, EPI, LO>,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<N>::SMEM);
-    if (attr != cudaSuccess) return attr;
+    static SmemLimit smem;
+    const cudaError_t e = smem.allow(reinterpret_cast<const void*>(tc_contract_kernel<MODE1, N, EPI, LO>), Cfg<N>::SMEM);
+    if (e != cudaSuccess) return e;
     const int grid = a.ntiles < sm_count() ? a.ntiles : sm_count();
     tc_contract_kernel<MODE1, N, EPI, LO><<<unsigned(grid), kThreads, Cfg<N>::SMEM, s>>>(a);
     return cudaGetLastError();
