@@ -145,7 +145,7 @@ struct adr_ctx {
 
     // FP64 on the tensor cores (contract_f64.cu): cut factors with their row parameters, phi tables
     bool f64_grid = false;                 // the grid is one the kernel is the faster on
-    bool f64tc = false;                    // ... and every factor is within its range
+    bool cut64[kFactorKinds][3] = {{false}};          // ... and these factors are cut for it; the others take the FMA kernel
     uint8_t* d_img64[kFactorKinds][3] = {{nullptr}};
     int* d_rows64[kFactorKinds][3] = {{nullptr}};
     int* d_cexp64[kFactorKinds][3] = {{nullptr}};        // column exponents, of the factors that have any (eq64)
@@ -258,21 +258,22 @@ cudaError_t upload_tc(adr_ctx* c, int kind, int m, const std::vector<double>& M)
 
 const void* dense_factor(const adr_ctx* c, int kind, int m);
 
-// Cut the uploaded factor of a kind for the FP64 tensor-core contraction. Factors outside its range
-// (an entry that is not finite or at least 2^400) take the context back to the FMA kernel.
+// Cut the uploaded factor of a kind for the FP64 tensor-core contraction. A factor outside its range (an entry that is
+// not finite, columns that differ by 2^400 and more) takes the FMA kernel: V_mu of a cell Peclet number near one is such,
+// and no concern of the scheme's other factors.
 cudaError_t upload_f64(adr_ctx* c, int kind, int m, const std::vector<double>& M) {
-    if (!c->f64_grid || !c->f64tc) return cudaSuccess;
+    c->cut64[kind][m] = false;
+    if (!c->f64_grid) return cudaSuccess;
     for (double v : M)
-        if (!(std::fabs(v) < std::ldexp(1.0, 400))) {
-            c->f64tc = false;
-            return cudaSuccess;
-        }
+        if (!std::isfinite(v)) return cudaSuccess;
     const int n = c->n[m];
+    const std::vector<int> cexp = adr::f64_column_exps(M, n);
+    for (int v : cexp)
+        if (v <= adr::kF64MinExp) return cudaSuccess;
     cudaError_t e = cudaSuccess;
     if (!c->d_img64[kind][m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_img64[kind][m]), adr::f64_image_bytes(n));
     if (e == cudaSuccess && !c->d_rows64[kind][m])
         e = cudaMalloc(reinterpret_cast<void**>(&c->d_rows64[kind][m]), adr::f64_rows(n) * sizeof(int));
-    const std::vector<int> cexp = adr::f64_column_exps(M, n);
     int*& d_cexp = c->d_cexp64[kind][m];
     const bool eq = c->eq64[kind][m] = !cexp.empty();
     if (e == cudaSuccess && eq && !d_cexp) e = cudaMalloc(reinterpret_cast<void**>(&d_cexp), cexp.size() * sizeof(int));
@@ -280,6 +281,7 @@ cudaError_t upload_f64(adr_ctx* c, int kind, int m, const std::vector<double>& M
     if (e == cudaSuccess)
         e = adr::launch_f64_factor(static_cast<const double*>(dense_factor(c, kind, m)), n, eq ? d_cexp : nullptr,
                                    c->d_img64[kind][m], c->d_rows64[kind][m], nullptr);
+    c->cut64[kind][m] = e == cudaSuccess;
     return e;
 }
 
@@ -553,7 +555,7 @@ void push_mode(Sched& S, int mu, int kind, const T* x, T* y, int epi = adr::EPI_
         return;
     }
     if constexpr (sizeof(T) == 8) {
-        if (c->f64tc) {
+        if (c->cut64[kind][mu - 1]) {
             push_mode_f64(S, mu, kind, x, y, epi, base, alpha, phik);
             return;
         }
@@ -2000,7 +2002,6 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
         free_dev(c->d_a);
     }
 
-    c->f64tc = c->f64_grid;
     c->eig_real = true;
     struct CachedE { int n; double beta, c; std::vector<double> E; };
     std::vector<CachedE> cache;

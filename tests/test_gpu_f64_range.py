@@ -10,6 +10,7 @@ import numpy as np
 import pytest
 
 from oracle import adr_oracle as O
+from parity import assert_parity
 from test_gpu_parity import adr, torch
 
 pytestmark = pytest.mark.gpu
@@ -65,3 +66,21 @@ def test_sums_that_cancel(e):
     assert np.isfinite(y).all()
     worst = float(np.abs(y).max())
     assert worst == 0.0 or np.log2(worst) <= max(bound, -1073.0), (worst, bound)
+
+
+def test_a_factor_out_of_range_concerns_no_other():
+    """V_1 of a cell Peclet number of 0.92 on 400 nodes has entries of 2^460; a Lawson scheme applies e^{tau A_mu} only, whose
+    entries are at most about 1: its passes stay on the tensor cores (kind 4 of a profiled step; 3: plain FMAs)."""
+    dims, tau = (400, 60), 1e-6
+    a, b, r = np.ones((62, 402)), (740.0, 0.0, 0.0), (0.0, 0.0, 1.0, -1.0)
+    ctx = adr.Context(dims, tau, "lawson4", "fp64")
+    ctx.set_coeffs(a, b, r)
+    u = np.random.default_rng(5).standard_normal(dims[::-1])
+    v = torch.tensor(u, device="cuda")
+    y = torch.empty_like(v)
+    ctx.apply_exp(0.5, v, y)
+    kinds = [k for k, _ in ctx.profile_step(v)]
+    ctx.synchronize()
+    ops = O.GridOps(O.ADRProblem(dims, a, b, r), tau)
+    assert_parity(y.cpu().numpy(), ops.expA(0.5, u), 1e-12, what="exp")
+    assert 3 not in kinds and kinds.count(4) == 8, kinds
