@@ -232,11 +232,57 @@ adr_status publish(adr_ctx* c) {
     return ADR_OK;
 }
 
+// What a context has for speed alone: the phi tables (epilogues evaluate phi themselves without them), the cut factors (the
+// FMA kernel takes the dense ones) and the face weights (the stencil forms them from the nodal array). Where memory is short
+// it does without. shed() gives them back, and says whether there was any; nothing of the context may be in
+// flight, and the face weights stay while steps rely on them.
+template <typename T>
+bool give_back(T*& p) {
+    if (!p) return false;
+    cudaFree(p);
+    p = nullptr;
+    return true;
+}
+bool shed(adr_ctx* c) {
+    bool any = false;
+    for (auto& p : c->d_phi64) any = give_back(p) || any;
+    for (auto& p : c->d_phi32) any = give_back(p) || any;
+    for (int k = 0; k < kFactorKinds; ++k)
+        for (int m = 0; m < 3; ++m) {
+            c->cut64[k][m] = false;
+            any = give_back(c->d_img64[k][m]) || any;
+        }
+    if (!c->coeffs_set)
+        for (auto& p : c->d_face)
+            if (p) {
+                free_dev(p);
+                any = true;
+            }
+    return any;
+}
+template <typename T>
+cudaError_t need(adr_ctx* c, T** p, size_t bytes) {
+    if (*p) return cudaSuccess;
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    if (e == cudaErrorMemoryAllocation && shed(c)) {
+        cudaGetLastError();
+        e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    }
+    if (e != cudaSuccess) *p = nullptr;
+    return e;
+}
+template <typename T>
+bool spare(T** p, size_t bytes) {
+    if (*p || cudaMalloc(reinterpret_cast<void**>(p), bytes) == cudaSuccess) return true;
+    cudaGetLastError();                    // done without: the next launch is not to report it
+    *p = nullptr;
+    return false;
+}
+
 // Upload an FP64 host array in the working precision.
 cudaError_t upload(adr_ctx* c, void** dst, const std::vector<double>& src) {
     const size_t bytes = src.size() * c->esize;
-    cudaError_t e = cudaSuccess;
-    if (!*dst) e = cudaMalloc(dst, bytes);
+    const cudaError_t e = need(c, dst, bytes);
     if (e != cudaSuccess) return e;
     if (c->fp64) return cudaMemcpy(*dst, src.data(), bytes, cudaMemcpyHostToDevice);
     std::vector<float> tmp(src.begin(), src.end());
@@ -246,10 +292,8 @@ cudaError_t upload(adr_ctx* c, void** dst, const std::vector<double>& src) {
 // Slice an FP64 factor for the tensor-core kernel and upload image + row scales.
 cudaError_t upload_tc(adr_ctx* c, int kind, int m, const std::vector<double>& M) {
     const adr::TcFactor f = adr::make_tc_factor(M, c->n[m]);
-    cudaError_t e = cudaSuccess;
-    if (!c->d_img[kind][m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_img[kind][m]), f.img.size());
-    if (e == cudaSuccess && !c->d_fsc[kind][m])
-        e = cudaMalloc(reinterpret_cast<void**>(&c->d_fsc[kind][m]), f.fscale.size() * sizeof(float));
+    cudaError_t e = need(c, &c->d_img[kind][m], f.img.size());
+    if (e == cudaSuccess) e = need(c, &c->d_fsc[kind][m], f.fscale.size() * sizeof(float));
     if (e == cudaSuccess) e = cudaMemcpy(c->d_img[kind][m], f.img.data(), f.img.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(c->d_fsc[kind][m], f.fscale.data(), f.fscale.size() * sizeof(float), cudaMemcpyHostToDevice);
@@ -270,14 +314,13 @@ cudaError_t upload_f64(adr_ctx* c, int kind, int m, const std::vector<double>& M
     const std::vector<int> cexp = adr::f64_column_exps(M, n);
     for (int v : cexp)
         if (v <= adr::kF64MinExp) return cudaSuccess;
-    cudaError_t e = cudaSuccess;
-    if (!c->d_img64[kind][m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_img64[kind][m]), adr::f64_image_bytes(n));
-    if (e == cudaSuccess && !c->d_rows64[kind][m])
-        e = cudaMalloc(reinterpret_cast<void**>(&c->d_rows64[kind][m]), adr::f64_rows(n) * sizeof(int));
     int*& d_cexp = c->d_cexp64[kind][m];
     const bool eq = c->eq64[kind][m] = !cexp.empty();
-    if (e == cudaSuccess && eq && !d_cexp) e = cudaMalloc(reinterpret_cast<void**>(&d_cexp), cexp.size() * sizeof(int));
-    if (e == cudaSuccess && eq) e = cudaMemcpy(d_cexp, cexp.data(), cexp.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (!spare(&c->d_img64[kind][m], adr::f64_image_bytes(n)) || !spare(&c->d_rows64[kind][m], adr::f64_rows(n) * sizeof(int)) ||
+        (eq && !spare(&d_cexp, cexp.size() * sizeof(int))))
+        return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    if (eq) e = cudaMemcpy(d_cexp, cexp.data(), cexp.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = adr::launch_f64_factor(static_cast<const double*>(dense_factor(c, kind, m)), n, eq ? d_cexp : nullptr,
                                    c->d_img64[kind][m], c->d_rows64[kind][m], nullptr);
@@ -1763,11 +1806,11 @@ adr_status setup_doubling(adr_ctx* c) {
     if (e != cudaSuccess) return cuda_fail(c, e, "upload doubling factors");
     const size_t abytes = size_t(c->apitch) * (c->n[1] + 2) * (c->dim == 3 ? c->n[2] + 2 : 1) * c->esize;
     if (!c->d_a0 && !c->fp64) {            // the FP64 stencil takes no array for zero
-        e = cudaMalloc(&c->d_a0, abytes);
+        e = need(c, &c->d_a0, abytes);
         if (e == cudaSuccess) e = cudaMemset(c->d_a0, 0, abytes);
     }
     for (int i = 0; i < 3 && e == cudaSuccess; ++i)
-        if (!c->wsd[i]) e = cudaMalloc(&c->wsd[i], c->N * c->esize);
+        e = need(c, &c->wsd[i], c->N * c->esize);
     if (e != cudaSuccess) return fail(c, ADR_ERR_ALLOC, std::string("doubling route: ") + cudaGetErrorString(e));
     return ADR_OK;
 }
@@ -1990,16 +2033,20 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
     if (e != cudaSuccess) return cuda_fail(c, e, "upload a");
     if (c->fp64 && c->p.form == ADR_FORM_FLUX) {   // face weights in place of the nodal array
         const long long next[3] = {1, c->apitch, (long long)c->apitch * N2};
-        for (int m = 0; m < c->dim && e == cudaSuccess; ++m) {
-            const double h = neumann ? 1.0 / c->n[m] : 1.0 / (c->n[m] + 1);
-            if (!c->d_face[m]) e = cudaMalloc(&c->d_face[m], amb.size() * sizeof(double));
-            if (e == cudaSuccess)
+        bool room = true;
+        for (int m = 0; m < c->dim && room; ++m) room = spare(&c->d_face[m], amb.size() * sizeof(double));
+        if (room) {
+            for (int m = 0; m < c->dim && e == cudaSuccess; ++m) {
+                const double h = 1.0 / (c->n[m] + 1);
                 e = adr::launch_f64_faces(static_cast<const double*>(c->d_a), static_cast<double*>(c->d_face[m]), 1.0 / (h * h),
                                           next[m], (long long)amb.size(), nullptr);
+            }
+            if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+            if (e != cudaSuccess) return cuda_fail(c, e, "face weights");
+            free_dev(c->d_a);
+        } else {
+            for (auto& p : c->d_face) free_dev(p);
         }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
-        if (e != cudaSuccess) return cuda_fail(c, e, "face weights");
-        free_dev(c->d_a);
     }
 
     c->eig_real = true;
@@ -2039,7 +2086,7 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
         if (!eg.real) { c->eig_real = false; continue; }
         e = upload(c, &c->d_V[m], eg.V);
         if (e == cudaSuccess) e = upload(c, &c->d_Vi[m], eg.Vinv);
-        if (e == cudaSuccess && !c->d_lam[m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_lam[m]), c->n[m] * sizeof(double));
+        if (e == cudaSuccess) e = need(c, &c->d_lam[m], c->n[m] * sizeof(double));
         if (e == cudaSuccess) e = cudaMemcpy(c->d_lam[m], eg.lam.data(), c->n[m] * sizeof(double), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = upload_f64(c, FK_V, m, eg.V);
         if (e == cudaSuccess) e = upload_f64(c, FK_VINV, m, eg.Vinv);
@@ -2048,7 +2095,7 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
         if (e == cudaSuccess && c->tc) {
             std::vector<float> zt(c->n[m]);
             for (int j = 0; j < c->n[m]; ++j) zt[j] = static_cast<float>(c->p.tau * eg.lam[j]);
-            if (!c->d_zt[m]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_zt[m]), zt.size() * sizeof(float));
+            e = need(c, &c->d_zt[m], zt.size() * sizeof(float));
             if (e == cudaSuccess) e = cudaMemcpy(c->d_zt[m], zt.data(), zt.size() * sizeof(float), cudaMemcpyHostToDevice);
         }
         if (e != cudaSuccess) return cuda_fail(c, e, "upload eigenpairs");
@@ -2078,21 +2125,23 @@ adr_status adr_set_coeffs(adr_ctx* c, int instance, const double* a_nodes, const
             // the contraction (FP64: 40 to 60 instructions a node; the series near 0 in every precision)
             for (int k = 1; k <= 2 && e == cudaSuccess; ++k) {
                 if (c->fp64) {
-                    if (!c->d_phi64[k]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_phi64[k]), c->N * sizeof(double));
                     ContractArgs<double> a;
                     phi_fields(c, k, a);
-                    if (e == cudaSuccess) e = adr::launch_phi_nodes(c->d_phi64[k], a, c->N, nullptr);
+                    if (spare(&c->d_phi64[k], c->N * sizeof(double))) e = adr::launch_phi_nodes(c->d_phi64[k], a, c->N, nullptr);
                 } else {
-                    if (!c->d_phi32[k]) e = cudaMalloc(reinterpret_cast<void**>(&c->d_phi32[k]), c->N * sizeof(float));
                     ContractArgs<float> a;
                     phi_fields(c, k, a);
-                    if (e == cudaSuccess)
+                    if (spare(&c->d_phi32[k], c->N * sizeof(float)))
                         e = c->tc ? adr::launch_phi_table(c->d_phi32[k], k, c->d_zt, c->n[0], c->n[1], c->N, nullptr)
                                   : adr::launch_phi_nodes(c->d_phi32[k], a, c->N, nullptr);
                 }
             }
             if (e != cudaSuccess) return cuda_fail(c, e, "phi tables");
         }
+    }
+    if (!c->d_a && !c->d_face[0]) {        // the face weights had to go
+        e = upload(c, &c->d_a, amb);
+        if (e != cudaSuccess) return cuda_fail(c, e, "upload a");
     }
     return publish(c);
 }
@@ -2235,6 +2284,10 @@ adr_status adr_integrate_host(adr_ctx* c, void* u_host, double t0, double T, int
     cudaError_t e = cudaSuccess;
     if (!c->d_host_state) {
         e = cudaMalloc(&c->d_host_state, bytes);
+        if (e == cudaErrorMemoryAllocation && cudaStreamSynchronize(c->stream) == cudaSuccess) {
+            drop_graph(c);                 // its launches hold what is given back
+            e = need(c, &c->d_host_state, bytes);
+        }
         if (e != cudaSuccess) return fail(c, ADR_ERR_ALLOC, std::string("state buffer: ") + cudaGetErrorString(e));
     }
     e = cudaMemcpyAsync(c->d_host_state, u_host, bytes, cudaMemcpyHostToDevice, c->stream);

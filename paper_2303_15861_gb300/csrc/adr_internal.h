@@ -87,7 +87,7 @@ struct StencilArgs {
                                      // (j3 * (n2 + 2) + j2) * apitch + j1 + 3
     int apitch = 0;                  // row pitch of a: multiple of 4, >= n1 + 5
     const T* face[3] = {nullptr, nullptr, nullptr};   // FP64 flux form: (1/2h^2) times the sums of a across the
-                                     // faces, at the lower node, laid out as a (NULL: a = 0)
+                                     // faces, at the lower node, laid out as a, which is then NULL (both NULL: a = 0)
     int dim = 3, n1 = 1, n2 = 1, n3 = 1;
     bool neumann = false;            // homogeneous Neumann faces at x_mu = 1: mirror ghosts
     bool adelta = false;             // (a - abar) Lap u instead of div((a - abar) grad u)

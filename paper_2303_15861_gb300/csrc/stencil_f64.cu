@@ -30,8 +30,8 @@ constexpr int kTX = 32, kTY = 8;         // threads of a block along x1 (V nodes
 struct Weights {
     double w2[3];                        // (b - beta) / (2h)
     double wa[3], wb[3];                 // abar / h^2, beta / (2h)
-    double ih2[3];
-    const double* face[3];               // face weights, laid out as StencilArgs::a (NULL: a = abar everywhere)
+    double ih2[3], hih2[3];              // 1 / h^2, and half of it
+    const double* face[3];               // face weights, laid out as StencilArgs::a (NULL: a = abar everywhere, or NODAL)
     // which terms there are: tested as integers, since a comparison of doubles costs an FP64 instruction
     bool adv;                            // a w2, or a wb that F takes, is not zero
     int start[kMaxOut];                  // a term of coefficient one: 1 u, 2 g, 3 F, 4 + e X_e; 0 none
@@ -59,8 +59,9 @@ __device__ __forceinline__ void stv(double* p, const double (&v)[V]) {
 // and the face weights below plane z stay in registers, the neighbours along x1 and x2 come from L1.
 // ADV: any first-derivative term; NX: stage inputs; UT: whether an output takes a multiple of u. An instruction under a false predicate still takes its turn on the
 // FP64 pipe, and the compiler turns short branches into predicates, so what decides about few instructions is a
-// template argument.
-template <int DIM, int V, bool ADELTA, bool NEEDF, bool ADV, int NX, bool UT>
+// template argument. NODAL: the face weights formed here from the nodal array, to the same bits, for contexts that had no
+// memory for them (256^3, one output: 506 -> 1090 us).
+template <int DIM, int V, bool ADELTA, bool NEEDF, bool ADV, int NX, bool UT, bool NODAL = false>
 __global__ void __launch_bounds__(kTX * kTY) stencil_f64_kernel(StencilArgs<double> p, Coefs<double> c, Weights w, int zb) {
     const int n1 = p.n1, n2 = p.n2, n3 = DIM == 3 ? p.n3 : 1;
     const int i1 = (int(blockIdx.x) * kTX + int(threadIdx.x % kTX)) * V;
@@ -71,11 +72,11 @@ __global__ void __launch_bounds__(kTX * kTY) stencil_f64_kernel(StencilArgs<doub
     const int z0 = DIM == 3 ? int(blockIdx.z) * zb : 0, z1 = DIM == 3 ? min(z0 + zb, n3) : 1;
     const double* u = p.u + (long long)i2 * n1 + i1 + z0 * plane_u;
     const long long ao = (long long)(i2 + 1) * p.apitch + (i1 + 4) + (DIM == 3 ? (z0 + 1) * plane_a : 0);
-    const double* aC = ADELTA && p.a ? p.a + ao : nullptr;
-    const bool faces = !ADELTA && w.face[0];
-    const double* f1 = faces ? w.face[0] + ao : nullptr;
-    const double* f2 = faces ? w.face[1] + ao : nullptr;
-    const double* f3 = faces && DIM == 3 ? w.face[2] + ao : nullptr;
+    const double* aC = (ADELTA || NODAL) && p.a ? p.a + ao : nullptr;
+    const bool faces = NODAL || (!ADELTA && w.face[0]);
+    const double* f1 = faces && !NODAL ? w.face[0] + ao : nullptr;
+    const double* f2 = faces && !NODAL ? w.face[1] + ao : nullptr;
+    const double* f3 = faces && !NODAL && DIM == 3 ? w.face[2] + ao : nullptr;
 
     double uM[V], uC[V], dM[V], fM[V];
     ldv<V>(u, uC);
@@ -83,7 +84,15 @@ __global__ void __launch_bounds__(kTX * kTY) stencil_f64_kernel(StencilArgs<doub
     for (int k = 0; k < V; ++k) uM[k] = fM[k] = 0.0;
     if (DIM == 3) {
         if (z0 > 0) ldv<V>(u - plane_u, uM);
-        if (faces) ldv<V>(f3 - plane_a, fM);
+        if (NODAL) {
+            double aM[V];
+            ldv<V>(aC - plane_a, aM);
+            ldv<V>(aC, fM);
+#pragma unroll
+            for (int k = 0; k < V; ++k) fM[k] = w.hih2[2] * (aM[k] + fM[k]);
+        } else if (faces) {
+            ldv<V>(f3 - plane_a, fM);
+        }
 #pragma unroll
         for (int k = 0; k < V; ++k) dM[k] = uC[k] - uM[k];
     }
@@ -109,7 +118,22 @@ __global__ void __launch_bounds__(kTX * kTY) stencil_f64_kernel(StencilArgs<doub
         if (i1 > 0) uW = __ldg(u - 1);
         if (i1 + V < n1) uE = __ldg(u + V);
         else if (p.neumann) uE = V == 2 ? uC[0] : uW;
-        if (faces) {
+        if (NODAL) {
+            double ac[V];
+            ldv<V>(aC, ac);
+            ldv<V>(aC - p.apitch, fS);
+            ldv<V>(aC + p.apitch, fN);
+            const double ae = __ldg(aC + V);
+            fW = w.hih2[0] * (__ldg(aC - 1) + ac[0]);
+            if (DIM == 3) ldv<V>(aC + plane_a, fP);
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+                fE[k] = w.hih2[0] * (ac[k] + (k + 1 < V ? ac[V - 1] : ae));
+                fS[k] = w.hih2[1] * (fS[k] + ac[k]);
+                fN[k] = w.hih2[1] * (ac[k] + fN[k]);
+                if (DIM == 3) fP[k] = w.hih2[2] * (ac[k] + fP[k]);
+            }
+        } else if (faces) {
             fW = __ldg(f1 - 1);
             ldv<V>(f1, fE);
             ldv<V>(f2 - p.apitch, fS);
@@ -208,8 +232,8 @@ __global__ void __launch_bounds__(kTX * kTY) stencil_f64_kernel(StencilArgs<doub
             }
             u += plane_u;
             idx += plane_u;
-            if (faces) { f1 += plane_a; f2 += plane_a; f3 += plane_a; }
-            if (ADELTA && aC) aC += plane_a;
+            if (faces && !NODAL) { f1 += plane_a; f2 += plane_a; f3 += plane_a; }
+            if ((ADELTA || NODAL) && aC) aC += plane_a;
         }
     }
 }
@@ -246,8 +270,15 @@ cudaError_t launch_v(const StencilArgs<double>& p, const Coefs<double>& c, const
     while (ty > 1 && gx * ((p.n2 + ty - 1) / ty) * gz < 2 * sms) ty /= 2;
     const dim3 grid(gx, (p.n2 + ty - 1) / ty, gz);
     const int threads = kTX * ty;
+    const bool nodal = !p.adelta && p.a && !w.face[0];       // has every term
     auto go = [&](auto adelta, auto f, auto adv) {
         constexpr bool AD = decltype(adelta)::value, NF = decltype(f)::value, AV = decltype(adv)::value;
+        if constexpr (!AD && AV) {
+            if (nodal) {
+                stencil_f64_kernel<DIM, V, false, NF, true, kMaxExtra, true, true><<<grid, threads, 0, s>>>(p, c, w, zb);
+                return;
+            }
+        }
         // odd rows and 2-D grids take the form that has every term
         if constexpr (DIM == 2 || V == 1) {
             stencil_f64_kernel<DIM, V, AD, NF, AV, kMaxExtra, true><<<grid, threads, 0, s>>>(p, c, w, zb);
@@ -266,7 +297,7 @@ cudaError_t launch_v(const StencilArgs<double>& p, const Coefs<double>& c, const
     };
     using Yes = std::integral_constant<bool, true>;
     using No = std::integral_constant<bool, false>;
-    auto with_adv = [&](auto adelta, auto f) { w.adv ? go(adelta, f, Yes{}) : go(adelta, f, No{}); };
+    auto with_adv = [&](auto adelta, auto f) { w.adv || nodal ? go(adelta, f, Yes{}) : go(adelta, f, No{}); };
     if (p.adelta) needF ? with_adv(Yes{}, Yes{}) : with_adv(Yes{}, No{});
     else          needF ? with_adv(No{}, Yes{}) : with_adv(No{}, No{});
     return cudaGetLastError();
@@ -289,6 +320,7 @@ cudaError_t launch_stencil(const StencilArgs<double>& p, cudaStream_t s) {
         w.wa[m] = p.abar * p.inv_h2[m];
         w.wb[m] = p.beta[m] * p.inv_2h[m];
         w.ih2[m] = p.inv_h2[m];
+        w.hih2[m] = 0.5 * p.inv_h2[m];
         w.face[m] = p.face[m];
     }
     c.r0 = p.r[0]; c.r1 = p.r[1]; c.r2 = p.r[2]; c.r3 = p.r[3];
