@@ -44,3 +44,22 @@ def test_pulses(dims, b, centre):
         ctx.apply_phi(k, v, y)
         ctx.synchronize()
         assert_parity(y.cpu().numpy(), ops.phi(k, 1.0, u0) if k else ops.expA(1.0, u0), 1e-12, what=f"phi_{k} {dims} {b}")
+
+
+@pytest.mark.parametrize("dims,b,tau", [((128, 128), (60, -40), 1e-2), ((300, 70), (80, 10), 5e-3), ((40, 66, 65), (30, -60, 10), 1e-2)])
+def test_exponentials_with_columns_of_several_sizes(dims, b, tau):
+    """Advection that carries the state out of the box within a step or two: the columns of e^{c tau A_1} differ, too, and
+    the stage combinations follow those passes."""
+    ctx, ops = problem(dims, b, tau, "lawson2b")
+    columns = np.abs(ops.mf.E_factors(1.0)[0]).max(axis=0)
+    assert columns.max() > 16 * columns.min()
+    u0 = pulse(dims, 0.5, 0.2) + 1e-3 * np.random.default_rng(2).standard_normal(dims[::-1])
+    v = torch.tensor(u0, device="cuda")
+    y = torch.empty_like(v)
+    for c in (0.5, 1.0):
+        ctx.apply_exp(c, v, y)
+        ctx.synchronize()
+        assert_parity(y.cpu().numpy(), ops.expA(c, u0), 1e-12, what=f"exp {dims} {c}")
+    ctx.integrate(v, 0.0, 2 * tau, 2)
+    ctx.synchronize()
+    assert_parity(v.cpu().numpy(), O.integrate(ops, u0, 2, "lawson2b"), 1e-12, what=f"lawson2b {dims}")
