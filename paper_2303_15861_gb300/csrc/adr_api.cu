@@ -2285,6 +2285,7 @@ adr_status adr_integrate_host(adr_ctx* c, void* u_host, double t0, double T, int
     if (!c->d_host_state) {
         e = cudaMalloc(&c->d_host_state, bytes);
         if (e == cudaErrorMemoryAllocation && cudaStreamSynchronize(c->stream) == cudaSuccess) {
+            cudaGetLastError();
             drop_graph(c);                 // its launches hold what is given back
             e = need(c, &c->d_host_state, bytes);
         }

@@ -16,25 +16,13 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart.
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-    return uint64_t((saddr & 0x3FFFFu) >> 4) | (uint64_t(1) << 16) | (uint64_t(1024 >> 4) << 32) |
-           (uint64_t(1) << 46) | (uint64_t(2) << 61);
-}
-
-// The same for the 64-byte swizzle (rows of 32 bf16, 8-row groups 512 B apart; layout code 4).
+// Shared-memory matrix descriptor: K-major, 64-byte swizzle (rows of 32 bf16, 8-row groups 512 B apart; layout code 4).
 __device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
     return uint64_t((saddr & 0x3FFFFu) >> 4) | (uint64_t(1) << 16) | (uint64_t(512 >> 4) << 32) |
            (uint64_t(1) << 46) | (uint64_t(4) << 61);
 }
 
-// byte offset of the 16-byte chunk j (8 bf16 along K) of row r in a 128B-swizzled tile:
-// address bits [4:6] are XORed with bits [7:9]
-__device__ __forceinline__ uint32_t swz(int r, int j) {
-    return uint32_t((r >> 3) * 1024 + (r & 7) * 128 + ((j ^ (r & 7)) << 4));
-}
-
-// ... and in a 64B-swizzled tile (rows of 64 B): address bits [4:5] are XORed with bits [7:8]
+// Byte offset of the 16-byte chunk j (8 bf16 along K) of row r in such a tile: address bits [4:5] are XORed with bits [7:8].
 __device__ __forceinline__ uint32_t swz64(int r, int j) {
     return uint32_t((r >> 3) * 512 + (r & 7) * 64 + ((j ^ ((r >> 1) & 3)) << 4));
 }
