@@ -57,7 +57,12 @@ typedef enum {
 } adr_status;
 
 typedef enum {
-    ADR_FP64 = 0,          /* FP64 state, stencil and contractions (FP64 FMA, large ones exact digits on tensor cores) */
+    ADR_FP64 = 0,          /* FP64 state, stencil and contractions: FP64 FMA, large ones
+                              fixed-point digits on the tensor cores. Those are as accurate
+                              relative to the largest result of a line (the n values that
+                              are contracted together); results further than 2^-53 below
+                              it are noise of that size, of either sign, where FMAs of
+                              positive values would keep their digits                    */
     ADR_FP32 = 1,          /* FP32 state, stencil and contractions (FP32 FMA)            */
     ADR_MIXED_TF32X3 = 2,  /* reserved: not implemented (returns ADR_ERR_UNSUPPORTED)    */
     ADR_MIXED_BF16X3 = 3   /* FP32 state and stencil; mu-mode contractions on the tensor

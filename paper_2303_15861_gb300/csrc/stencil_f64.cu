@@ -9,10 +9,10 @@
 // registers), and terms whose coefficient is zero are left out by branches that every thread takes alike.
 // Per node and direction: d+ (shared), two FMAs with the face weights; M = u+ - u- and one FMA
 // where b - beta is not zero; for F, L = d+ - d- and one FMA with abar / h^2, and one FMA of M with beta / (2h).
-// u + tau/2 g in 3-D: 15 FP64 instructions a node instead of about 75; F and g: 27 instead of 85.
+// u + tau/2 g in 3-D: 15.6 FP64 instructions a node instead of about 75; F and g: 32 instead of 85 (ncu).
 // Time of a launch, per-node kernel -> this one (us): 256^3 2139 -> 504 (one output), 2460 -> 607 and 692 (two outputs, one and two
 // stage inputs); 128^3 F and g 379 -> 142, g - G0 283 -> 66; 60^3 Neumann, a Lap u form 39 -> 17; 32^2 12.6 -> 7.3. The FP64 pipe
-// is then 85% busy.
+// is then 86 to 90% busy.
 #include <cuda_runtime.h>
 
 #include <type_traits>
