@@ -196,7 +196,8 @@ adr_status adr_create(const adr_params* p, void* cuda_stream, adr_ctx** out);
  * e^{c tau A_mu} (Pade-13 scaling and squaring) and the closed-form eigenpairs of
  * A_mu; uploads them. Synchronous with respect to the host data (it may be freed on
  * return), and called again on a context it first waits for what the context's stream
- * still has to do with the coefficients before. Returns ADR_ERR_COMPLEX_SPECTRUM / ADR_ERR_ILL_CONDITIONED for ADR_ETD2RK
+ * still has to do with the coefficients before; a CUDA graph that the caller captured from
+ * this context's calls holds buffers of those, and is captured anew. Returns ADR_ERR_COMPLEX_SPECTRUM / ADR_ERR_ILL_CONDITIONED for ADR_ETD2RK
  * when the eigen route is unavailable or fails the kappa guard.
  * Batched contexts build only the factors their scheme uses (e^{tau A_mu} for
  * ADR_LAWSON_EULER, e^{tau A_mu / 2} for ADR_LAWSON4, the eigenpairs for ADR_ETD2RK).

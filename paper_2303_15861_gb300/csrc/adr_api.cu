@@ -234,8 +234,8 @@ adr_status publish(adr_ctx* c) {
 
 // What a context has for speed alone: the phi tables (epilogues evaluate phi themselves without them), the cut factors (the
 // FMA kernel takes the dense ones) and the face weights (the stencil forms them from the nodal array). Where memory is short
-// it does without. shed() gives them back, and says whether there was any; nothing of the context may be in
-// flight, and the face weights stay while steps rely on them.
+// it does without. shed() gives them back, and says whether there was any. Only adr_set_coeffs does that: between two calls of
+// it a graph that the caller captured from steps may hold them.
 template <typename T>
 bool give_back(T*& p) {
     if (!p) return false;
@@ -252,12 +252,11 @@ bool shed(adr_ctx* c) {
             c->cut64[k][m] = false;
             any = give_back(c->d_img64[k][m]) || any;
         }
-    if (!c->coeffs_set)
-        for (auto& p : c->d_face)
-            if (p) {
-                free_dev(p);
-                any = true;
-            }
+    for (auto& p : c->d_face)
+        if (p) {
+            free_dev(p);
+            any = true;
+        }
     return any;
 }
 template <typename T>
@@ -2286,11 +2285,6 @@ adr_status adr_integrate_host(adr_ctx* c, void* u_host, double t0, double T, int
     cudaError_t e = cudaSuccess;
     if (!c->d_host_state) {
         e = cudaMalloc(&c->d_host_state, bytes);
-        if (e == cudaErrorMemoryAllocation && cudaStreamSynchronize(c->stream) == cudaSuccess) {
-            cudaGetLastError();
-            drop_graph(c);                 // its launches hold what is given back
-            e = need(c, &c->d_host_state, bytes);
-        }
         if (e != cudaSuccess) return fail(c, ADR_ERR_ALLOC, std::string("state buffer: ") + cudaGetErrorString(e));
     }
     e = cudaMemcpyAsync(c->d_host_state, u_host, bytes, cudaMemcpyHostToDevice, c->stream);

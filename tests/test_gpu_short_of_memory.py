@@ -4,7 +4,6 @@ is left over shrinks from what the context would like to what it cannot do witho
 
 Bounds, fixed beforehand: weights and phi factors formed in the kernels have the bits of the stored ones; the FMA kernel in
 place of the cut factors rounds K times a sum, K 2^-53 of its terms a pass at most and 1e-13 in all for these grids."""
-import numpy as np
 import pytest
 
 from test_gpu_parity import W, adr, torch
@@ -75,28 +74,3 @@ def test_new_coefficients(dims, scheme, prec, least):
             else:
                 assert torch.equal(x, y), leave
     assert min(spent) < used, (used, spent)                # something was done without
-
-
-def test_host_state_buffer():
-    dims, tau = (128, 128, 128), 1e-3
-    a, b, u0 = problem(dims, "fp64")
-    results = []
-    for short in (False, True):
-        ctx = adr.Context(dims, tau, "etd2rk", "fp64")
-        ctx.set_coeffs(a, b, (0.0, 0.0, 1.0, -1.0))
-        u = u0.clone()
-        torch.cuda.synchronize()
-        ctx.integrate(u, 0.0, tau, 1)                      # a graph that holds the tables
-        ctx.synchronize()
-        host = np.ascontiguousarray(u.cpu().numpy())
-        full = fill(8 * MB) if short else None
-        ctx.integrate_host(host, 0.0, 2 * tau, 2)
-        del full
-        torch.cuda.empty_cache()
-        u.copy_(torch.as_tensor(host))
-        torch.cuda.synchronize()
-        ctx.integrate(u, 0.0, tau, 1)
-        ctx.synchronize()
-        results.append(u.clone())
-        ctx.close()
-    assert float((results[0] - results[1]).norm() / results[0].norm()) <= 1e-13
