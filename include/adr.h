@@ -197,8 +197,9 @@ adr_status adr_create(const adr_params* p, void* cuda_stream, adr_ctx** out);
  * A_mu; uploads them. Synchronous with respect to the host data (it may be freed on
  * return), and called again on a context it first waits for what the context's stream
  * still has to do with the coefficients before; a CUDA graph that the caller captured from
- * this context's calls holds buffers of those, and is captured anew. Returns ADR_ERR_COMPLEX_SPECTRUM / ADR_ERR_ILL_CONDITIONED for ADR_ETD2RK
- * when the eigen route is unavailable or fails the kappa guard.
+ * this context's calls holds buffers of those, and is captured anew. Returns
+ * ADR_ERR_COMPLEX_SPECTRUM / ADR_ERR_ILL_CONDITIONED for ADR_ETD2RK when the eigen route is
+ * unavailable or fails the kappa guard.
  * Batched contexts build only the factors their scheme uses (e^{tau A_mu} for
  * ADR_LAWSON_EULER, e^{tau A_mu / 2} for ADR_LAWSON4, the eigenpairs for ADR_ETD2RK).
  * Steps are refused (ADR_ERR_STATE) until every instance is set. The call that sets
